@@ -346,17 +346,15 @@ lqcd_status lqcd_field_dots(int a, const float *X, int b, const float *Y, long l
  * synchronisation of cudaMalloc/cudaFree would stall other streams).
  * Same results as lqcd_small_eig, but C (n x n complex row-major), evals (n
  * complex) and Y, Z (n x n, or both NULL for eigenvalues only) are DEVICE
- * pointers on the current device, and nothing is allocated: the scratch lives
- * in a file-scope device array sized for n <= 80 (about 200 KiB, held by every
- * GPU that loads the library until the process exits).  n > 80 returns
- * LQCD_ERR_ARG.  The first call on a device looks up that array's device
- * address and sets the kernel's shared-memory limit, so make the first call
+ * pointers on the current device, and nothing is allocated: the working set is
+ * the kernel's shared memory and the status word a file-scope device variable.
+ * n > 80 returns LQCD_ERR_ARG.  The first call on a device looks up that
+ * variable's device address and sets the kernel's shared-memory limit, so make the first call
  * before any stream capture; that set-up is kept for the life of the process
  * (a cudaDeviceReset between calls is not supported).  Work is ordered on
  * 'cuda_stream' (cudaStream_t, NULL = default stream) and the call returns
- * after it completes.  All calls on
- * a device share the scratch array and it keeps the last call's contents: calls
- * whose kernels overlap on the GPU (other streams, other host threads) race.
+ * after it completes.  All calls on a device share the status word: calls
+ * whose kernels overlap on the GPU (other streams, other host threads) race on it.
  * LQCD_ERR_NOCONV if the QR iteration did not converge. */
 lqcd_status lqcd_small_eig_noalloc(int n, const double *C, double *evals, double *Y, double *Z,
                                    void *cuda_stream);

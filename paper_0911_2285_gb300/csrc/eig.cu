@@ -11,6 +11,20 @@
 // substitution, mapped back with Q. Conventions: right vectors have unit
 // 2-norm with their largest-modulus entry real positive; left vectors satisfy
 // z^H y = 1.
+//
+// What bounds it: one problem lives on one SM, and a QR sweep is a chain of
+// rotations (about 2500 of them for a 40 x 40 window matrix, 5500 for 60 x 60)
+// that cannot overlap, so the time is rotations x the latency of one: form it,
+// apply it to two rows, apply it to two columns. FP64 instructions take 64
+// cycles each and issue at 2 lanes per clock per SM (measured), so the scalars
+// that one thread used to form with the FP64 library (square roots, hypot,
+// divisions: thousands of cycles each, the other warps waiting) were most of
+// it. Here warp 0 forms the next rotation while the other warps are still
+// applying the last one to their rows, two half-warps share each pair (one
+// output each), a rotation costs two barriers, and shifts, deflation scans,
+// norms, pivot searches and substitutions run across the lanes of a warp.
+// Measured: restart coefficients (both eigen-solves and the FP64 finish) 60 x 60
+// 20.2 -> 4.6 ms, 40 x 40 10.9 -> 2.5 ms; FP64 eigen-solve 60 x 60 18.2 -> 10.9 ms.
 #include <mutex>
 
 #include "../../include/lqcd.h"
@@ -20,8 +34,10 @@
 namespace lqcd {
 namespace {
 
-constexpr int ET = 128;          // threads per eigen CTA
+constexpr int ET = 256;          // threads per eigen CTA
+constexpr int EW = ET / 32;      // warps
 constexpr double EPS = 2.220446049250313e-16;
+constexpr unsigned FULL = 0xffffffffu;
 
 __device__ __forceinline__ double2 czero() { return make_double2(0.0, 0.0); }
 __device__ __forceinline__ double2 cone() { return make_double2(1.0, 0.0); }
@@ -29,220 +45,53 @@ __device__ __forceinline__ double2 cone() { return make_double2(1.0, 0.0); }
 // |re| + |im|: the modulus surrogate used for negligibility tests (no sqrt).
 __device__ __forceinline__ double cabs1(double2 a) { return fabs(a.x) + fabs(a.y); }
 
-// 1/sqrt(a) for a > 0 in FP64. FP64 arithmetic issues at 1/64 of the FP32 rate
-// on this GPU, so the library's FP64 square root and divide are long serial
-// chains; inside FP32's normal range, an FP32 reciprocal square root seeds
-// Newton-Raphson for f(y) = 1/y^2 - a, y <- y (3 - a y^2) / 2, which doubles
-// the correct bits per step: two steps take the FP32 seed (about 22 bits) to
-// FP64 accuracy. Outside that range: 1 / sqrt(a).
-__device__ __forceinline__ double rsqrt_fp64(double a) {
-    if (!(a > 1e-30 && a < 1e30)) return 1.0 / sqrt(a);
-    double y = (double)rsqrtf((float)a);
-    const double h = 0.5 * a;
-    y = y * fma(-h * y, y, 1.5);
-    y = y * fma(-h * y, y, 1.5);
-    return y;
+// FP32 <-> FP64 conversion of a positive number inside FP32's normal range on the
+// integer pipe (the FP64 pipe's conversions take its 64-cycle latency); to FP32
+// by truncation, which is good enough for the Newton seeds below.
+__device__ __forceinline__ float seed_f32(double a) {
+    return __uint_as_float((unsigned)(((__double2hiint(a) - (896 << 20)) << 3) | ((unsigned)__double2loint(a) >> 29)));
+}
+__device__ __forceinline__ double exact_f64(float a) {
+    const unsigned b = __float_as_uint(a);
+    return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
 }
 
-// 1/a in FP64 the same way: FP32 reciprocal seed, Newton-Raphson for
-// f(y) = 1/y - a, y <- y (2 - a y), two steps. Outside FP32's normal range: 1 / a.
+// a positive and inside [2^-99, 2^99): squares and Newton seeds stay in FP32's
+// normal range. On the high word: an FP64 comparison costs the FP64 pipe's latency.
+__device__ __forceinline__ bool mid_range(double a) { return ((unsigned)__double2hiint(a) >> 20) - 924u < 198u; }
+
+// 1/sqrt(a) for a > 0 in FP64: inside FP32's normal range an FP32 reciprocal
+// square root y (relative error about 2^-21) and one step of third order: with
+// e = 1 - a y^2, 1/sqrt(a) = y (1 + e/2 + 3 e^2/8 + O(e^3)). Outside: 1 / sqrt(a).
+__device__ __forceinline__ double rsqrt_fp64(double a) {
+    if (!mid_range(a)) return 1.0 / sqrt(a);
+    const double y = exact_f64(rsqrtf(seed_f32(a)));
+    const double e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// 1/a in FP64 the same way: FP32 reciprocal seed y, e = 1 - a y,
+// 1/a = y (1 + e + e^2 + O(e^3)). Outside FP32's normal range: 1 / a.
 __device__ __forceinline__ double rcp_fp64(double a) {
     const double m = fabs(a);
-    if (!(m > 1e-30 && m < 1e30)) return 1.0 / a;
-    double y = (double)__frcp_rn((float)a);
-    y = y * fma(-a, y, 2.0);
-    y = y * fma(-a, y, 2.0);
-    return y;
+    if (!mid_range(m)) return 1.0 / a;
+    const double y = copysign(exact_f64(__frcp_rn(seed_f32(m))), a);
+    const double e = fma(-a, y, 1.0);
+    return fma(y * e, 1.0 + e, y);
 }
 
-// Unitary rotation G = [[cx, cy], [-conj(cy), conj(cx)]] with G [x; y] = [n; 0],
-// cx = conj(x)/n, cy = conj(y)/n, n = sqrt(|x|^2 + |y|^2): one reciprocal square
-// root. (One thread forms it: FP64 issue, not the barriers around it, bounds
-// this solver, and every warp forming it would quadruple that work.)
-__device__ __forceinline__ void givens(double2 x, double2 y, double2& cx, double2& cy) {
-    const double n2 = cabs2(x) + cabs2(y);
-    if (n2 == 0.0) { cx = cone(); cy = czero(); return; }
-    const double inv = rsqrt_fp64(n2);
-    cx = inv * conj_(x);
-    cy = inv * conj_(y);
+// sqrt(a) for a >= 0: a / sqrt(a) and one correction of the product's rounding.
+__device__ __forceinline__ double sqrt_fp64(double a) {
+    if (!mid_range(a)) return sqrt(a);
+    const double r = rsqrt_fp64(a), s = a * r;
+    return fma(0.5 * r, fma(-s, s, a), s);
 }
 
-// ---------------------------------------------------------------------------
-// Block-cooperative eigen-solver on A (n x n, leading dim lda, shared memory).
-// On return A holds the Schur form T, Q the Schur vectors. Returns 0 on
-// success, 1 if QR failed to converge.
-__device__ int schur(double2* A, double2* Q, int n, int lda, double2* v /* n */, double* sh) {
-    const int tid = threadIdx.x;
-    // Q = I
-    for (int e = tid; e < n * lda; e += blockDim.x) Q[e] = ((e / lda) == (e % lda)) ? cone() : czero();
-    __syncthreads();
-    // Householder reduction to upper Hessenberg. A column with nothing below its
-    // subdiagonal is skipped, and a reflection spans only the rows up to the
-    // column's last nonzero: the projected matrices of eigBiCG are tridiagonal,
-    // or after a restart diagonal + coupling arrow + tridiagonal, so most
-    // columns need no work.
-    for (int k = 0; k + 2 < n; ++k) {
-        // v = x + e^{i theta} ||x|| e1, x = A[k+1:last+1, k]
-        if (tid == 0) {
-            double nrm2 = 0.0, tail = 0.0;
-            int last = k + 1;
-            for (int i = k + 1; i < n; ++i) {
-                const double a2 = cabs2(A[i * lda + k]);
-                nrm2 += a2;
-                if (i >= k + 2) tail += a2;
-                if (a2 != 0.0) last = i;
-            }
-            double alpha = sqrt(nrm2);
-            double2 x0 = A[(k + 1) * lda + k];
-            double ax0 = cabs_(x0);
-            double2 ph = ax0 > 0.0 ? make_double2(x0.x / ax0, x0.y / ax0) : cone();
-            sh[0] = tail > 0.0 ? alpha : 0.0;   // 0: skip the step
-            sh[1] = alpha > 0.0 ? 1.0 / (alpha * (alpha + ax0)) : 0.0;   // tau = 2/||v||^2
-            sh[2] = ph.x; sh[3] = ph.y;
-            sh[5] = (double)last;
-        }
-        __syncthreads();
-        double alpha = sh[0], tau = sh[1];
-        double2 ph = make_double2(sh[2], sh[3]);
-        const int last = (int)sh[5];
-        if (alpha == 0.0) { __syncthreads(); continue; }
-        for (int i = k + 1 + tid; i <= last; i += blockDim.x) v[i - k - 1] = A[i * lda + k];
-        __syncthreads();
-        if (tid == 0) v[0] = v[0] + alpha * ph;
-        __syncthreads();
-        const int len = last - k;
-        // rows k+1..n-1 of A: A -= tau v (v^H A), columns k..n-1
-        for (int j = k + tid; j < n; j += blockDim.x) {
-            double2 w = czero();
-            for (int i = 0; i < len; ++i) w = w + cdot(v[i], A[(k + 1 + i) * lda + j]);
-            w = tau * w;
-            for (int i = 0; i < len; ++i) A[(k + 1 + i) * lda + j] = A[(k + 1 + i) * lda + j] - v[i] * w;
-        }
-        __syncthreads();
-        // columns k+1..n-1 of A (all rows) and of Q: X -= tau (X v) v^H
-        for (int i = tid; i < 2 * n; i += blockDim.x) {
-            double2* row = i < n ? A + i * lda : Q + (i - n) * lda;
-            double2 u = czero();
-            for (int l = 0; l < len; ++l) u = u + row[k + 1 + l] * v[l];
-            u = tau * u;
-            for (int l = 0; l < len; ++l) row[k + 1 + l] = row[k + 1 + l] - mulc(u, v[l]);
-        }
-        __syncthreads();
-        for (int i = k + 2 + tid; i <= last; i += blockDim.x) A[i * lda + k] = czero();
-        __syncthreads();
-    }
-    // Frobenius norm for the negligibility tests.
-    if (tid == 0) {
-        double f = 0.0;
-        for (int i = 0; i < n; ++i)
-            for (int j = (i > 0 ? i - 1 : 0); j < n; ++j) f += cabs2(A[i * lda + j]);
-        sh[4] = sqrt(f);
-    }
-    __syncthreads();
-    const double anorm = sh[4] > 0.0 ? sh[4] : 1.0;
-    // Single-shift implicit QR with deflation from the bottom.
-    __shared__ int s_l, s_hi, s_fail;
-    __shared__ double2 s_cx, s_cy, s_mu;
-    if (tid == 0) { s_hi = n - 1; s_fail = 0; }
-    __syncthreads();
-    int iters = 0, total = 0;
-    while (true) {
-        if (tid == 0) {
-            int hi = s_hi;
-            int l = hi;
-            while (l > 0) {
-                double tst = cabs1(A[(l - 1) * lda + l - 1]) + cabs1(A[l * lda + l]);
-                if (tst == 0.0) tst = anorm;
-                if (cabs1(A[l * lda + l - 1]) <= EPS * tst) { A[l * lda + l - 1] = czero(); break; }
-                --l;
-            }
-            s_l = l;
-        }
-        __syncthreads();
-        int hi = s_hi, l = s_l;
-        if (hi <= 0) break;
-        if (l == hi) {
-            __syncthreads();
-            if (tid == 0) s_hi = hi - 1;
-            iters = 0;
-            __syncthreads();
-            continue;
-        }
-        ++iters; ++total;
-        if (iters > 60 || total > 60 * n) { if (tid == 0) s_fail = 1; __syncthreads(); break; }
-        if (tid == 0) {
-            double2 a = A[(hi - 1) * lda + hi - 1], b = A[(hi - 1) * lda + hi];
-            double2 c = A[hi * lda + hi - 1], d = A[hi * lda + hi];
-            double2 mu;
-            if (iters % 11 == 10) {
-                // exceptional shift
-                mu = d + make_double2(0.75 * cabs1(c), 0.0);
-            } else {
-                double2 t = 0.5 * (a - d);
-                double2 bc = b * c;
-                double2 disc2 = t * t + bc;
-                // complex sqrt
-                double r = cabs_(disc2);
-                double sx = sqrt(0.5 * (r + disc2.x));
-                double sy = sqrt(0.5 * (r - disc2.x));
-                if (disc2.y < 0) sy = -sy;
-                double2 disc = make_double2(sx, sy);
-                double2 den1 = t + disc, den2 = t - disc;
-                double2 den = cabs2(den1) >= cabs2(den2) ? den1 : den2;
-                mu = cabs2(den) > 0.0 ? d - cdiv(bc, den) : d;
-            }
-            s_mu = mu;
-        }
-        __syncthreads();
-        double2 mu = s_mu;
-        for (int k = l; k < hi; ++k) {
-            if (tid == 0) {
-                double2 x, y;
-                if (k == l) { x = A[l * lda + l] - mu; y = A[(l + 1) * lda + l]; }
-                else { x = A[k * lda + k - 1]; y = A[(k + 1) * lda + k - 1]; }
-                double2 cx, cy;
-                givens(x, y, cx, cy);
-                s_cx = cx; s_cy = cy;
-            }
-            __syncthreads();
-            const double2 cx = s_cx, cy = s_cy;
-            const double2 cxc = conj_(cx), cyc = conj_(cy);
-            // rows k, k+1:  [a; b] <- G [a; b]
-            const int j0 = (k == l) ? l : k - 1;
-            for (int j = j0 + tid; j < n; j += blockDim.x) {
-                double2 a = A[k * lda + j], b = A[(k + 1) * lda + j];
-                A[k * lda + j] = cx * a + cy * b;
-                A[(k + 1) * lda + j] = cxc * b - cyc * a;
-            }
-            __syncthreads();
-            // columns k, k+1 of A (rows 0..min(k+2, hi)) and of Q (all rows):  [a, b] <- [a, b] G^H
-            const int i1 = min(k + 2, hi);
-            for (int i = tid; i < (i1 + 1) + n; i += blockDim.x) {
-                double2* row = i <= i1 ? A + i * lda : Q + (i - i1 - 1) * lda;
-                double2 a = row[k], b = row[k + 1];
-                row[k] = a * cxc + b * cyc;
-                row[k + 1] = b * cx - a * cy;
-            }
-            __syncthreads();
-            if (k > l && tid == 0) A[(k + 1) * lda + k - 1] = czero();
-            __syncthreads();
-        }
-    }
-    __syncthreads();
-    int fail = s_fail;
-    __syncthreads();
-    return fail;
-}
-
-// ---------------------------------------------------------------------------
-// The same reduction in double-float arithmetic (pairs of FP32 numbers, about
-// 48 significant bits; Knuth's two-sum and Dekker's FMA two-product, as for the
-// reliable-update residual), for the restart's eigen-solves of H^(m) and
-// H^(m-1): the FP32 pipeline issues 64 times faster than FP64 on this GPU, and
-// the Householder and QR updates are the bulk of the solve. A and Q keep their
-// 16-byte slots (one double2 or one double-float complex); the scalars of a
-// step (norms, shift, rotation) are formed by one thread in FP64. On return A,
-// Q hold T and the Schur vectors in FP64 again.
+// ------------------------------------------------------ double-float numbers
+// The restart's eigen-solves of H^(m) and H^(m-1) run the reduction in
+// double-float arithmetic (pairs of FP32 numbers, about 48 significant bits;
+// Knuth's two-sum and Dekker's FMA two-product, as for the reliable-update
+// residual): the FP32 pipe issues 64 times faster than FP64 on this GPU.
 __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
     const float p = a.h * b.h;
     float e = fmaf(a.h, b.h, -p);
@@ -251,382 +100,746 @@ __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
     const float h = p + e;
     return {h, e - (h - p)};
 }
-__device__ __forceinline__ dfc dc_mul(dfc a, dfc b) {
-    return {df_mul(a.x, b.x) - df_mul(a.y, b.y), df_mul(a.x, b.y) + df_mul(a.y, b.x)};
-}
-__device__ __forceinline__ dfc dc_conj(dfc a) { return {a.x, -a.y}; }
-__device__ __forceinline__ dfc dc_scale(dfl s, dfc a) { return {df_mul(s, a.x), df_mul(s, a.y)}; }
-__device__ __forceinline__ dfl dc_abs2(dfc a) { return df_mul(a.x, a.x) + df_mul(a.y, a.y); }
-__device__ __forceinline__ float dc_abs1f(dfc a) { return fabsf(a.x.h) + fabsf(a.y.h); }
 __device__ __forceinline__ dfc dc_from(double2 a) { return {df_split(a.x), df_split(a.y)}; }
 __device__ __forceinline__ double2 dc_to(dfc a) { return make_double2(df_value(a.x), df_value(a.y)); }
-__device__ __forceinline__ dfc dc_zero() { return {{0.f, 0.f}, {0.f, 0.f}}; }
-__device__ __forceinline__ dfc dc_one() { return {{1.f, 0.f}, {0.f, 0.f}}; }
-
-constexpr float EPS_DF = 1.4e-14f;   // about four units of double-float rounding
-
-__device__ int schur_df(double2* A64, double2* Q64, int n, int lda, double2* v64, double* sh) {
-    const int tid = threadIdx.x;
-    dfc* A = reinterpret_cast<dfc*>(A64);
-    dfc* Q = reinterpret_cast<dfc*>(Q64);
-    dfc* v = reinterpret_cast<dfc*>(v64);
-    for (int e = tid; e < n * lda; e += blockDim.x) {   // in place: each thread converts its own slots
-        if (e % lda < n) {
-            const double2 a = A64[e];
-            A[e] = dc_from(a);
-        }
-        Q[e] = ((e / lda) == (e % lda)) ? dc_one() : dc_zero();
-    }
-    __syncthreads();
-    // Householder reduction (columns already Hessenberg skipped, reflections up
-    // to the column's last nonzero), as in schur().
-    for (int k = 0; k + 2 < n; ++k) {
-        if (tid == 0) {
-            dfl nrm2 = {0.f, 0.f}, tail = {0.f, 0.f};
-            int last = k + 1;
-            for (int i = k + 1; i < n; ++i) {
-                const dfl a2 = dc_abs2(A[i * lda + k]);
-                nrm2 = nrm2 + a2;
-                if (i >= k + 2) tail = tail + a2;
-                if (a2.h != 0.f) last = i;
-            }
-            const double alpha = sqrt(df_value(nrm2));
-            const double2 x0 = dc_to(A[(k + 1) * lda + k]);
-            const double ax0 = cabs_(x0);
-            const double2 ph = ax0 > 0.0 ? make_double2(x0.x / ax0, x0.y / ax0) : make_double2(1.0, 0.0);
-            sh[0] = tail.h > 0.f ? alpha : 0.0;   // 0: skip the step
-            sh[1] = alpha > 0.0 ? 1.0 / (alpha * (alpha + ax0)) : 0.0;
-            sh[2] = ph.x; sh[3] = ph.y;
-            sh[5] = (double)last;
-        }
-        __syncthreads();
-        const double alpha = sh[0];
-        const dfl tau = df_split(sh[1]);
-        const double2 ph = make_double2(sh[2], sh[3]);
-        const int last = (int)sh[5];
-        if (alpha == 0.0) { __syncthreads(); continue; }
-        for (int i = k + 1 + tid; i <= last; i += blockDim.x) v[i - k - 1] = A[i * lda + k];
-        __syncthreads();
-        if (tid == 0) v[0] = v[0] + dc_from(make_double2(alpha * ph.x, alpha * ph.y));
-        __syncthreads();
-        const int len = last - k;
-        for (int j = k + tid; j < n; j += blockDim.x) {
-            dfc w = dc_zero();
-            for (int i = 0; i < len; ++i) w = w + dc_mul(dc_conj(v[i]), A[(k + 1 + i) * lda + j]);
-            w = dc_scale(tau, w);
-            for (int i = 0; i < len; ++i) A[(k + 1 + i) * lda + j] = A[(k + 1 + i) * lda + j] - dc_mul(v[i], w);
-        }
-        __syncthreads();
-        for (int i = tid; i < 2 * n; i += blockDim.x) {
-            dfc* row = i < n ? A + i * lda : Q + (i - n) * lda;
-            dfc u = dc_zero();
-            for (int l = 0; l < len; ++l) u = u + dc_mul(row[k + 1 + l], v[l]);
-            u = dc_scale(tau, u);
-            for (int l = 0; l < len; ++l) row[k + 1 + l] = row[k + 1 + l] - dc_mul(u, dc_conj(v[l]));
-        }
-        __syncthreads();
-        for (int i = k + 2 + tid; i <= last; i += blockDim.x) A[i * lda + k] = dc_zero();
-        __syncthreads();
-    }
-    if (tid == 0) {
-        dfl f = {0.f, 0.f};
-        for (int i = 0; i < n; ++i)
-            for (int j = (i > 0 ? i - 1 : 0); j < n; ++j) f = f + dc_abs2(A[i * lda + j]);
-        sh[4] = sqrt(df_value(f));
-    }
-    __syncthreads();
-    const float anorm = sh[4] > 0.0 ? (float)sh[4] : 1.f;
-    __shared__ int s_l, s_hi, s_fail;
-    __shared__ dfc s_cx, s_cy, s_mu;
-    if (tid == 0) { s_hi = n - 1; s_fail = 0; }
-    __syncthreads();
-    int iters = 0, total = 0;
-    while (true) {
-        if (tid == 0) {
-            const int hi = s_hi;
-            int l = hi;
-            while (l > 0) {
-                float tst = dc_abs1f(A[(l - 1) * lda + l - 1]) + dc_abs1f(A[l * lda + l]);
-                if (tst == 0.f) tst = anorm;
-                if (dc_abs1f(A[l * lda + l - 1]) <= EPS_DF * tst) { A[l * lda + l - 1] = dc_zero(); break; }
-                --l;
-            }
-            s_l = l;
-        }
-        __syncthreads();
-        const int hi = s_hi, l = s_l;
-        if (hi <= 0) break;
-        if (l == hi) {
-            __syncthreads();
-            if (tid == 0) s_hi = hi - 1;
-            iters = 0;
-            __syncthreads();
-            continue;
-        }
-        ++iters; ++total;
-        if (iters > 60 || total > 60 * n) { if (tid == 0) s_fail = 1; __syncthreads(); break; }
-        if (tid == 0) {   // Wilkinson shift in FP64
-            const double2 a = dc_to(A[(hi - 1) * lda + hi - 1]), b = dc_to(A[(hi - 1) * lda + hi]);
-            const double2 c = dc_to(A[hi * lda + hi - 1]), d = dc_to(A[hi * lda + hi]);
-            double2 mu;
-            if (iters % 11 == 10) {
-                mu = d + make_double2(0.75 * cabs1(c), 0.0);
-            } else {
-                const double2 t = 0.5 * (a - d);
-                const double2 bc = b * c;
-                const double2 disc2 = t * t + bc;
-                const double r = cabs_(disc2);
-                const double sx = sqrt(0.5 * (r + disc2.x));
-                double sy = sqrt(0.5 * (r - disc2.x));
-                if (disc2.y < 0) sy = -sy;
-                const double2 disc = make_double2(sx, sy);
-                const double2 den1 = t + disc, den2 = t - disc;
-                const double2 den = cabs2(den1) >= cabs2(den2) ? den1 : den2;
-                mu = cabs2(den) > 0.0 ? d - cdiv(bc, den) : d;
-            }
-            s_mu = dc_from(mu);
-        }
-        __syncthreads();
-        const dfc mu = s_mu;
-        for (int k = l; k < hi; ++k) {
-            if (tid == 0) {
-                dfc x, y;
-                if (k == l) { x = A[l * lda + l] - mu; y = A[(l + 1) * lda + l]; }
-                else { x = A[k * lda + k - 1]; y = A[(k + 1) * lda + k - 1]; }
-                const double n2 = df_value(dc_abs2(x) + dc_abs2(y));
-                if (n2 == 0.0) { s_cx = dc_one(); s_cy = dc_zero(); }
-                else {
-                    const dfl inv = df_split(rsqrt_fp64(n2));
-                    s_cx = dc_scale(inv, dc_conj(x));
-                    s_cy = dc_scale(inv, dc_conj(y));
-                }
-            }
-            __syncthreads();
-            const dfc cx = s_cx, cy = s_cy;
-            const dfc cxc = dc_conj(cx), cyc = dc_conj(cy);
-            const int j0 = (k == l) ? l : k - 1;
-            for (int j = j0 + tid; j < n; j += blockDim.x) {
-                const dfc a = A[k * lda + j], b = A[(k + 1) * lda + j];
-                A[k * lda + j] = dc_mul(cx, a) + dc_mul(cy, b);
-                A[(k + 1) * lda + j] = dc_mul(cxc, b) - dc_mul(cyc, a);
-            }
-            __syncthreads();
-            const int i1 = min(k + 2, hi);
-            for (int i = tid; i < (i1 + 1) + n; i += blockDim.x) {
-                dfc* row = i <= i1 ? A + i * lda : Q + (i - i1 - 1) * lda;
-                const dfc a = row[k], b = row[k + 1];
-                row[k] = dc_mul(a, cxc) + dc_mul(b, cyc);
-                row[k + 1] = dc_mul(b, cx) - dc_mul(a, cy);
-            }
-            __syncthreads();
-            if (k > l && tid == 0) A[(k + 1) * lda + k - 1] = dc_zero();
-            __syncthreads();
-        }
-    }
-    __syncthreads();
-    const int fail = s_fail;
-    for (int e = tid; e < n * lda; e += blockDim.x) {   // back to FP64, in place
-        if (e % lda < n) {
-            const dfc a = A[e];
-            A64[e] = dc_to(a);
-        }
-        const dfc q = Q[e];
-        Q64[e] = dc_to(q);
-    }
-    __syncthreads();
-    return fail;
+__device__ __forceinline__ dfl df_scale(dfl a, float s) { return {a.h * s, a.l * s}; }   // s a power of two
+__device__ __forceinline__ dfl df_fast_sum(float h, float l) {   // |l| small against |h|
+    const float s = h + l;
+    return {s, l - (s - h)};
 }
-
-// Order of the eigenvalues on the diagonal of T: smallest |lambda|, then Im.
-__device__ void order_eigs(const double2* T, int n, int lda, int* ord) {
-    if (threadIdx.x == 0) {
-        // squared moduli order the same way as moduli (ties included)
-        for (int i = 0; i < n; ++i) ord[i] = i;
-        for (int i = 1; i < n; ++i) {
-            int key = ord[i];
-            double2 lk = T[key * lda + key];
-            double ak = cabs2(lk);
-            int j = i - 1;
-            while (j >= 0) {
-                double2 lj = T[ord[j] * lda + ord[j]];
-                double aj = cabs2(lj);
-                bool after = (aj > ak) || (aj == ak && lj.y > lk.y);
-                if (!after) break;
-                ord[j + 1] = ord[j];
-                --j;
-            }
-            ord[j + 1] = key;
-        }
-    }
-    __syncthreads();
+// 1/sqrt(a), a.h inside [1e-28, 1e28]: FP32 seed and one third-order step whose
+// residual e = 1 - a y^2 keeps every product's rounding error.
+__device__ __forceinline__ dfl df_rsqrt(dfl a) {
+    const float y = rsqrtf(a.h);
+    const float t = y * y, tl = fmaf(y, y, -t);
+    float e = fmaf(-a.h, t, 1.f);
+    e = fmaf(-a.l, t, e);
+    e = fmaf(-a.h, tl, e);
+    return df_fast_sum(y, y * (e * fmaf(0.375f, e, 0.5f)));
 }
-
-// Eigenvectors for the eigenvalues T[ord[i], ord[i]], i < nsel.
-// Y, Z (global or shared), column i of an n x nsel row-major array (ld = ldyz).
-// W1, W2: scratch of n*nsel each (y', w in Schur coordinates).
-__device__ void eigvecs(const double2* T, const double2* Q, int n, int lda, const int* ord, int nsel,
-                        double2* Y, double2* Z, int ldyz, double2* W1, double2* W2, double anorm) {
-    const int tid = threadIdx.x;
-    const double smin = fmax(EPS * anorm, 1e-300);
-    // Back / forward substitution, one (vector, side) per thread.
-    for (int t = tid; t < 2 * nsel; t += blockDim.x) {
-        const int i = t % nsel;
-        const bool left = t >= nsel;
-        const int k = ord[i];
-        const double2 lam = T[k * lda + k];
-        double2* w = (left ? W2 : W1) + (size_t)i * n;
-        for (int j = 0; j < n; ++j) w[j] = czero();
-        w[k] = cone();
-        if (!left) {
-            for (int j = k - 1; j >= 0; --j) {
-                double2 sacc = czero();
-                for (int l = j + 1; l <= k; ++l) sacc = sacc + T[j * lda + l] * w[l];
-                double2 d = T[j * lda + j] - lam;
-                if (cabs1(d) < smin) d = make_double2(smin, 0.0);
-                w[j] = -(rcp_fp64(cabs2(d)) * (sacc * conj_(d)));
-                if (cabs1(w[j]) > 1e150) {
-                    for (int l = j; l <= k; ++l) w[l] = 1e-150 * w[l];
-                }
-            }
-        } else {
-            for (int j = k + 1; j < n; ++j) {
-                double2 sacc = czero();
-                for (int l = k; l < j; ++l) sacc = sacc + w[l] * T[l * lda + j];
-                double2 d = T[j * lda + j] - lam;
-                if (cabs1(d) < smin) d = make_double2(smin, 0.0);
-                w[j] = -(rcp_fp64(cabs2(d)) * (sacc * conj_(d)));
-                if (cabs1(w[j]) > 1e150) {
-                    for (int l = k; l <= j; ++l) w[l] = 1e-150 * w[l];
-                }
-            }
-        }
-    }
-    __syncthreads();
-    // Y = Q y', Z = Q conj(w)
-    for (int e = tid; e < 2 * n * nsel; e += blockDim.x) {
-        const bool left = e >= n * nsel;
-        const int ee = left ? e - n * nsel : e;
-        const int row = ee / nsel, i = ee % nsel;
-        const double2* w = (left ? W2 : W1) + (size_t)i * n;
-        double2 acc = czero();
-        for (int l = 0; l < n; ++l) acc = acc + Q[row * lda + l] * (left ? conj_(w[l]) : w[l]);
-        (left ? Z : Y)[row * ldyz + i] = acc;
-    }
-    __syncthreads();
-    // Normalise: ||y|| = 1, largest entry real positive, z^H y = 1.
-    for (int i = tid; i < nsel; i += blockDim.x) {
-        double nrm2 = 0.0, best = -1.0;
-        int arg = 0;
-        for (int r = 0; r < n; ++r) {
-            double a2 = cabs2(Y[r * ldyz + i]);
-            nrm2 += a2;
-            if (a2 > best) { best = a2; arg = r; }
-        }
-        double nrm = sqrt(nrm2);
-        double2 pk = Y[arg * ldyz + i];
-        double apk = cabs_(pk);
-        // factor = conj(pk)/|pk| / nrm
-        double2 f = (apk > 0.0 && nrm > 0.0) ? (1.0 / (apk * nrm)) * conj_(pk) : make_double2(nrm > 0.0 ? 1.0 / nrm : 1.0, 0.0);
-        double2 d = czero();
-        for (int r = 0; r < n; ++r) {
-            double2 yv = f * Y[r * ldyz + i];
-            Y[r * ldyz + i] = yv;
-            d = d + cdot(Z[r * ldyz + i], yv);
-        }
-        double2 g = cabs2(d) > 0.0 ? cdiv(cone(), conj_(d)) : cone();
-        for (int r = 0; r < n; ++r) Z[r * ldyz + i] = g * Z[r * ldyz + i];
-    }
-    __syncthreads();
+// 1/a the same way.
+__device__ __forceinline__ dfl df_rcp(dfl a) {
+    const float y = __frcp_rn(a.h);
+    float e = fmaf(-a.h, y, 1.f);
+    e = fmaf(-a.l, y, e);
+    return df_fast_sum(y, y * fmaf(e, e, e));
 }
+__device__ __forceinline__ bool df_seed_ok(float h) { return h > 1e-28f && h < 1e28f; }
 
-// Full eigen-solve of the n x n matrix in A (shared). Outputs sorted
-// eigenvalues to lam (n), and vectors for the first nsel.
-__device__ int eig_block(double2* A, double2* Q, int n, int lda, int nsel, double2* lam, double2* Y,
-                         double2* Z, int ldyz, double2* W1, double2* W2, double2* v, double* sh, int* ord,
-                         bool dfloat = false) {
-    int fail = dfloat ? schur_df(A, Q, n, lda, v, sh) : schur(A, Q, n, lda, v, sh);
-    double anorm = sh[4];
-    order_eigs(A, n, lda, ord);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) lam[i] = A[ord[i] * lda + ord[i]];
-    __syncthreads();
-    if (nsel > 0) eigvecs(A, Q, n, lda, ord, nsel, Y, Z, ldyz, W1, W2, anorm);
-    return fail;
-}
-
-// Dynamic shared memory layout for an eigen CTA of capacity nmax.
-struct EigSmem {
-    double2* A; double2* Q; double2* v; double* sh; int* ord;
-    __device__ EigSmem(char* base, int nmax) {
-        A = reinterpret_cast<double2*>(base);
-        Q = A + nmax * nmax;
-        v = Q + nmax * nmax;
-        sh = reinterpret_cast<double*>(v + nmax);
-        ord = reinterpret_cast<int*>(sh + 8);
+// ------------------------------------------------------- number types
+// What the reduction needs of a complex number type C: u a + v b, c - a b,
+// running sums of products, the rotation, the shift and the negligibility test.
+struct NumD {
+    using C = double2;
+    using R = double;
+    static __device__ __forceinline__ C zero() { return czero(); }
+    static __device__ __forceinline__ C one() { return cone(); }
+    static __device__ __forceinline__ C from(double2 a) { return a; }
+    static __device__ __forceinline__ double2 to(C a) { return a; }
+    static __device__ __forceinline__ C lin2(C u, C a, C v, C b) {
+        return make_double2(fma(-v.y, b.y, fma(v.x, b.x, fma(-u.y, a.y, u.x * a.x))),
+                            fma(v.y, b.x, fma(v.x, b.y, fma(u.y, a.x, u.x * a.y))));
     }
-    static size_t bytes(int nmax) {
-        return (size_t)(2 * nmax * nmax + nmax) * sizeof(double2) + 8 * sizeof(double) + nmax * sizeof(int) + 16;
+    static __device__ __forceinline__ C fms(C c, C a, C b) {
+        return make_double2(fma(a.y, b.y, fma(-a.x, b.x, c.x)), fma(-a.y, b.x, fma(-a.x, b.y, c.y)));
+    }
+    static __device__ __forceinline__ C scale(R s, C a) { return s * a; }
+    struct Sum {
+        C s = czero();
+        __device__ __forceinline__ void add(C a, C b) {
+            s = make_double2(fma(-a.y, b.y, fma(a.x, b.x, s.x)), fma(a.y, b.x, fma(a.x, b.y, s.y)));
+        }
+        __device__ __forceinline__ C value() const { return s; }
+    };
+    static __device__ __forceinline__ R abs2(C a) { return fma(a.y, a.y, a.x * a.x); }
+    static __device__ __forceinline__ R add(R a, R b) { return a + b; }
+    static __device__ __forceinline__ double rvalue(R a) { return a; }
+    static __device__ __forceinline__ R rfrom(double a) { return a; }
+    static __device__ __forceinline__ R rzero() { return 0.0; }
+    static __device__ __forceinline__ R shfl_xor(R a, int o) { return __shfl_xor_sync(FULL, a, o); }
+    static __device__ __forceinline__ bool negligible(C sub, C d0, C d1, double anorm) {
+        double t = cabs1(d0) + cabs1(d1);
+        if (t == 0.0) t = anorm;
+        return cabs1(sub) <= EPS * t;
+    }
+    static __device__ __forceinline__ double wide_abs2(C a) { return abs2(a); }
+    // G = [[cx, cy], [-conj(cy), conj(cx)]] with G [x; y] = [n; 0], cx = conj(x)/n,
+    // cy = conj(y)/n, n = sqrt(|x|^2 + |y|^2).
+    static __device__ __forceinline__ void givens(C x, C y, C& cx, C& cy) {
+        const double n2 = abs2(x) + abs2(y);
+        if (!mid_range(n2) && n2 == 0.0) { cx = one(); cy = zero(); return; }
+        const double inv = rsqrt_fp64(n2);
+        cx = make_double2(inv * x.x, -(inv * x.y));
+        cy = make_double2(inv * y.x, -(inv * y.y));
     }
 };
 
+struct NumF {
+    using C = dfc;
+    using R = dfl;
+    static __device__ __forceinline__ C zero() { return {{0.f, 0.f}, {0.f, 0.f}}; }
+    static __device__ __forceinline__ C one() { return {{1.f, 0.f}, {0.f, 0.f}}; }
+    static __device__ __forceinline__ C from(double2 a) { return dc_from(a); }
+    static __device__ __forceinline__ double2 to(C a) { return dc_to(a); }
+    static __device__ __forceinline__ C lin2(C u, C a, C v, C b) {
+        Dot2 re, im;
+        re.first(u.x, a.x); re.add(-u.y, a.y); re.add(v.x, b.x); re.add(-v.y, b.y);
+        im.first(u.x, a.y); im.add(u.y, a.x); im.add(v.x, b.y); im.add(v.y, b.x);
+        return {re.done(), im.done()};
+    }
+    static __device__ __forceinline__ C mul(C a, C b) {
+        Dot2 re, im;
+        re.first(a.x, b.x); re.add(-a.y, b.y);
+        im.first(a.x, b.y); im.add(a.y, b.x);
+        return {re.done(), im.done()};
+    }
+    static __device__ __forceinline__ C fms(C c, C a, C b) {
+        Dot2 re{c.x.h, c.x.l}, im{c.y.h, c.y.l};
+        re.add(-a.x, b.x); re.add(a.y, b.y);
+        im.add(-a.x, b.y); im.add(-a.y, b.x);
+        return {re.done(), im.done()};
+    }
+    static __device__ __forceinline__ C scale(R s, C a) { return {df_mul(s, a.x), df_mul(s, a.y)}; }
+    struct Sum {
+        Dot2 re{0.f, 0.f}, im{0.f, 0.f};
+        __device__ __forceinline__ void add(C a, C b) {
+            re.add(a.x, b.x); re.add(-a.y, b.y);
+            im.add(a.x, b.y); im.add(a.y, b.x);
+        }
+        __device__ __forceinline__ C value() const { return {re.done(), im.done()}; }
+    };
+    static __device__ __forceinline__ R abs2(C a) {
+        Dot2 s;
+        s.first(a.x, a.x);
+        s.add(a.y, a.y);
+        return s.done();
+    }
+    static __device__ __forceinline__ R add(R a, R b) { return a + b; }
+    static __device__ __forceinline__ double rvalue(R a) { return df_value(a); }
+    static __device__ __forceinline__ R rfrom(double a) { return df_split(a); }
+    static __device__ __forceinline__ R rzero() { return {0.f, 0.f}; }
+    static __device__ __forceinline__ R shfl_xor(R a, int o) {
+        return {__shfl_xor_sync(FULL, a.h, o), __shfl_xor_sync(FULL, a.l, o)};
+    }
+    static constexpr float EPS_DF = 1.4e-14f;   // about four units of double-float rounding
+    static __device__ __forceinline__ float abs1(C a) { return fabsf(a.x.h) + fabsf(a.y.h); }
+    static __device__ __forceinline__ bool negligible(C sub, C d0, C d1, double anorm) {
+        float t = abs1(d0) + abs1(d1);
+        if (t == 0.f) t = (float)anorm;
+        return abs1(sub) <= EPS_DF * t;
+    }
+    static __device__ __forceinline__ double wide_abs2(C a) { return df_value(abs2(a)); }
+    static __device__ __forceinline__ void givens(C x, C y, C& cx, C& cy) {
+        Dot2 s;
+        s.first(x.x, x.x); s.add(x.y, x.y); s.add(y.x, y.x); s.add(y.y, y.y);
+        const dfl n2 = s.done();
+        dfl inv;
+        if (df_seed_ok(n2.h)) {
+            inv = df_rsqrt(n2);
+        } else {
+            if (n2.h == 0.f) { cx = one(); cy = zero(); return; }
+            inv = df_split(rsqrt_fp64(df_value(n2)));
+        }
+        cx = {df_mul(inv, x.x), -df_mul(inv, x.y)};
+        cy = {df_mul(inv, y.x), -df_mul(inv, y.y)};
+    }
+};
+
+// Wilkinson shift of [[a, b], [c, d]]: the eigenvalue nearer d is d - corr with
+// corr = b c / (t + sqrt(t^2 + b c)), t = (a - d)/2, with the larger denominator.
+// A shift only steers the convergence, so double-float arithmetic serves both
+// number types, on entries scaled by a power of two (max |entry| near 1), so that
+// FP32's exponent range does not matter. Returns corr of the scaled entries.
+__device__ __forceinline__ dfc shift_correction(dfc a, dfc b, dfc c, dfc d) {
+    const dfc t = {df_scale(a.x - d.x, 0.5f), df_scale(a.y - d.y, 0.5f)};
+    const dfc bc = NumF::mul(b, c);
+    const dfc q = NumF::lin2(t, t, b, c);   // t^2 + b c
+    const dfl m2 = NumF::abs2(q);
+    dfc s = NumF::zero();   // sqrt(q), principal branch
+    if (m2.h > 1e-36f) {    // |entries| <= 2, so no upper bound is needed
+        const dfl m = df_mul(m2, df_rsqrt(m2));
+        // the larger of |Re s|, |Im s| from (|q| + |Re q|)/2, the other from Im q
+        const bool pos = q.x.h >= 0.f;
+        const dfl w = df_scale(m + (pos ? q.x : -q.x), 0.5f);
+        const dfl iw = df_rsqrt(w), big = df_mul(w, iw), small = df_scale(df_mul(q.y, iw), 0.5f);
+        if (pos) s = {big, small};
+        else s = q.y.h < 0.f ? dfc{-small, -big} : dfc{small, big};
+    }
+    const dfc p = t + s, n = t - s;
+    const dfl ap = NumF::abs2(p), an = NumF::abs2(n);
+    const bool plus = ap.h >= an.h;
+    const dfc den = plus ? p : n;
+    const dfl d2 = plus ? ap : an;
+    if (!df_seed_ok(d2.h)) return NumF::zero();
+    const dfc num = NumF::mul(bc, {den.x, -den.y});
+    const dfl r = df_rcp(d2);
+    return {df_mul(num.x, r), df_mul(num.y, r)};
+}
+// An FP64 number in FP32's exponent range (or zero) as h + l, both parts truncated:
+// one FP64 instruction instead of four (conversions run on the FP64 pipe).
+__device__ __forceinline__ dfl quick_split(double v) {
+    const double m = fabs(v);
+    if (!mid_range(m)) return {0.f, 0.f};
+    const float h = seed_f32(m);
+    const double r = m - exact_f64(h);   // >= 0, exact
+    const float l = mid_range(r) ? seed_f32(r) : 0.f;
+    return v < 0.0 ? dfl{-h, -l} : dfl{h, l};
+}
+__device__ double2 wilkinson_shift(double2 a, double2 b, double2 c, double2 d) {
+    const unsigned hw[8] = {(unsigned)__double2hiint(a.x), (unsigned)__double2hiint(a.y), (unsigned)__double2hiint(b.x),
+                            (unsigned)__double2hiint(b.y), (unsigned)__double2hiint(c.x), (unsigned)__double2hiint(c.y),
+                            (unsigned)__double2hiint(d.x), (unsigned)__double2hiint(d.y)};
+    unsigned ex = 0;   // largest exponent field
+#pragma unroll
+    for (int i = 0; i < 8; ++i) ex = max(ex, (hw[i] >> 20) & 0x7ffu);
+    if (ex < 64u || ex > 1982u) return d;   // zero, non-finite or near the ends of FP64's range
+    const double up = __hiloint2double((int)(2046u - ex) << 20, 0), down = __hiloint2double((int)ex << 20, 0);
+    auto in = [&](double2 v) { return dfc{quick_split(up * v.x), quick_split(up * v.y)}; };   // 2^(1023-ex) v
+    return d - down * dc_to(shift_correction(in(a), in(b), in(c), in(d)));
+}
+__device__ dfc wilkinson_shift(dfc a, dfc b, dfc c, dfc d) {
+    float mx = fmaxf(fmaxf(NumF::abs1(a), NumF::abs1(b)), fmaxf(NumF::abs1(c), NumF::abs1(d)));
+    if (!(mx > 1e-30f && mx < 1e30f)) return d;
+    const unsigned ex = __float_as_uint(mx) & 0x7f800000u;
+    const float up = __uint_as_float(0x7f000000u - ex), down = __uint_as_float(ex);   // 2^(127-e), 2^(e-127)
+    auto in = [&](dfc v) { return dfc{df_scale(v.x, up), df_scale(v.y, up)}; };
+    const dfc r = shift_correction(in(a), in(b), in(c), in(d));
+    return d - dfc{df_scale(r.x, down), df_scale(r.y, down)};
+}
+__device__ __forceinline__ double2 exceptional_shift(double2 c, double2 d) { return d + make_double2(0.75 * cabs1(c), 0.0); }
+__device__ __forceinline__ dfc exceptional_shift(dfc c, dfc d) { return d + dfc{{0.75f * NumF::abs1(c), 0.f}, {0.f, 0.f}}; }
+
+// ---------------------------------------------------------------------------
+// Block-cooperative reduction of A (n x n, row stride lda, shared memory, numbers
+// of type M::C in 16-byte slots) to Schur form: on return A holds T and Q the
+// Schur vectors, both in FP64. Returns 0 on success, 1 if QR failed to
+// converge. v: n slots; sh: 8 doubles (sh[4] = Frobenius norm of the Hessenberg
+// form on return). lda is odd, so that a column is read without bank conflicts.
+//
+// Half-warps share each pair of a rotation: lanes 0-15 form the first output of
+// 16 pairs, lanes 16-31 the second, after both have read the pair.
+template <class M>
+__device__ int schur(double2* A64, double2* Q64, int n, int lda, double2* v64, double* sh) {
+    using C = typename M::C;
+    using R = typename M::R;
+    static_assert(sizeof(C) == sizeof(double2), "numbers are converted in place");
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    C* A = reinterpret_cast<C*>(A64);
+    C* Q = reinterpret_cast<C*>(Q64);
+    C* v = reinterpret_cast<C*>(v64);
+    __shared__ C s_cx[2], s_cy[2];
+    __shared__ R s_tau;
+    __shared__ int s_len, s_l, s_hi, s_fail;
+    for (int e = tid; e < n * lda; e += ET) {   // in place: each thread converts its own slots
+        const int i = e / lda, j = e % lda;
+        if (j < n) {
+            const double2 a = A64[e];
+            A[e] = M::from(a);
+        }
+        Q[e] = i == j ? M::one() : M::zero();
+    }
+    __syncthreads();
+    // Householder reduction to upper Hessenberg. A column with nothing below its
+    // subdiagonal is skipped, and a reflection spans only the rows up to the
+    // column's last nonzero: the projected matrices of eigBiCG are tridiagonal,
+    // or after a restart diagonal + coupling arrow + tridiagonal, so most
+    // columns need no work. Warp 0 forms the reflection, a column element per lane.
+    for (int k = 0; k + 2 < n; ++k) {
+        if (warp == 0) {
+            R nrm2 = M::rzero(), tail = M::rzero();
+            int last = k + 1;
+            for (int i = k + 1 + lane; i < n; i += 32) {
+                const R a2 = M::abs2(A[i * lda + k]);
+                nrm2 = M::add(nrm2, a2);
+                if (i >= k + 2) tail = M::add(tail, a2);
+                if (M::rvalue(a2) != 0.0) last = i;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                nrm2 = M::add(nrm2, M::shfl_xor(nrm2, o));
+                tail = M::add(tail, M::shfl_xor(tail, o));
+                last = max(last, __shfl_xor_sync(FULL, last, o));
+            }
+            const bool work = M::rvalue(tail) > 0.0;
+            if (work) {   // v = x + e^{i theta} ||x|| e1, tau = 2/||v||^2
+                const double alpha = sqrt_fp64(M::rvalue(nrm2));
+                const double2 x0 = M::to(A[(k + 1) * lda + k]);
+                const double a0 = NumD::abs2(x0);
+                double2 ph = cone();
+                double ax0 = 0.0;
+                if (a0 > 0.0) {
+                    const double r0 = rsqrt_fp64(a0);
+                    ax0 = a0 * r0;
+                    ph = r0 * x0;
+                }
+                for (int i = k + 1 + lane; i <= last; i += 32) {
+                    C x = A[i * lda + k];
+                    if (i == k + 1) x = M::from(x0 + alpha * ph);
+                    v[i - k - 1] = x;
+                }
+                if (lane == 0) s_tau = M::rfrom(rcp_fp64(alpha * (alpha + ax0)));
+            }
+            if (lane == 0) s_len = work ? last - k : 0;
+        }
+        __syncthreads();
+        const int len = s_len;
+        if (len == 0) { __syncthreads(); continue; }
+        const R tau = s_tau;
+        // rows k+1..last of A: A -= tau v (v^H A), columns k..n-1
+        for (int j = k + tid; j < n; j += ET) {
+            typename M::Sum w;
+            for (int i = 0; i < len; ++i) w.add(conj_(v[i]), A[(k + 1 + i) * lda + j]);
+            const C tw = M::scale(tau, w.value());
+            for (int i = 0; i < len; ++i) A[(k + 1 + i) * lda + j] = M::fms(A[(k + 1 + i) * lda + j], v[i], tw);
+        }
+        __syncthreads();
+        // columns k+1..last of A (all rows) and of Q: X -= tau (X v) v^H; column k below the subdiagonal is zero
+        for (int i = tid; i < 2 * n; i += ET) {
+            C* row = (i < n ? A + i * lda : Q + (i - n) * lda) + k + 1;
+            typename M::Sum u;
+            for (int l = 0; l < len; ++l) u.add(row[l], v[l]);
+            const C tu = M::scale(tau, u.value());
+            for (int l = 0; l < len; ++l) row[l] = M::fms(row[l], tu, conj_(v[l]));
+            if (i >= k + 2 && i <= k + len) A[i * lda + k] = M::zero();
+        }
+        __syncthreads();
+    }
+    // Frobenius norm for the negligibility tests.
+    {
+        double f = 0.0;
+        for (int e = tid; e < n * n; e += ET) {
+            const int i = e / n, j = e % n;
+            if (j + 1 >= i) f += M::wide_abs2(A[i * lda + j]);
+        }
+        f = warp_sum(f);
+        __shared__ double s_f[EW];
+        if (lane == 0) s_f[warp] = f;
+        __syncthreads();
+        if (tid == 0) {
+            double t = 0.0;
+            for (int w = 0; w < EW; ++w) t += s_f[w];
+            sh[4] = sqrt(t);
+            s_fail = 0;
+        }
+        __syncthreads();
+    }
+    const double anorm = sh[4] > 0.0 ? sh[4] : 1.0;
+    // Single-shift implicit QR with deflation from the bottom. Warp 0 steers: it
+    // scans the subdiagonal (one entry per lane), forms the shift and the first
+    // rotation of a sweep, and each next rotation as soon as its own rows of the
+    // column update are done.
+    const int half = lane >> 4;
+    int hi = n - 1, iters = 0, total = 0;   // warp 0 only
+    while (true) {
+        if (warp == 0) {
+            int l = 0;
+            bool fail = false;
+            while (hi > 0) {
+                l = 0;
+                for (int base = hi & ~31; base >= 0; base -= 32) {
+                    const int i = base + lane;
+                    const bool neg = i > 0 && i <= hi &&
+                                     M::negligible(A[i * lda + i - 1], A[(i - 1) * lda + i - 1], A[i * lda + i], anorm);
+                    const unsigned b = __ballot_sync(FULL, neg);
+                    if (b) { l = base + 31 - __clz(b); break; }
+                }
+                if (l < hi) break;
+                --hi;
+                iters = 0;
+            }
+            if (hi > 0) {
+                ++iters; ++total;
+                fail = iters > 60 || total > 60 * n;
+                if (!fail) {
+                    const C c = A[hi * lda + hi - 1], d = A[hi * lda + hi];
+                    const C mu = iters % 11 == 10 ? exceptional_shift(c, d)
+                                                  : wilkinson_shift(A[(hi - 1) * lda + hi - 1], A[(hi - 1) * lda + hi], c, d);
+                    C cx, cy;
+                    M::givens(A[l * lda + l] - mu, A[(l + 1) * lda + l], cx, cy);
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (l > 0) A[l * lda + l - 1] = M::zero();
+                        s_cx[l & 1] = cx;
+                        s_cy[l & 1] = cy;
+                    }
+                }
+            }
+            if (lane == 0) {
+                s_l = l;
+                s_hi = fail ? 0 : hi;
+                if (fail) s_fail = 1;
+            }
+        }
+        __syncthreads();
+        const int l = s_l, h = s_hi;
+        if (h <= 0) break;
+        for (int k = l; k < h; ++k) {
+            const C cx = s_cx[k & 1], cy = s_cy[k & 1];
+            // rows k, k+1:  [a; b] <- G [a; b]
+            {
+                const int j0 = k == l ? l : k - 1;
+                const C u = half ? conj_(cx) : cx, w = half ? -conj_(cy) : cy;
+                C* row = A + (k + half) * lda;
+                const C* oth = A + (k + 1 - half) * lda;
+                for (int base = j0 + (warp << 4); base < n; base += 16 * EW) {
+                    const int j = base + (lane & 15), jc = min(j, n - 1);
+                    C out = M::lin2(u, row[jc], w, oth[jc]);
+                    if (half && j < k) out = M::zero();   // the bulge entry that the rotation annihilates
+                    __syncwarp();
+                    if (j < n) row[j] = out;
+                }
+            }
+            __syncthreads();
+            // columns k, k+1 of A (rows 0..min(k+2, h), from the last upwards) and of Q
+            // (all rows):  [a, b] <- [a, b] G^H
+            {
+                const int i1 = min(k + 2, h);
+                const C u = half ? cx : conj_(cx), w = half ? -cy : conj_(cy);
+                for (int base = warp << 4; base < i1 + 1 + n; base += 16 * EW) {
+                    const int t = base + (lane & 15), tc = min(t, i1 + n);
+                    C* row = (tc <= i1 ? A + (i1 - tc) * lda : Q + (tc - i1 - 1) * lda) + k;
+                    const C out = M::lin2(u, row[half], w, row[1 - half]);
+                    __syncwarp();
+                    if (t == tc) row[half] = out;
+                    // rows k+1 and k+2 are warp 0's first: the next rotation
+                    if (base == 0 && k + 1 < h) {
+                        __syncwarp();
+                        C nx, ny;
+                        M::givens(A[(k + 1) * lda + k], A[(k + 2) * lda + k], nx, ny);
+                        if (lane == 0) { s_cx[(k + 1) & 1] = nx; s_cy[(k + 1) & 1] = ny; }
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+    const int fail = s_fail;
+    __syncthreads();
+    for (int e = tid; e < n * lda; e += ET) {   // back to FP64, in place
+        if (e % lda < n) {
+            const C a = A[e], q = Q[e];
+            A64[e] = M::to(a);
+            Q64[e] = M::to(q);
+        }
+    }
+    __syncthreads();
+    return fail;
+}
+
+// Order of the eigenvalues on the diagonal of T: smallest |lambda|, then Im, then
+// position. Squared moduli order the same way as moduli (ties included). key: n slots.
+__device__ void order_eigs(const double2* T, int n, int lda, int* ord, double2* key) {
+    for (int i = threadIdx.x; i < n; i += ET) {
+        key[i] = make_double2(cabs2(T[i * lda + i]), T[i * lda + i].y);
+        ord[i] = i;   // every slot a valid index, should a NaN leave one without a rank
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += ET) {
+        const double2 a = key[i];
+        int rank = 0;
+        for (int j = 0; j < n; ++j) {
+            const double2 b = key[j];
+            const bool before = b.x < a.x || (b.x == a.x && (b.y < a.y || (b.y == a.y && j < i)));
+            rank += before ? 1 : 0;
+        }
+        ord[rank] = i;
+    }
+    __syncthreads();
+}
+
+constexpr int ES = (MAX_SMALL + 31) / 32;   // elements of a vector per lane
+
+__device__ __forceinline__ double2 shfl_c(double2 a, int src) {
+    return make_double2(__shfl_sync(FULL, a.x, src), __shfl_sync(FULL, a.y, src));
+}
+
+// Eigenvectors for the eigenvalues T[ord[i], ord[i]], i < nsel, one warp per
+// eigenvalue. Y, Z (global), column i of an n x nsel row-major array (ld =
+// ldyz). wbuf: n slots per warp. rev: T is of the matrix with rows and columns in
+// reverse order (load_reversed); the vectors are written in the original order.
+// Substitution in outer-product form: as soon as w_l is known, every lane adds
+// its rows' terms with w_l, so a step is two dependent complex multiply-adds
+// whatever the length (the row-sum form is a serial chain of that length).
+__device__ void eigvecs(const double2* T, const double2* Q, int n, int lda, const int* ord, int nsel,
+                        double2* Y, double2* Z, int ldyz, double2* wbuf, double anorm, bool rev) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double smin = fmax(EPS * anorm, 1e-300);
+    double2* wb = wbuf + warp * n;
+    for (int i = warp; i < nsel; i += EW) {
+        const int k = ord[i];
+        const double2 lam = T[k * lda + k];
+        double2 dinv[ES], vec[2][ES];
+#pragma unroll
+        for (int t = 0; t < ES; ++t) {
+            const int j = lane + 32 * t;
+            dinv[t] = czero();
+            if (j < n && j != k) {
+                double2 d = T[j * lda + j] - lam;
+                if (cabs1(d) < smin) d = make_double2(smin, 0.0);
+                const double m = fmax(fabs(d.x), fabs(d.y));
+                if (m > 1e-14 && m < 1e14) dinv[t] = rcp_fp64(cabs2(d)) * conj_(d);
+                else dinv[t] = cdiv(cone(), d);
+            }
+        }
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {   // 0: right (rows above k), 1: left (columns right of k)
+            double2 s[ES];
+#pragma unroll
+            for (int t = 0; t < ES; ++t) {
+                const int j = lane + 32 * t;
+                s[t] = czero();
+                if (side == 0 ? j < k : (j > k && j < n)) s[t] = side == 0 ? T[j * lda + k] : T[k * lda + j];
+                if (j < n) wb[j] = j == k ? cone() : czero();
+            }
+            __syncwarp();
+            const int steps = side == 0 ? k : n - 1 - k;
+            for (int q = 1; q <= steps; ++q) {
+                const int l = side == 0 ? k - q : k + q;
+                const int own = l >> 5;
+                double2 sv = s[0], dv = dinv[0];
+#pragma unroll
+                for (int t = 1; t < ES; ++t)
+                    if (own == t) { sv = s[t]; dv = dinv[t]; }
+                double2 w = shfl_c(-(sv * dv), l & 31);
+                // |w| above about 1e150 (exponent test): rescale the whole vector
+                if (max(__double2hiint(w.x) & 0x7fffffff, __double2hiint(w.y) & 0x7fffffff) > 0x5f100000) {
+                    __syncwarp();
+                    w = 1e-150 * w;
+#pragma unroll
+                    for (int t = 0; t < ES; ++t) {
+                        const int j = lane + 32 * t;
+                        s[t] = 1e-150 * s[t];
+                        if (j < n) wb[j] = 1e-150 * wb[j];
+                    }
+                    __syncwarp();
+                }
+                if (lane == 0) wb[l] = w;
+#pragma unroll
+                for (int t = 0; t < ES; ++t) {
+                    const int j = lane + 32 * t;
+                    if (side == 0 ? 32 * t < l : 32 * t + 31 > l)   // warp-uniform: this slice still has rows to go
+                        if (side == 0 ? j < l : (j > l && j < n))
+                            s[t] = NumD::fms(s[t], -(side == 0 ? T[j * lda + l] : T[l * lda + j]), w);
+                }
+            }
+            __syncwarp();
+            // y = Q y', z = Q conj(w)
+            double2 acc[ES];
+#pragma unroll
+            for (int t = 0; t < ES; ++t) acc[t] = czero();
+            const int l0 = side == 0 ? 0 : k, l1 = side == 0 ? k : n - 1;
+            for (int l = l0; l <= l1; ++l) {
+                const double2 w = side == 0 ? wb[l] : conj_(wb[l]);
+#pragma unroll
+                for (int t = 0; t < ES; ++t) {
+                    const int r = lane + 32 * t;
+                    if (32 * t < n && r < n) acc[t] = NumD::fms(acc[t], -Q[r * lda + l], w);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < ES; ++t) vec[side][t] = acc[t];
+            __syncwarp();
+        }
+        // Normalise: ||y|| = 1, largest entry real positive, z^H y = 1.
+        double nrm2 = 0.0, best = -1.0;
+        int arg = 0;
+#pragma unroll
+        for (int t = 0; t < ES; ++t) {
+            const int r = lane + 32 * t;
+            if (r < n) {
+                const double a2 = cabs2(vec[0][t]);
+                nrm2 += a2;
+                if (a2 > best || (rev && a2 == best)) { best = a2; arg = r; }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            nrm2 += __shfl_xor_sync(FULL, nrm2, o);
+            const double ob = __shfl_xor_sync(FULL, best, o);
+            const int oa = __shfl_xor_sync(FULL, arg, o);
+            if (ob > best || (ob == best && (rev ? oa > arg : oa < arg))) { best = ob; arg = oa; }
+        }
+        double2 pk = vec[0][0];
+#pragma unroll
+        for (int t = 1; t < ES; ++t)
+            if ((arg >> 5) == t) pk = vec[0][t];
+        pk = shfl_c(pk, arg & 31);
+        // factor = conj(pk)/|pk| / nrm
+        const double inrm = nrm2 > 0.0 ? rsqrt_fp64(nrm2) : 1.0;
+        const double2 f = best > 0.0 && nrm2 > 0.0 ? (rsqrt_fp64(best) * inrm) * conj_(pk) : make_double2(inrm, 0.0);
+        double2 d = czero();
+#pragma unroll
+        for (int t = 0; t < ES; ++t)
+            if (lane + 32 * t < n) {
+                vec[0][t] = f * vec[0][t];
+                d = d + cdot(vec[1][t], vec[0][t]);
+            }
+        d = warp_sum(d);
+        const double2 g = cabs2(d) > 0.0 ? cdiv(cone(), conj_(d)) : cone();
+#pragma unroll
+        for (int t = 0; t < ES; ++t) {
+            const int r = lane + 32 * t;
+            if (r < n) {
+                const int ro = rev ? n - 1 - r : r;
+                Y[ro * ldyz + i] = vec[0][t];
+                Z[ro * ldyz + i] = g * vec[1][t];
+            }
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+}
+
+// Dynamic shared memory of an eigen CTA of capacity nmax. Rows are lda = n | 1
+// slots apart (odd: the lanes of a warp read a column without bank conflicts).
+__host__ __device__ constexpr int eig_lda(int n) { return n | 1; }
+struct EigSmem {
+    double2 *A, *Q, *v, *wb;
+    double* sh;
+    int* ord;
+    __device__ EigSmem(char* base, int nmax) {
+        A = reinterpret_cast<double2*>(base);
+        Q = A + nmax * eig_lda(nmax);
+        v = Q + nmax * eig_lda(nmax);
+        wb = v + nmax;
+        sh = reinterpret_cast<double*>(wb + EW * nmax);
+        ord = reinterpret_cast<int*>(sh + 8);
+    }
+    static size_t bytes(int nmax) {
+        return (size_t)(2 * nmax * eig_lda(nmax) + nmax + EW * nmax) * sizeof(double2) + 8 * sizeof(double) +
+               nmax * sizeof(int) + 16;
+    }
+};
+
+// A window's projected matrix H (leading n x n, row stride ldh) with rows and columns
+// in reverse order: the tridiagonal part first, then the coupling arrow's hub, then
+// the kept Ritz values. In this order the tridiagonal columns are Hessenberg already
+// and only the last block (the arrow) needs reflections; in the original order each
+// reflection's fill-in moves one row down and all n columns need one of the arrow's
+// length (1.4e6 against 0.25e6 cycles in FP64 at n = 60).
+__device__ void load_reversed(const double2* H, int ldh, int n, double2* A) {
+    for (int e = threadIdx.x; e < n * n; e += ET) A[(n - 1 - e / n) * eig_lda(n) + n - 1 - e % n] = H[(e / n) * ldh + e % n];
+    __syncthreads();
+}
+
+// Full eigen-solve of the n x n matrix in S.A (row stride eig_lda(n); rev: in reverse
+// order). Outputs sorted eigenvalues to lam (n), and vectors for the first nsel.
+template <class M>
+__device__ int eig_block(EigSmem& S, int n, int nsel, double2* lam, double2* Y, double2* Z, int ldyz, bool rev = false) {
+    const int lda = eig_lda(n);
+    const int fail = schur<M>(S.A, S.Q, n, lda, S.v, S.sh);
+    const double anorm = S.sh[4];
+    order_eigs(S.A, n, lda, S.ord, S.v);
+    for (int i = threadIdx.x; i < n; i += ET) lam[i] = S.A[S.ord[i] * lda + S.ord[i]];
+    __syncthreads();
+    if (nsel > 0) eigvecs(S.A, S.Q, n, lda, S.ord, nsel, Y, Z, ldyz, S.wb, anorm, rev);
+    return fail;
+}
+
 __global__ void __launch_bounds__(ET) small_eig_kernel(int n, const double2* Ain, int lda_in, int nsel,
-                                                       double2* lam, double2* Y, double2* Z, int ldyz,
-                                                       double2* W, int* info) {
+                                                       double2* lam, double2* Y, double2* Z, int ldyz, int* info) {
     extern __shared__ __align__(16) char smem[];
     EigSmem S(smem, n);
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) S.A[e] = Ain[(e / n) * lda_in + (e % n)];
+    for (int e = threadIdx.x; e < n * n; e += ET) S.A[(e / n) * eig_lda(n) + e % n] = Ain[(e / n) * lda_in + (e % n)];
     __syncthreads();
-    int fail = eig_block(S.A, S.Q, n, n, nsel, lam, Y, Z, ldyz, W, W + (size_t)n * max(nsel, 1), S.v, S.sh, S.ord);
+    const int fail = eig_block<NumD>(S, n, nsel, lam, Y, Z, ldyz);
     if (threadIdx.x == 0 && info) *info = fail;
+}
+
+// LU with complete pivoting of the n x n matrix a (row stride ld), one warp.
+// Stops before a pivot p that keep(|p|^2, i) rejects (i = its index); returns the
+// pivots kept; rowp / colp: the row and column order. The pivot search reads an
+// element per lane; ties go to the first in row-major order.
+template <class Keep>
+__device__ int warp_lu_complete(double2* a, int n, int ld, int* rowp, int* colp, Keep keep) {
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < n; i += 32) { rowp[i] = i; colp[i] = i; }
+    __syncwarp();
+    int i = 0;
+    for (; i < n; ++i) {
+        const int w = n - i;
+        double best = -1.0;
+        int arg = 0;
+        for (int e = lane; e < w * w; e += 32) {
+            const double v = cabs2(a[(i + e / w) * ld + i + e % w]);
+            if (v > best) { best = v; arg = e; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double ob = __shfl_xor_sync(FULL, best, o);
+            const int oa = __shfl_xor_sync(FULL, arg, o);
+            if (ob > best || (ob == best && oa < arg)) { best = ob; arg = oa; }
+        }
+        if (!keep(best, i)) break;
+        const int p = i + arg / w, q = i + arg % w;
+        if (p != i) {
+            for (int c = lane; c < n; c += 32) { const double2 t = a[i * ld + c]; a[i * ld + c] = a[p * ld + c]; a[p * ld + c] = t; }
+            if (lane == 0) { const int t = rowp[i]; rowp[i] = rowp[p]; rowp[p] = t; }
+        }
+        __syncwarp();
+        if (q != i) {
+            for (int r = lane; r < n; r += 32) { const double2 t = a[r * ld + i]; a[r * ld + i] = a[r * ld + q]; a[r * ld + q] = t; }
+            if (lane == 0) { const int t = colp[i]; colp[i] = colp[q]; colp[q] = t; }
+        }
+        __syncwarp();
+        const double2 piv = a[i * ld + i];
+        for (int r = i + 1 + lane; r < n; r += 32) a[r * ld + i] = cdiv(a[r * ld + i], piv);
+        __syncwarp();
+        const int u = w - 1;
+        for (int e = lane; e < u * u; e += 32) {
+            const int r = i + 1 + e / u, c = i + 1 + e % u;
+            a[r * ld + c] = NumD::fms(a[r * ld + c], a[r * ld + i], a[i * ld + c]);
+        }
+        __syncwarp();
+    }
+    return i;
 }
 
 // ------------------------------------------------------- BiCG-eigen (coeffs)
 // Work arrays (global, per problem) for the restart coefficient computation.
 struct RestartWork {
-    double2 *y1, *z1, *y2, *z2, *HY, *T, *u, *q, *W1, *W2, *lamtmp, *lamtmp2, *M;
-    int *rowp, *colp;
+    double2 *y1, *z1, *y2, *z2, *HY, *u, *q, *yt, *zt, *lamtmp, *lamtmp2;
     static size_t elems(int m, int nev) {
         const int r = 2 * nev;
-        return (size_t)m * nev * 4 + (size_t)m * r + (size_t)r * r * 3 + (size_t)m * m * 2 + 2 * m + (size_t)nev * nev + 64;
+        return (size_t)m * nev * 4 + (size_t)m * r * 3 + (size_t)r * r * 2 + 2 * m + 64;
     }
     __device__ RestartWork(double2* base, int m, int nev) {
         const int r = 2 * nev;
         y1 = base; z1 = y1 + m * nev; y2 = z1 + m * nev; z2 = y2 + m * nev;
-        HY = z2 + m * nev; T = HY + m * r; u = T + r * r; q = u + r * r;
-        W1 = q + r * r; W2 = W1 + m * m; lamtmp = W2 + m * m; lamtmp2 = lamtmp + m; M = lamtmp2 + m;
-        rowp = reinterpret_cast<int*>(M + nev * nev);
-        colp = rowp + 32;
+        HY = z2 + m * nev; u = HY + m * r; q = u + r * r;
+        yt = q + r * r; zt = yt + m * r; lamtmp = zt + m * r; lamtmp2 = lamtmp + m;
     }
 };
 
 // Algorithm BiCG-eigen in coefficient space, first part: which = 0 computes
 // eig(H^(m)) -> y1, z1 (nev smallest); which = 1 computes eig(H^(m-1)) -> y2, z2,
-// padded with a zero row. The two parts use disjoint scratch, so two CTAs can
-// run them at the same time.
+// padded with a zero row. The two parts use disjoint work arrays: the two CTAs
+// of a cluster run them at the same time.
 __device__ int restart_eigs_part(const double2* H, int ldh, int m, int nev, int which, EigSmem& S,
                                  RestartWork& Wk) {
     const int tid = threadIdx.x;
     const int n = which ? m - 1 : m;
-    for (int e = tid; e < n * n; e += blockDim.x) S.A[e] = H[(e / n) * ldh + (e % n)];
-    __syncthreads();
-    double2* scratch = which ? Wk.W2 : Wk.W1;   // 2 n nev <= m^2
-    int fail = eig_block(S.A, S.Q, n, n, nev, which ? Wk.lamtmp2 : Wk.lamtmp, which ? Wk.y2 : Wk.y1,
-                         which ? Wk.z2 : Wk.z1, nev, scratch, scratch + (size_t)n * nev, S.v, S.sh, S.ord, true);
+    load_reversed(H, ldh, n, S.A);
+    const int fail = eig_block<NumF>(S, n, nev, which ? Wk.lamtmp2 : Wk.lamtmp, which ? Wk.y2 : Wk.y1,
+                                     which ? Wk.z2 : Wk.z1, nev, true);
     if (which)
-        for (int i = tid; i < nev; i += blockDim.x) { Wk.y2[(m - 1) * nev + i] = czero(); Wk.z2[(m - 1) * nev + i] = czero(); }
+        for (int i = tid; i < nev; i += ET) { Wk.y2[(m - 1) * nev + i] = czero(); Wk.z2[(m - 1) * nev + i] = czero(); }
     __syncthreads();
     return fail;
 }
 
 // Second part: bi-orthogonalize, T = zt^H H yt, eig(T), Yc = yt u, Zc = zt q.
-// Writes Yc, Zc (m x r, ld = ldc), lam (r); returns r.
+// Writes Yc, Zc (m x r, ld = ldc), lam (r); returns r. FP64 throughout.
 __device__ int restart_finish_part(const double2* H, int ldh, int m, int nev, double2* Yc, double2* Zc, int ldc,
                                    double2* lam, EigSmem& S, RestartWork& Wk, int* fail_out) {
     const int tid = threadIdx.x;
-    int fail = 0;
     // 3. y2 -= y1 (z1^H y2), z2 -= z1 (y1^H z2)   (coefficients in S.A as scratch)
     double2* G1 = S.A;                 // nev x nev : z1^H y2
     double2* G2 = S.A + nev * nev;     // nev x nev : y1^H z2
-    for (int e = tid; e < 2 * nev * nev; e += blockDim.x) {
+    double2* Mx = G2 + nev * nev;      // nev x nev : z2^H y2 (3 nev^2 < m^2 slots in all)
+    int* rowp = reinterpret_cast<int*>(S.v);
+    int* colp = rowp + MAX_M / 2;
+    for (int e = tid; e < 2 * nev * nev; e += ET) {
         const bool second = e >= nev * nev;
         const int ee = second ? e - nev * nev : e;
         const int i = ee / nev, j = ee % nev;
@@ -637,7 +850,7 @@ __device__ int restart_finish_part(const double2* H, int ldh, int m, int nev, do
         (second ? G2 : G1)[i * nev + j] = acc;
     }
     __syncthreads();
-    for (int e = tid; e < 2 * m * nev; e += blockDim.x) {
+    for (int e = tid; e < 2 * m * nev; e += ET) {
         const bool second = e >= m * nev;
         const int ee = second ? e - m * nev : e;
         const int r = ee / nev, j = ee % nev;
@@ -649,91 +862,71 @@ __device__ int restart_finish_part(const double2* H, int ldh, int m, int nev, do
         X[r * nev + j] = X[r * nev + j] - acc;
     }
     __syncthreads();
-    // 4. M = z2^H y2, LU with complete pivoting (thread 0), rank by pivot >= 1e-10
-    for (int e = tid; e < nev * nev; e += blockDim.x) {
+    // 4. M = z2^H y2, LU with complete pivoting, rank by pivot >= 1e-10
+    for (int e = tid; e < nev * nev; e += ET) {
         const int i = e / nev, j = e % nev;
         double2 acc = czero();
         for (int r = 0; r < m; ++r) acc = acc + cdot(Wk.z2[r * nev + i], Wk.y2[r * nev + j]);
-        Wk.M[i * nev + j] = acc;
+        Mx[i * nev + j] = acc;
     }
     __syncthreads();
     __shared__ int s_rank;
-    if (tid == 0) {
-        double2* a = Wk.M;
-        int rank = 0;
-        for (int i = 0; i < nev; ++i) { Wk.rowp[i] = i; Wk.colp[i] = i; }
-        for (int i = 0; i < nev; ++i) {
-            double best = -1.0; int pr = i, pc = i;
-            for (int r = i; r < nev; ++r)
-                for (int c = i; c < nev; ++c) {
-                    double v = cabs2(a[r * nev + c]);
-                    if (v > best) { best = v; pr = r; pc = c; }
-                }
-            if (best < 1e-20) break;   // |pivot| < 1e-10
-            if (pr != i) {
-                for (int c = 0; c < nev; ++c) { double2 t = a[i * nev + c]; a[i * nev + c] = a[pr * nev + c]; a[pr * nev + c] = t; }
-                int t = Wk.rowp[i]; Wk.rowp[i] = Wk.rowp[pr]; Wk.rowp[pr] = t;
-            }
-            if (pc != i) {
-                for (int r = 0; r < nev; ++r) { double2 t = a[r * nev + i]; a[r * nev + i] = a[r * nev + pc]; a[r * nev + pc] = t; }
-                int t = Wk.colp[i]; Wk.colp[i] = Wk.colp[pc]; Wk.colp[pc] = t;
-            }
-            for (int r = i + 1; r < nev; ++r) a[r * nev + i] = cdiv(a[r * nev + i], a[i * nev + i]);
-            for (int r = i + 1; r < nev; ++r)
-                for (int c = i + 1; c < nev; ++c) a[r * nev + c] = a[r * nev + c] - a[r * nev + i] * a[i * nev + c];
-            ++rank;
-        }
-        s_rank = rank;
+    if (tid < 32) {
+        const int rank = warp_lu_complete(Mx, nev, nev, rowp, colp, [](double p2, int) { return p2 >= 1e-20; });
+        if (tid == 0) s_rank = rank;
     }
     __syncthreads();
     const int rank = s_rank;
     const int r = nev + rank;
-    // 5. yt = [y1, y2(:,colp) U^{-1}], zt = [z1, z2(:,rowp) L^{-H}]  (in HY/W1 as m x r arrays)
-    double2* yt = Wk.W1;   // m x r (ld r)
-    double2* zt = Wk.W2;
-    for (int e = tid; e < m * nev; e += blockDim.x) {
+    // 5. yt = [y1, y2(:,colp) U^{-1}], zt = [z1, z2(:,rowp) L^{-H}]  (m x r)
+    for (int e = tid; e < m * nev; e += ET) {
         const int row = e / nev, i = e % nev;
-        yt[row * r + i] = Wk.y1[row * nev + i];
-        zt[row * r + i] = Wk.z1[row * nev + i];
+        Wk.yt[row * r + i] = Wk.y1[row * nev + i];
+        Wk.zt[row * r + i] = Wk.z1[row * nev + i];
     }
-    for (int row = tid; row < 2 * m; row += blockDim.x) {
+    for (int j = tid; j < rank; j += ET) G1[j] = cdiv(cone(), Mx[j * nev + j]);   // 1 / U_jj
+    __syncthreads();
+    for (int row = tid; row < 2 * m; row += ET) {
         const bool zs = row >= m;
         const int rr = zs ? row - m : row;
-        double2* out = (zs ? zt : yt) + rr * r + nev;
+        double2* out = (zs ? Wk.zt : Wk.yt) + rr * r + nev;
         const double2* in = (zs ? Wk.z2 : Wk.y2) + rr * nev;
         for (int j = 0; j < rank; ++j) {
-            double2 acc = in[zs ? Wk.rowp[j] : Wk.colp[j]];
+            double2 acc = in[zs ? rowp[j] : colp[j]];
             for (int i = 0; i < j; ++i) {
-                if (!zs) acc = acc - out[i] * Wk.M[i * nev + j];            // U_{ij}
-                else acc = acc - out[i] * conj_(Wk.M[j * nev + i]);         // conj(L_{ji})
+                if (!zs) acc = acc - out[i] * Mx[i * nev + j];            // U_{ij}
+                else acc = acc - out[i] * conj_(Mx[j * nev + i]);         // conj(L_{ji})
             }
-            out[j] = zs ? acc : cdiv(acc, Wk.M[j * nev + j]);
+            out[j] = zs ? acc : acc * G1[j];
         }
     }
     __syncthreads();
-    // 6. T = zt^H H yt (r x r)
-    for (int e = tid; e < m * r; e += blockDim.x) {
+    // 6. T = zt^H H yt (r x r). H has four or five nonzeros per row but for the arrow's: skip the zeros.
+    for (int e = tid; e < m * r; e += ET) {
         const int row = e / r, j = e % r;
         double2 acc = czero();
-        for (int l = 0; l < m; ++l) acc = acc + H[row * ldh + l] * yt[l * r + j];
+        for (int l = 0; l < m; ++l) {
+            const double2 h = H[row * ldh + l];
+            if (h.x != 0.0 || h.y != 0.0) acc = acc + h * Wk.yt[l * r + j];
+        }
         Wk.HY[row * r + j] = acc;
     }
     __syncthreads();
-    for (int e = tid; e < r * r; e += blockDim.x) {
+    for (int e = tid; e < r * r; e += ET) {
         const int i = e / r, j = e % r;
         double2 acc = czero();
-        for (int l = 0; l < m; ++l) acc = acc + cdot(zt[l * r + i], Wk.HY[l * r + j]);
-        S.A[e] = acc;
+        for (int l = 0; l < m; ++l) acc = acc + cdot(Wk.zt[l * r + i], Wk.HY[l * r + j]);
+        S.A[i * eig_lda(r) + j] = acc;
     }
     __syncthreads();
     // 7. eig(T): all r pairs -> u, q, lam
-    fail |= eig_block(S.A, S.Q, r, r, r, lam, Wk.u, Wk.q, r, Wk.T, Wk.HY, S.v, S.sh, S.ord);
+    const int fail = eig_block<NumD>(S, r, r, lam, Wk.u, Wk.q, r);
     // 8. Yc = yt u, Zc = zt q
-    for (int e = tid; e < 2 * m * r; e += blockDim.x) {
+    for (int e = tid; e < 2 * m * r; e += ET) {
         const bool zs = e >= m * r;
         const int ee = zs ? e - m * r : e;
         const int row = ee / r, j = ee % r;
-        const double2* X = zs ? zt : yt;
+        const double2* X = zs ? Wk.zt : Wk.yt;
         const double2* C = zs ? Wk.q : Wk.u;
         double2 acc = czero();
         for (int l = 0; l < r; ++l) acc = acc + X[row * r + l] * C[l * r + j];
@@ -744,56 +937,65 @@ __device__ int restart_finish_part(const double2* H, int ldh, int m, int nev, do
     return r;
 }
 
-__global__ void __launch_bounds__(ET) restart_single_kernel(int m, int nev, const double2* H, int* r_out,
-                                                            double2* Yc, double2* Zc, double2* lam,
-                                                            double2* work, int* info) {
+// Both CTAs of a two-CTA cluster arrive and wait (release / acquire: global writes
+// before it are visible after it in the other CTA).
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// One restart's coefficients by the two CTAs of a cluster: each eigen-solve on its
+// own SM, then CTA 0 finishes. fails: two words. Returns r in CTA 0 (fail in *fail),
+// -1 in CTA 1.
+__device__ int restart_cluster(const double2* H, int ldh, int m, int nev, double2* Yc, double2* Zc, int ldc,
+                               double2* lam, EigSmem& S, RestartWork& Wk, int* fails, int* fail) {
+    const int which = blockIdx.x & 1;
+    const int f = restart_eigs_part(H, ldh, m, nev, which, S, Wk);
+    if (threadIdx.x == 0) fails[which] = f;
+    __syncthreads();
+    cluster_sync();
+    if (which) return -1;
+    int f2 = 0;
+    const int r = restart_finish_part(H, ldh, m, nev, Yc, Zc, ldc, lam, S, Wk, &f2);
+    *fail = f2 | __ldcg(fails) | __ldcg(fails + 1);
+    return r;
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ET)
+    restart_single_kernel(int m, int nev, const double2* H, int* r_out, double2* Yc, double2* Zc, double2* lam,
+                          double2* work, int* fails, int* info) {
     extern __shared__ __align__(16) char smem[];
     EigSmem S(smem, m);
     RestartWork Wk(work, m, nev);
-    int fail = restart_eigs_part(H, m, m, nev, 0, S, Wk);
-    fail |= restart_eigs_part(H, m, m, nev, 1, S, Wk);
-    int f2 = 0;
-    int r = restart_finish_part(H, m, m, nev, Yc, Zc, 2 * nev, lam, S, Wk, &f2);
-    if (threadIdx.x == 0) { *r_out = r; *info = fail | f2; }
+    int fail = 0;
+    const int r = restart_cluster(H, m, m, nev, Yc, Zc, 2 * nev, lam, S, Wk, fails, &fail);
+    if (r >= 0 && threadIdx.x == 0) { *r_out = r; *info = fail; }
 }
 
-// Restart of every slot whose window is full (vs == m), in two kernels: the two
-// eigen-solves (one CTA each, grid (nslots, 2)), then the rest (one CTA per
-// slot): coefficients and H = diag(lam).
-__global__ void __launch_bounds__(ET) restart_eigs_kernel(SlotState* states, const SlotPtrs* ptrs,
-                                                          double2* work_base, size_t work_stride, int* fails) {
-    const SlotState& st = states[blockIdx.x];
-    const SlotPtrs& P = ptrs[blockIdx.x];
-    if (!(st.status == ST_RUNNING && st.m > 0 && st.vs == st.m)) return;
-    extern __shared__ __align__(16) char smem[];
-    const int m = st.m, nev = st.nev;
-    EigSmem S(smem, m);
-    RestartWork Wk(work_base + work_stride * blockIdx.x, m, nev);
-    int fail = restart_eigs_part(P.H, m, m, nev, blockIdx.y, S, Wk);
-    if (threadIdx.x == 0) fails[2 * blockIdx.x + blockIdx.y] = fail;
-}
-
-__global__ void __launch_bounds__(ET) restart_slots_kernel(SlotState* states, const SlotPtrs* ptrs,
-                                                           double2* work_base, size_t work_stride, const int* fails) {
-    SlotState& st = states[blockIdx.x];
-    const SlotPtrs& P = ptrs[blockIdx.x];
+// Restart of every slot whose window is full (vs == m), one cluster per slot (grid
+// 2 nslots): the two eigen-solves, the coefficients and H = diag(lam). The other
+// slots' clusters return at once (uniform over the cluster: CTA 0 writes the
+// slot's state only after the cluster barrier).
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ET)
+    restart_slots_kernel(SlotState* states, const SlotPtrs* ptrs, double2* work_base, size_t work_stride, int* fails) {
+    const int slot = blockIdx.x >> 1;
+    SlotState& st = states[slot];
+    const SlotPtrs& P = ptrs[slot];
     __shared__ int go;
     if (threadIdx.x == 0) {
         go = (st.status == ST_RUNNING && st.m > 0 && st.vs == st.m);
-        if (!go) st.restart_r = 0;
+        if (!go && (blockIdx.x & 1) == 0) st.restart_r = 0;
     }
     __syncthreads();
     if (!go) return;
     extern __shared__ __align__(16) char smem[];
     const int m = st.m, nev = st.nev;
     EigSmem S(smem, m);
-    RestartWork Wk(work_base + work_stride * blockIdx.x, m, nev);
-    const int ldc = 2 * nev + 1;
+    RestartWork Wk(work_base + work_stride * slot, m, nev);
     int fail = 0;
-    int r = restart_finish_part(P.H, m, m, nev, P.coefY, P.coefZ, ldc, P.lam, S, Wk, &fail);
-    fail |= fails[2 * blockIdx.x] | fails[2 * blockIdx.x + 1];
+    const int r = restart_cluster(P.H, m, m, nev, P.coefY, P.coefZ, 2 * nev + 1, P.lam, S, Wk, fails + 2 * slot, &fail);
+    if (r < 0) return;
     // H = diag(lam)
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+    for (int e = threadIdx.x; e < m * m; e += ET) {
         const int i = e / m, j = e % m;
         P.H[e] = (i == j && i < r) ? P.lam[i] : czero();
     }
@@ -808,18 +1010,16 @@ __global__ void __launch_bounds__(ET) restart_slots_kernel(SlotState* states, co
 
 // Final Ritz pairs of a window: eig(H^(vs)), nev smallest, scales folded.
 // Block j: slot slot0 + j, outputs at Yc + j ostride, Zc + j ostride, lam + j lstride,
-// nout[j], work area work + j wstride (the windows' final Ritz pairs of several
-// slots at once: each depends only on its own window).
+// nout[j] (the windows' final Ritz pairs of several slots at once: each depends
+// only on its own window).
 __global__ void __launch_bounds__(ET) final_ritz_kernel(SlotState* states, const SlotPtrs* ptrs, int slot0,
                                                         double2* Yc, double2* Zc, double2* lam, int* nout,
-                                                        double2* work, size_t ostride, size_t lstride,
-                                                        size_t wstride) {
+                                                        size_t ostride, size_t lstride) {
     const int slot = slot0 + blockIdx.x;
     Yc += blockIdx.x * ostride;
     Zc += blockIdx.x * ostride;
     lam += blockIdx.x * lstride;
     nout += blockIdx.x;
-    work += blockIdx.x * wstride;
     const SlotState& st = states[slot];
     const SlotPtrs& P = ptrs[slot];
     const int n = st.vs, m = st.m;
@@ -827,10 +1027,9 @@ __global__ void __launch_bounds__(ET) final_ritz_kernel(SlotState* states, const
     if (n == 0) { if (threadIdx.x == 0) *nout = 0; return; }
     extern __shared__ __align__(16) char smem[];
     EigSmem S(smem, n);
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) S.A[e] = P.H[(e / n) * m + (e % n)];
-    __syncthreads();
-    eig_block(S.A, S.Q, n, n, nsel, lam, Yc, Zc, nsel, work, work + (size_t)n * nsel, S.v, S.sh, S.ord);
-    for (int e = threadIdx.x; e < n * nsel; e += blockDim.x) {
+    load_reversed(P.H, m, n, S.A);
+    eig_block<NumD>(S, n, nsel, lam, Yc, Zc, nsel, true);
+    for (int e = threadIdx.x; e < n * nsel; e += ET) {
         const int row = e / nsel;
         Yc[e] = P.vscale[row] * Yc[e];
         Zc[e] = P.wscale[row] * Zc[e];
@@ -838,77 +1037,146 @@ __global__ void __launch_bounds__(ET) final_ritz_kernel(SlotState* states, const
     if (threadIdx.x == 0) *nout = nsel;
 }
 
-// LU with partial pivoting, one CTA.
-__global__ void lu_factor_kernel(int n, double2* A, int lda, int* piv, int* info) {
-    __shared__ int s_p;
-    __shared__ int s_bad;
-    if (threadIdx.x == 0) s_bad = 0;
+// 1/d of a pivot: conj(d) / |d|^2 where the square stays inside FP32's normal
+// range, Smith's division otherwise.
+__device__ __forceinline__ double2 pivot_rcp(double2 d) {
+    const double m = fmax(fabs(d.x), fabs(d.y));
+    if (m > 1e-14 && m < 1e14) return rcp_fp64(cabs2(d)) * conj_(d);
+    return cdiv(cone(), d);
+}
+
+// LU with partial pivoting, one CTA per matrix (blockIdx.x selects one of two of
+// the same size), in shared memory. Warp 0 searches the pivot column, a row per
+// lane, and forms 1/pivot; the rank-1 updates are bound by FP64 issue.
+struct LuJob {
+    double2* A;
+    int* piv;
+    int* info;
+};
+__global__ void __launch_bounds__(ET) lu_factor_kernel(int n, LuJob j0, LuJob j1, int lda) {
+    const LuJob job = blockIdx.x ? j1 : j0;
+    extern __shared__ __align__(16) char smem[];
+    double2* A = reinterpret_cast<double2*>(smem);
+    const int ld = eig_lda(n), tid = threadIdx.x, lane = tid & 31;
+    __shared__ int s_p, s_bad;
+    __shared__ double2 s_inv;
+    for (int e = tid; e < n * n; e += ET) A[(e / n) * ld + e % n] = job.A[(size_t)(e / n) * lda + e % n];
+    if (tid == 0) s_bad = 0;
     __syncthreads();
     for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
-            int p = k; double best = -1.0;
-            for (int i = k; i < n; ++i) { double v = cabs2(A[i * lda + k]); if (v > best) { best = v; p = i; } }
-            s_p = p; piv[k] = p;
-            if (best == 0.0) s_bad = 1;
+        if (tid < 32) {
+            double best = -1.0;
+            int p = k;
+            for (int i = k + lane; i < n; i += 32) {
+                const double v = cabs2(A[i * ld + k]);
+                if (v > best) { best = v; p = i; }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ob = __shfl_xor_sync(FULL, best, o);
+                const int op = __shfl_xor_sync(FULL, p, o);
+                if (ob > best || (ob == best && op < p)) { best = ob; p = op; }
+            }
+            const double2 inv = best > 0.0 ? pivot_rcp(A[p * ld + k]) : czero();
+            if (lane == 0) {
+                s_p = p;
+                job.piv[k] = p;
+                s_inv = inv;
+                if (!(best > 0.0)) s_bad = 1;
+            }
         }
         __syncthreads();
         const int p = s_p;
+        const double2 inv = s_inv;
         if (p != k)
-            for (int j = threadIdx.x; j < n; j += blockDim.x) {
-                double2 t = A[k * lda + j]; A[k * lda + j] = A[p * lda + j]; A[p * lda + j] = t;
-            }
+            for (int j = tid; j < n; j += ET) { const double2 t = A[k * ld + j]; A[k * ld + j] = A[p * ld + j]; A[p * ld + j] = t; }
         __syncthreads();
-        const double2 d = A[k * lda + k];
-        if (cabs2(d) > 0.0)
-            for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) A[i * lda + k] = cdiv(A[i * lda + k], d);
+        if (inv.x != 0.0 || inv.y != 0.0)
+            for (int i = k + 1 + tid; i < n; i += ET) A[i * ld + k] = A[i * ld + k] * inv;
         __syncthreads();
-        for (int e = threadIdx.x; e < (n - k - 1) * (n - k - 1); e += blockDim.x) {
-            const int i = k + 1 + e / (n - k - 1), j = k + 1 + e % (n - k - 1);
-            A[i * lda + j] = A[i * lda + j] - A[i * lda + k] * A[k * lda + j];
+        const int w = n - k - 1;
+        for (int e = tid; e < w * w; e += ET) {
+            const int i = k + 1 + e / w, j = k + 1 + e % w;
+            A[i * ld + j] = NumD::fms(A[i * ld + j], A[i * ld + k], A[k * ld + j]);
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0 && info) *info = s_bad;
+    for (int e = tid; e < n * n; e += ET) job.A[(size_t)(e / n) * lda + e % n] = A[(e / n) * ld + e % n];
+    if (tid == 0 && job.info) *job.info = s_bad;
 }
 
-// Solve with the LU factors; one thread per right-hand-side column.
-__global__ void lu_solve_kernel(int n, const double2* LU, int lda, const int* piv, int trans, int nrhs,
-                                double2* B, int ldb) {
-    for (int c = threadIdx.x; c < nrhs; c += blockDim.x) {
-        if (!trans) {
-            for (int k = 0; k < n; ++k) {   // P
-                int p = piv[k];
-                if (p != k) { double2 t = B[k * ldb + c]; B[k * ldb + c] = B[p * ldb + c]; B[p * ldb + c] = t; }
-            }
-            for (int i = 0; i < n; ++i) {   // L y = b
-                double2 acc = B[i * ldb + c];
-                for (int j = 0; j < i; ++j) acc = acc - LU[i * lda + j] * B[j * ldb + c];
-                B[i * ldb + c] = acc;
-            }
-            for (int i = n - 1; i >= 0; --i) {   // U x = y
-                double2 acc = B[i * ldb + c];
-                for (int j = i + 1; j < n; ++j) acc = acc - LU[i * lda + j] * B[j * ldb + c];
-                B[i * ldb + c] = cdiv(acc, LU[i * lda + i]);
-            }
-        } else {
-            // A^H x = b with P A = L U:  A^H = U^H L^H P  ->  U^H y = b, L^H w = y, x = P^T w
-            for (int i = 0; i < n; ++i) {
-                double2 acc = B[i * ldb + c];
-                for (int j = 0; j < i; ++j) acc = acc - conj_(LU[j * lda + i]) * B[j * ldb + c];
-                B[i * ldb + c] = cdiv(acc, conj_(LU[i * lda + i]));
-            }
-            for (int i = n - 1; i >= 0; --i) {
-                double2 acc = B[i * ldb + c];
-                for (int j = i + 1; j < n; ++j) acc = acc - conj_(LU[j * lda + i]) * B[j * ldb + c];
-                B[i * ldb + c] = acc;
-            }
-            for (int k = n - 1; k >= 0; --k) {
-                int p = piv[k];
-                if (p != k) { double2 t = B[k * ldb + c]; B[k * ldb + c] = B[p * ldb + c]; B[p * ldb + c] = t; }
+// Solve with the LU factors: one warp per right-hand-side column, LS columns per
+// CTA, the factors in shared memory. Outer-product substitution: a step is one
+// broadcast and one complex multiply-add per lane instead of a serial row sum.
+constexpr int LS = 4;
+__global__ void __launch_bounds__(32 * LS) lu_solve_kernel(int n, const double2* LU, int lda, const int* piv, int trans,
+                                                          int nrhs, double2* B, int ldb) {
+    extern __shared__ __align__(16) char smem[];
+    double2* F = reinterpret_cast<double2*>(smem);
+    const int ld = eig_lda(n), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double2* x = F + n * ld + warp * n;
+    int* pv = reinterpret_cast<int*>(F + n * ld + LS * n);
+    for (int e = tid; e < n * n; e += 32 * LS) F[(e / n) * ld + e % n] = LU[(size_t)(e / n) * lda + e % n];
+    for (int e = tid; e < n; e += 32 * LS) pv[e] = piv[e];
+    __syncthreads();
+    const int c = blockIdx.x * LS + warp;
+    if (c >= nrhs) return;
+    for (int i = lane; i < n; i += 32) x[i] = B[(size_t)i * ldb + c];
+    __syncwarp();
+    if (!trans && lane == 0)   // P b
+        for (int k = 0; k < n; ++k) {
+            const int p = pv[k];
+            if (p != k) { const double2 t = x[k]; x[k] = x[p]; x[p] = t; }
+        }
+    __syncwarp();
+    double2 s[ES], dinv[ES];
+#pragma unroll
+    for (int t = 0; t < ES; ++t) {
+        const int j = lane + 32 * t;
+        s[t] = dinv[t] = czero();
+        if (j < n) {
+            s[t] = x[j];
+            const double2 d = pivot_rcp(F[j * ld + j]);
+            dinv[t] = trans ? conj_(d) : d;
+        }
+    }
+    // not transposed: L y = b (unit), then U x = y; transposed (A^H = U^H L^H P):
+    // U^H y = b, then L^H w = y (unit), x = P^T w
+#pragma unroll
+    for (int pass = 0; pass < 2; ++pass) {
+        const bool divide = trans ? pass == 0 : pass == 1;
+        for (int q = 0; q < n; ++q) {
+            const int l = pass == 0 ? q : n - 1 - q;
+            const int own = l >> 5;
+            double2 v = s[0], dv = dinv[0];
+#pragma unroll
+            for (int t = 1; t < ES; ++t)
+                if (own == t) { v = s[t]; dv = dinv[t]; }
+            if (divide) v = v * dv;
+            const double2 w = shfl_c(v, l & 31);
+#pragma unroll
+            for (int t = 0; t < ES; ++t) {
+                const int j = lane + 32 * t;
+                if (j == l) s[t] = w;
+                if (32 * t < n && (pass == 0 ? (j > l && j < n) : j < l))
+                    s[t] = NumD::fms(s[t], trans ? conj_(F[l * ld + j]) : F[j * ld + l], w);
             }
         }
     }
+#pragma unroll
+    for (int t = 0; t < ES; ++t)
+        if (lane + 32 * t < n) x[lane + 32 * t] = s[t];
+    __syncwarp();
+    if (trans && lane == 0)   // P^T w
+        for (int k = n - 1; k >= 0; --k) {
+            const int p = pv[k];
+            if (p != k) { const double2 t = x[k]; x[k] = x[p]; x[p] = t; }
+        }
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) B[(size_t)i * ldb + c] = x[i];
 }
+size_t lu_factor_smem(int n) { return (size_t)n * eig_lda(n) * sizeof(double2); }
+size_t lu_solve_smem(int n) { return (size_t)(n * eig_lda(n) + LS * n) * sizeof(double2) + n * sizeof(int); }
 
 // One factor of P A = L U applied to B (n x nrhs, or nrows x n for LU_RIGHT_U),
 // one thread per column (per row for LU_RIGHT_U):
@@ -957,57 +1225,19 @@ __global__ void lu_part_kernel(int n, const double2* LU, int lda, const int* piv
 // Rank-revealing selection on a small square block B (n <= 32, row-major, ld):
 // LU with complete pivoting on a copy, stopped at the first pivot below
 // tau * |first pivot|. out[0] = r (pivots kept), out[1 + i] = row index of pivot
-// i, out[1 + n + i] = its column index (i < r). One thread.
-__global__ void pivot_select_kernel(int n, const double2* B, int ld, double tau, int* out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double2 a[32][32];
-    int rows[32], cols[32];
-    for (int i = 0; i < n; ++i) {
-        rows[i] = cols[i] = i;
-        for (int j = 0; j < n; ++j) a[i][j] = B[i * ld + j];
-    }
-    double p0 = 0.0;
-    int r = 0;
-    for (int k = 0; k < n; ++k) {
-        int pi = k, pj = k;
-        double best = -1.0;
-        for (int i = k; i < n; ++i)
-            for (int j = k; j < n; ++j) {
-                const double v = cabs2(a[i][j]);
-                if (v > best) { best = v; pi = i; pj = j; }
-            }
-        best = sqrt(best);
-        if (k == 0) p0 = best;
-        if (!(best > tau * p0) || best == 0.0) break;
-        if (pi != k) {
-            for (int j = 0; j < n; ++j) { double2 t = a[k][j]; a[k][j] = a[pi][j]; a[pi][j] = t; }
-            int t = rows[k]; rows[k] = rows[pi]; rows[pi] = t;
-        }
-        if (pj != k) {
-            for (int i = 0; i < n; ++i) { double2 t = a[i][k]; a[i][k] = a[i][pj]; a[i][pj] = t; }
-            int t = cols[k]; cols[k] = cols[pj]; cols[pj] = t;
-        }
-        for (int i = k + 1; i < n; ++i) {
-            const double2 l = cdiv(a[i][k], a[k][k]);
-            for (int j = k + 1; j < n; ++j) a[i][j] = a[i][j] - l * a[k][j];
-        }
-        r = k + 1;
-    }
-    out[0] = r;
-    for (int i = 0; i < n; ++i) { out[1 + i] = rows[i]; out[1 + n + i] = cols[i]; }
-}
-
-__global__ void small_gemm_kernel(int n, int k, int m, const double2* A, int lda, int transA,
-                                  const double2* B, int ldb, double2* C, int ldc) {
-    for (int e = threadIdx.x + blockIdx.x * blockDim.x; e < n * m; e += blockDim.x * gridDim.x) {
-        const int i = e / m, j = e % m;
-        double2 acc = czero();
-        for (int l = 0; l < k; ++l) {
-            double2 a = transA ? conj_(A[l * lda + i]) : A[i * lda + l];
-            acc = acc + a * B[l * ldb + j];
-        }
-        C[i * ldc + j] = acc;
-    }
+// i, out[1 + n + i] = its column index (i < r). One warp.
+__global__ void __launch_bounds__(32) pivot_select_kernel(int n, const double2* B, int ld, double tau, int* out) {
+    __shared__ double2 a[32 * 33];
+    __shared__ int rowp[32], colp[32];
+    for (int e = threadIdx.x; e < n * n; e += 32) a[(e / n) * 33 + e % n] = B[(size_t)(e / n) * ld + e % n];
+    __syncwarp();
+    double first = 0.0;
+    const int r = warp_lu_complete(a, n, 33, rowp, colp, [&](double p2, int i) {
+        if (i == 0) first = p2;
+        return p2 > tau * tau * first && p2 != 0.0;
+    });
+    if (threadIdx.x == 0) out[0] = r;
+    for (int i = threadIdx.x; i < n; i += 32) { out[1 + i] = rowp[i]; out[1 + n + i] = colp[i]; }
 }
 
 }  // namespace
@@ -1023,18 +1253,17 @@ cudaError_t prepare_eig_kernels() {
     if ((e = set_smem((const void*)small_eig_kernel, EigSmem::bytes(MAX_SMALL))) != cudaSuccess) return e;
     if ((e = set_smem((const void*)restart_single_kernel, EigSmem::bytes(MAX_M))) != cudaSuccess) return e;
     if ((e = set_smem((const void*)restart_slots_kernel, EigSmem::bytes(MAX_M))) != cudaSuccess) return e;
-    if ((e = set_smem((const void*)restart_eigs_kernel, EigSmem::bytes(MAX_M))) != cudaSuccess) return e;
+    if ((e = set_smem((const void*)lu_factor_kernel, lu_factor_smem(MAX_SMALL))) != cudaSuccess) return e;
+    if ((e = set_smem((const void*)lu_solve_kernel, lu_solve_smem(MAX_SMALL))) != cudaSuccess) return e;
     return set_smem((const void*)final_ritz_kernel, EigSmem::bytes(MAX_M));
 }
 
 size_t eig_work_elems() {
-    size_t a = RestartWork::elems(MAX_M, MAX_M / 2);
-    size_t b = (size_t)2 * MAX_SMALL * MAX_SMALL + 16;
-    return a > b ? a : b;
+    return RestartWork::elems(MAX_M, MAX_M / 2);
 }
 
 cudaError_t launch_small_eig(int n, const double2* A, int lda, int nsel, double2* lam, double2* Y, double2* Z,
-                             int ldyz, int* info, double2* w, cudaStream_t st) {
+                             int ldyz, int* info, cudaStream_t st) {
     if (n < 1 || n > MAX_SMALL) return cudaErrorInvalidValue;
     // The kernel's shared-memory limit is only ever set to the largest size
     // (bytes(MAX_SMALL)); a smaller per-call value would lower it for every
@@ -1042,7 +1271,7 @@ cudaError_t launch_small_eig(int n, const double2* A, int lda, int nsel, double2
     cudaError_t e = set_smem((const void*)small_eig_kernel, EigSmem::bytes(MAX_SMALL));
     if (e != cudaSuccess) return e;
     const size_t sm = EigSmem::bytes(n);
-    small_eig_kernel<<<1, ET, sm, st>>>(n, A, lda, nsel, lam, Y, Z, ldyz, w, info);
+    small_eig_kernel<<<1, ET, sm, st>>>(n, A, lda, nsel, lam, Y, Z, ldyz, info);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1053,7 +1282,8 @@ cudaError_t launch_restart_coeffs_single(int m, int nev, const double2* H, int* 
     const size_t sm = EigSmem::bytes(m);
     cudaError_t e = set_smem((const void*)restart_single_kernel, EigSmem::bytes(MAX_M));   // never lowered
     if (e != cudaSuccess) return e;
-    restart_single_kernel<<<1, ET, sm, st>>>(m, nev, H, r, Yc, Zc, lam, w, info);
+    int* fails = reinterpret_cast<int*>(w + eig_work_elems() - 4);   // inside the area's slack
+    restart_single_kernel<<<2, ET, sm, st>>>(m, nev, H, r, Yc, Zc, lam, w, fails, info);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1066,37 +1296,33 @@ cudaError_t launch_restart_coeffs(SlotState* states, const SlotPtrs* ptrs, int n
     const size_t stride = eig_work_elems();
     int* fails = reinterpret_cast<int*>(w + stride * MAX_SLOTS);   // 2 ints per slot after the slot work areas
     size_t sm = EigSmem::bytes(MAX_M);
-    restart_eigs_kernel<<<dim3(nslots, 2), ET, sm, st>>>(states, ptrs, w, stride, fails);
-    restart_slots_kernel<<<nslots, ET, sm, st>>>(states, ptrs, w, stride, fails);
-    count_launches(2);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_final_ritz(SlotState* states, const SlotPtrs* ptrs, int slot, double2* Yc, double2* Zc,
-                              double2* lam, int* nout, double2* w, cudaStream_t st) {
-    return launch_final_ritz_slots(states, ptrs, slot, 1, Yc, Zc, lam, nout, 0, 0, w, st);
-}
-
-cudaError_t launch_final_ritz_slots(SlotState* states, const SlotPtrs* ptrs, int slot0, int nslots, double2* Yc,
-                                    double2* Zc, double2* lam, int* nout, size_t ostride, size_t lstride,
-                                    double2* w, cudaStream_t st) {
-    if (nslots < 1 || nslots > MAX_SLOTS) return cudaErrorInvalidValue;
-    size_t sm = EigSmem::bytes(MAX_M);
-    final_ritz_kernel<<<nslots, ET, sm, st>>>(states, ptrs, slot0, Yc, Zc, lam, nout, w, ostride, lstride,
-                                              eig_work_elems());
+    restart_slots_kernel<<<2 * nslots, ET, sm, st>>>(states, ptrs, w, stride, fails);
     count_launches(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_lu_factor(int n, double2* A, int lda, int* piv, int* info, cudaStream_t st) {
-    lu_factor_kernel<<<1, 256, 0, st>>>(n, A, lda, piv, info);
+cudaError_t launch_final_ritz_slots(SlotState* states, const SlotPtrs* ptrs, int slot0, int nslots, double2* Yc,
+                                    double2* Zc, double2* lam, int* nout, size_t ostride, size_t lstride,
+                                    cudaStream_t st) {
+    if (nslots < 1 || nslots > MAX_SLOTS) return cudaErrorInvalidValue;
+    size_t sm = EigSmem::bytes(MAX_M);
+    final_ritz_kernel<<<nslots, ET, sm, st>>>(states, ptrs, slot0, Yc, Zc, lam, nout, ostride, lstride);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_lu_factor(int n, double2* A, int lda, int* piv, int* info, cudaStream_t st, double2* A2,
+                             int* piv2, int* info2) {
+    if (n < 1 || n > MAX_SMALL) return cudaErrorInvalidValue;
+    lu_factor_kernel<<<A2 ? 2 : 1, ET, lu_factor_smem(n), st>>>(n, LuJob{A, piv, info}, LuJob{A2, piv2, info2}, lda);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_lu_solve(int n, const double2* LU, int lda, const int* piv, int trans, int nrhs, double2* B,
                             int ldb, cudaStream_t st) {
-    lu_solve_kernel<<<1, 128, 0, st>>>(n, LU, lda, piv, trans, nrhs, B, ldb);
+    if (n < 1 || n > MAX_SMALL || nrhs < 1) return cudaErrorInvalidValue;
+    lu_solve_kernel<<<(nrhs + LS - 1) / LS, 32 * LS, lu_solve_smem(n), st>>>(n, LU, lda, piv, trans, nrhs, B, ldb);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1115,16 +1341,6 @@ cudaError_t launch_pivot_select(int n, const double2* B, int ld, double tau, int
     return cudaGetLastError();
 }
 
-cudaError_t launch_small_gemm(int n, int k, int m, const double2* A, int lda, int transA, const double2* B,
-                              int ldb, double2* C, int ldc, cudaStream_t st) {
-    int blocks = (n * m + 255) / 256;
-    if (blocks < 1) blocks = 1;
-    small_gemm_kernel<<<blocks, 256, 0, st>>>(n, k, m, A, lda, transA, B, ldb, C, ldc);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-
 // ============================================================================
 // Allocation-free variant of the small eigen-solver (no counterpart in the paper).
 //
@@ -1133,48 +1349,44 @@ cudaError_t launch_small_gemm(int n, int k, int m, const double2* A, int lda, in
 // host applications that hand all device memory to their own pool or fixed
 // budget up front, and latency-critical loops where the implicit device
 // synchronisation of cudaMalloc/cudaFree would stall work on other streams.
-// lqcd_small_eig_noalloc takes device pointers for the input and every output
-// and keeps its scratch (the substitution vectors and a status word) in the
-// file-scope device array below: at most NOALLOC_MAX_N = 80, i.e. 2*80*80 + 16
-// complex doubles (about 200 KiB), held by every GPU that loads the library
-// until the process exits. The array is shared by all calls on a device and
-// keeps the last call's contents: the status word is cleared by each call, the
-// substitution vectors are fully rewritten before they are read. Calls whose
-// kernels overlap on the GPU (different streams, or host threads) race on it.
-// The per-device set-up (the array's address, the shared-memory limit) is kept
+// lqcd_small_eig_noalloc takes device pointers for the input and every output;
+// its working set is the kernel's shared memory, and its status word lives in
+// the file-scope device variable below. The word is shared by all calls on a
+// device and cleared by each: calls whose kernels overlap on the GPU (different
+// streams, or host threads) race on it.
+// The per-device set-up (the word's address, the shared-memory limit) is kept
 // for the life of the process: a cudaDeviceReset between calls is not supported.
 // Every other launcher of the same kernel keeps its shared-memory limit at the
 // maximum, so no other call can lower it below what this entry point needs.
 namespace {
 
 constexpr int NOALLOC_MAX_N = MAX_SMALL;
-constexpr size_t NOALLOC_SCRATCH = (size_t)2 * NOALLOC_MAX_N * NOALLOC_MAX_N;
 
-static __device__ __align__(256) double2 g_noalloc_scratch[NOALLOC_SCRATCH + 16];
+static __device__ int g_noalloc_info;
 
 struct NoAllocSetup {
     bool ready = false;
-    double2* scratch = nullptr;   // device address of g_noalloc_scratch on this device
+    int* info = nullptr;   // device address of g_noalloc_info on this device
 };
 constexpr int NOALLOC_MAX_DEVICES = 64;
 NoAllocSetup g_noalloc_dev[NOALLOC_MAX_DEVICES];
 std::mutex g_noalloc_mutex;
 
-// Once per device, with that device current: the array's device address and the
+// Once per device, with that device current: the word's device address and the
 // kernel's shared-memory opt-in.
-cudaError_t noalloc_setup(int dev, double2** scratch) {
+cudaError_t noalloc_setup(int dev, int** info) {
     std::lock_guard<std::mutex> lock(g_noalloc_mutex);
     NoAllocSetup& d = g_noalloc_dev[dev];
     if (!d.ready) {
         void* p = nullptr;
-        cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+        cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_info);
         if (e != cudaSuccess) return e;
         e = set_smem((const void*)small_eig_kernel, EigSmem::bytes(NOALLOC_MAX_N));
         if (e != cudaSuccess) return e;
-        d.scratch = reinterpret_cast<double2*>(p);
+        d.info = reinterpret_cast<int*>(p);
         d.ready = true;
     }
-    *scratch = d.scratch;
+    *info = d.info;
     return cudaSuccess;
 }
 
@@ -1187,16 +1399,15 @@ extern "C" lqcd_status lqcd_small_eig_noalloc(int n, const double* C, double* ev
     if (n < 1 || n > NOALLOC_MAX_N || !C || !evals || (Y == nullptr) != (Z == nullptr)) return LQCD_ERR_ARG;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= NOALLOC_MAX_DEVICES) return LQCD_ERR_CUDA;
-    double2* scratch = nullptr;
-    if (noalloc_setup(dev, &scratch) != cudaSuccess) return LQCD_ERR_CUDA;
+    int* info = nullptr;
+    if (noalloc_setup(dev, &info) != cudaSuccess) return LQCD_ERR_CUDA;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    int* info = reinterpret_cast<int*>(scratch + NOALLOC_SCRATCH);
     const int nsel = Y ? n : 0;
     if (cudaMemsetAsync(info, 0, sizeof(int), st) != cudaSuccess) return LQCD_ERR_CUDA;
     (void)cudaGetLastError();   // an earlier, unrelated launch error is not this call's
     small_eig_kernel<<<1, ET, EigSmem::bytes(n), st>>>(n, reinterpret_cast<const double2*>(C), n, nsel,
                                                        reinterpret_cast<double2*>(evals), reinterpret_cast<double2*>(Y),
-                                                       reinterpret_cast<double2*>(Z), n, scratch, info);
+                                                       reinterpret_cast<double2*>(Z), n, info);
     count_launches(1);
     if (cudaPeekAtLastError() != cudaSuccess) { (void)cudaGetLastError(); return LQCD_ERR_CUDA; }
     int hinfo = 0;

@@ -155,7 +155,7 @@ cudaError_t launch_bicg_finish(const Geom& g, const void* links64, double kappa,
 
 // eigBiCG restart: coefficient kernel (one CTA per slot) and window product.
 // Work buffers: eig_work_elems() double2 per slot (restart; the buffer holds MAX_SLOTS
-// slot areas plus 16 double2 for status words) or per call (the others).
+// slot areas plus 16 double2 for status words) or per call (launch_restart_coeffs_single).
 size_t eig_work_elems();
 // Opt the eigen kernels into large dynamic shared memory (call once, outside graph capture).
 cudaError_t prepare_eig_kernels();
@@ -167,11 +167,13 @@ cudaError_t launch_window_gemm(int prec, int two_nev, SlotState* st_, const Slot
 // eig of an n x n row-major matrix; Y, Z (n x nsel row-major columns) for the
 // nsel smallest-|lambda| eigenvalues; lam gets all n eigenvalues (sorted).
 cudaError_t launch_small_eig(int n, const double2* A, int lda, int nsel, double2* lam,
-                             double2* Y, double2* Z, int ldyz, int* info, double2* work, cudaStream_t st);
+                             double2* Y, double2* Z, int ldyz, int* info, cudaStream_t st);
 cudaError_t launch_restart_coeffs_single(int m, int nev, const double2* H, int* r, double2* Yc,
                                          double2* Zc, double2* lam, int* info, double2* work, cudaStream_t st);
 // LU with partial pivoting of n x n (row-major, in place), piv[n]; info != 0 if singular.
-cudaError_t launch_lu_factor(int n, double2* A, int lda, int* piv, int* info, cudaStream_t st);
+// A2 (may be null): a second matrix of the same n and lda in the same launch. n <= 80.
+cudaError_t launch_lu_factor(int n, double2* A, int lda, int* piv, int* info, cudaStream_t st,
+                             double2* A2 = nullptr, int* piv2 = nullptr, int* info2 = nullptr);
 // Solve A X = B (trans = 0) or A^H X = B (trans = 1) with the LU factors; B is n x nrhs (ldb), in place.
 cudaError_t launch_lu_solve(int n, const double2* LU, int lda, const int* piv, int trans, int nrhs,
                             double2* B, int ldb, cudaStream_t st);
@@ -185,19 +187,13 @@ cudaError_t launch_lu_part(int n, const double2* LU, int lda, const int* piv, in
 // LU stopped at the first pivot below tau * |first pivot|; out[0] = pivots kept r,
 // out[1 + i], out[1 + n + i] = row and column index of pivot i.
 cudaError_t launch_pivot_select(int n, const double2* B, int ld, double tau, int* out, cudaStream_t st);
-// Final Ritz pairs of one slot's window: eig(H^(vs)), nev smallest;
-// coefficients Y (vs x nev) and Z into Yc/Zc with the window scales folded in.
-cudaError_t launch_final_ritz(SlotState* st_, const SlotPtrs* ptrs, int slot, double2* Yc, double2* Zc,
-                              double2* lam, int* nout, double2* work, cudaStream_t st);
-// The same for slots slot0 .. slot0+nslots-1 in one launch (one block each):
-// slot slot0 + j writes Yc/Zc + j ostride, lam + j lstride, nout[j], and uses
-// the work area work + j eig_work_elems().
+// Final Ritz pairs of the windows of slots slot0 .. slot0+nslots-1 in one launch (one
+// block each): eig(H^(vs)), nev smallest; slot slot0 + j writes the coefficients
+// (vs x nev) with the window scales folded in to Yc/Zc + j ostride, the values to
+// lam + j lstride and their number to nout[j].
 cudaError_t launch_final_ritz_slots(SlotState* st_, const SlotPtrs* ptrs, int slot0, int nslots, double2* Yc,
                                     double2* Zc, double2* lam, int* nout, size_t ostride, size_t lstride,
-                                    double2* work, cudaStream_t st);
-// Small matrix helpers: C = A B (all row-major, n x k x m), one CTA.
-cudaError_t launch_small_gemm(int n, int k, int m, const double2* A, int lda, int transA,
-                              const double2* B, int ldb, double2* C, int ldc, cudaStream_t st);
+                                    cudaStream_t st);
 
 // Even-odd (Schur complement) operator A_hat = 1 - k^2 D_oe D_eo on the odd half
 // lattice (evenodd.cu). Half fields: V/2 sites, half index h = s >> 1.

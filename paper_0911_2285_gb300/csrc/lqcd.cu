@@ -905,8 +905,7 @@ lqcd_status refactor(lqcd_ctx* c) {
     copy_block_kernel<<<64, 256, 0, c->stream>>>(c->Mdef, ld, c->Mlu, ld, n, n);
     count_launches(2);
     CK(cudaGetLastError());
-    CK(launch_lu_factor(n, c->Hlu, ld, c->Hpiv, c->dinfo, c->stream));
-    CK(launch_lu_factor(n, c->Mlu, ld, c->Mpiv, c->dinfo + 1, c->stream));
+    CK(launch_lu_factor(n, c->Hlu, ld, c->Hpiv, c->dinfo, c->stream, c->Mlu, c->Mpiv, c->dinfo + 1));
     return LQCD_OK;
 }
 
@@ -1223,8 +1222,7 @@ lqcd_status grow_slot(lqcd_ctx* c, int s, bool ritz_ready = false) {
     double2* Zc = Yc + (size_t)MAX_M * MAX_M;
     double2* lam = Zc + (size_t)MAX_M * MAX_M;
     if (!ritz_ready)
-        CK(launch_final_ritz_slots(c->d_state, c->d_ptrs, s, 1, Yc, Zc, lam, c->ritz_n + s, 0, 0, c->eigwork,
-                                   c->stream));
+        CK(launch_final_ritz_slots(c->d_state, c->d_ptrs, s, 1, Yc, Zc, lam, c->ritz_n + s, 0, 0, c->stream));
     std::vector<double2> hl(nsel);
     CK(cudaMemcpyAsync(hl.data(), lam, sizeof(double2) * nsel, cudaMemcpyDeviceToHost, c->stream));
     const SlotPtrs& P = c->h_ptrs[s];
@@ -1249,7 +1247,7 @@ lqcd_status grow_from_windows(lqcd_ctx* c, int k) {
         double2* Yc = c->ritz_all;
         CK(launch_final_ritz_slots(c->d_state, c->d_ptrs, 0, k, Yc, Yc + (size_t)MAX_M * MAX_M,
                                    Yc + (size_t)2 * MAX_M * MAX_M, c->ritz_n, RITZ_STRIDE, RITZ_STRIDE,
-                                   c->eigwork, c->stream));
+                                   c->stream));
     }
     for (int s = 0; s < k; ++s) {
         lqcd_status r = grow_slot(c, s, true);
@@ -1491,7 +1489,7 @@ extern "C" lqcd_status lqcd_eigs(lqcd_ctx* c, int* n_inout, double* evals, doubl
     CK(cudaGetLastError());
     CK(launch_lu_part(n, Mp, ldp, Mpiv, LU_LEFT_PL, n, G, n, c->stream));
     CK(launch_lu_part(n, Mp, ldp, Mpiv, LU_RIGHT_U, n, G, n, c->stream));
-    CK(launch_small_eig(n, G, n, n, lam, Y, Z, n, c->dinfo + 16, c->eigwork, c->stream));
+    CK(launch_small_eig(n, G, n, n, lam, Y, Z, n, c->dinfo + 16, c->stream));
     CK(launch_lu_part(n, Mp, ldp, Mpiv, LU_LEFT_U, n, Y, n, c->stream));
     CK(launch_lu_part(n, Mp, ldp, Mpiv, LU_LEFT_LH, n, Z, n, c->stream));
     std::vector<double2> hl(n);
@@ -1566,21 +1564,21 @@ extern "C" lqcd_status lqcd_last_window(lqcd_ctx* c, int slot, int* vs, double* 
 // ============================================================ test hooks
 extern "C" lqcd_status lqcd_small_eig(int n, const double* C, double* evals, double* Yout, double* Zout) {
     if (n < 1 || n > MAX_SMALL || !C || !evals) return LQCD_ERR_ARG;
-    double2 *dA = nullptr, *dl = nullptr, *dY = nullptr, *dZ = nullptr, *dw = nullptr;
+    double2 *dA = nullptr, *dl = nullptr, *dY = nullptr, *dZ = nullptr;
     int* dinfo = nullptr;
     size_t nn = (size_t)n * n;
     lqcd_status ret = LQCD_OK;
     cudaError_t e;
     if ((e = cudaMalloc(&dA, nn * 16)) != cudaSuccess || (e = cudaMalloc(&dl, n * 16)) != cudaSuccess ||
         (e = cudaMalloc(&dY, nn * 16)) != cudaSuccess || (e = cudaMalloc(&dZ, nn * 16)) != cudaSuccess ||
-        (e = cudaMalloc(&dw, eig_work_elems() * 16)) != cudaSuccess || (e = cudaMalloc(&dinfo, 16)) != cudaSuccess) {
+        (e = cudaMalloc(&dinfo, 16)) != cudaSuccess) {
         set_error("cudaMalloc", e);
         ret = LQCD_ERR_OOM;
     }
     int info = 0;
     if (ret == LQCD_OK) {
         e = cudaMemcpy(dA, C, nn * 16, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = launch_small_eig(n, dA, n, n, dl, dY, dZ, n, dinfo, dw, 0);
+        if (e == cudaSuccess) e = launch_small_eig(n, dA, n, n, dl, dY, dZ, n, dinfo, 0);
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
         if (e == cudaSuccess) e = cudaMemcpy(evals, dl, n * 16, cudaMemcpyDeviceToHost);
         if (e == cudaSuccess && Yout) e = cudaMemcpy(Yout, dY, nn * 16, cudaMemcpyDeviceToHost);
@@ -1589,7 +1587,7 @@ extern "C" lqcd_status lqcd_small_eig(int n, const double* C, double* evals, dou
         if (e != cudaSuccess) { set_error("small eig", e); ret = LQCD_ERR_CUDA; }
         else if (info) { g_last_error = "QR iteration did not converge"; ret = LQCD_ERR_NOCONV; }
     }
-    cudaFree(dA); cudaFree(dl); cudaFree(dY); cudaFree(dZ); cudaFree(dw); cudaFree(dinfo);
+    cudaFree(dA); cudaFree(dl); cudaFree(dY); cudaFree(dZ); cudaFree(dinfo);
     return ret;
 }
 
