@@ -9,7 +9,7 @@
 // cross terms of the low parts). The convergence certificate of a solve is
 // still the native FP64 residual.
 #pragma once
-#include "common.cuh"
+#include "fp64.cuh"
 
 namespace lqcd {
 
@@ -25,15 +25,24 @@ __device__ __forceinline__ dfl operator+(dfl a, dfl b) {
     return {h, e - (h - s)};
 }
 __device__ __forceinline__ dfl operator-(dfl a, dfl b) { return a + (-b); }
+// a + f b, f = +-1
+__device__ __forceinline__ dfl df_axpy(dfl a, float f, dfl b) {
+    const float s = fmaf(f, b.h, a.h), v = s - a.h;
+    float e = (a.h - (s - v)) + fmaf(f, b.h, -v);
+    e += fmaf(f, b.l, a.l);
+    const float h = s + e;
+    return {h, e - (h - s)};
+}
 __device__ __forceinline__ dfc operator+(dfc a, dfc b) { return {a.x + b.x, a.y + b.y}; }
 __device__ __forceinline__ dfc operator-(dfc a, dfc b) { return {a.x - b.x, a.y - b.y}; }
 __device__ __forceinline__ dfc operator-(dfc a) { return {-a.x, -a.y}; }
 
+// One FP64 instruction each (the conversions run on the integer pipe).
 __device__ __forceinline__ dfl df_split(double v) {
-    const float h = __double2float_rn(v);
-    return {h, __double2float_rn(v - (double)h)};
+    const float h = narrow(v);
+    return {h, narrow(v - widen(h))};
 }
-__device__ __forceinline__ double df_value(dfl a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ double df_value(dfl a) { return widen(a.h) + widen(a.l); }
 
 // Compensated sum of products a_i b_i: s + c, c collecting every rounding error.
 struct Dot2 {
@@ -54,77 +63,22 @@ struct Dot2 {
         s = s2;
         c += q + e;
     }
+    // + (h + l), exact product signs folded in by the caller
+    __device__ __forceinline__ void plus(float h, float l) {
+        const float s2 = s + h, bp = s2 - s;
+        c += ((s - (s2 - bp)) + (h - bp)) + l;
+        s = s2;
+    }
+    // + f (h + l), f = +-1: the same two-sum with the sign in the multiply-adds
+    __device__ __forceinline__ void plus(float f, float h, float l) {
+        const float s2 = fmaf(f, h, s), bp = s2 - s;
+        c += fmaf(f, l, (s - (s2 - bp)) + fmaf(f, h, -bp));
+        s = s2;
+    }
     __device__ __forceinline__ dfl done() const {
         const float h = s + c;
         return {h, c - (h - s)};
     }
 };
-
-// Link element (mu, e) of site s: float4 (h.re, h.im, l.re, l.im) in [mu][9][V].
-struct LinksDF {
-    const float4* u;
-    int V;
-    __device__ __forceinline__ void load(int mu, int s, dfc (&m)[3][3]) const {
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            const float4 t = __ldg(u + (size_t)(mu * 9 + e) * V + s);
-            m[e / 3][e % 3] = {{t.x, t.z}, {t.y, t.w}};
-        }
-    }
-};
-
-// Field in double-float form, same complex indexing as the FP64 layout.
-struct FieldDF {
-    const float4* p;
-    int V;
-    __device__ __forceinline__ void load(int s, dfc (&v)[12]) const {
-#pragma unroll
-        for (int c = 0; c < 12; ++c) {
-            const float4 t = __ldg(p + ((size_t)(c >> 1) * V + s) * 2 + (c & 1));
-            v[c] = {{t.x, t.z}, {t.y, t.w}};
-        }
-    }
-};
-
-__device__ __forceinline__ void su3_mul_df(const dfc (&u)[3][3], const dfc (&h)[2][3], dfc (&o)[2][3]) {
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            Dot2 re, im;
-            re.first(u[r][0].x, h[a][0].x);
-            re.add(-u[r][0].y, h[a][0].y);
-            im.first(u[r][0].x, h[a][0].y);
-            im.add(u[r][0].y, h[a][0].x);
-#pragma unroll
-            for (int c = 1; c < 3; ++c) {
-                re.add(u[r][c].x, h[a][c].x);
-                re.add(-u[r][c].y, h[a][c].y);
-                im.add(u[r][c].x, h[a][c].y);
-                im.add(u[r][c].y, h[a][c].x);
-            }
-            o[a][r] = {re.done(), im.done()};
-        }
-}
-__device__ __forceinline__ void su3_dag_mul_df(const dfc (&u)[3][3], const dfc (&h)[2][3], dfc (&o)[2][3]) {
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            Dot2 re, im;
-            re.first(u[0][r].x, h[a][0].x);
-            re.add(u[0][r].y, h[a][0].y);
-            im.first(u[0][r].x, h[a][0].y);
-            im.add(-u[0][r].y, h[a][0].x);
-#pragma unroll
-            for (int c = 1; c < 3; ++c) {
-                re.add(u[c][r].x, h[a][c].x);
-                re.add(u[c][r].y, h[a][c].y);
-                im.add(u[c][r].x, h[a][c].y);
-                im.add(-u[c][r].y, h[a][c].x);
-            }
-            o[a][r] = {re.done(), im.done()};
-        }
-}
 
 }  // namespace lqcd

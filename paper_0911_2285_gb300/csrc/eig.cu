@@ -29,6 +29,7 @@
 
 #include "../../include/lqcd.h"
 #include "dfloat.cuh"
+#include "fp64.cuh"
 #include "kernels.cuh"
 
 namespace lqcd {
@@ -44,48 +45,6 @@ __device__ __forceinline__ double2 cone() { return make_double2(1.0, 0.0); }
 
 // |re| + |im|: the modulus surrogate used for negligibility tests (no sqrt).
 __device__ __forceinline__ double cabs1(double2 a) { return fabs(a.x) + fabs(a.y); }
-
-// FP32 <-> FP64 conversion of a positive number inside FP32's normal range on the
-// integer pipe (the FP64 pipe's conversions take its 64-cycle latency); to FP32
-// by truncation, which is good enough for the Newton seeds below.
-__device__ __forceinline__ float seed_f32(double a) {
-    return __uint_as_float((unsigned)(((__double2hiint(a) - (896 << 20)) << 3) | ((unsigned)__double2loint(a) >> 29)));
-}
-__device__ __forceinline__ double exact_f64(float a) {
-    const unsigned b = __float_as_uint(a);
-    return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
-}
-
-// a positive and inside [2^-99, 2^99): squares and Newton seeds stay in FP32's
-// normal range. On the high word: an FP64 comparison costs the FP64 pipe's latency.
-__device__ __forceinline__ bool mid_range(double a) { return ((unsigned)__double2hiint(a) >> 20) - 924u < 198u; }
-
-// 1/sqrt(a) for a > 0 in FP64: inside FP32's normal range an FP32 reciprocal
-// square root y (relative error about 2^-21) and one step of third order: with
-// e = 1 - a y^2, 1/sqrt(a) = y (1 + e/2 + 3 e^2/8 + O(e^3)). Outside: 1 / sqrt(a).
-__device__ __forceinline__ double rsqrt_fp64(double a) {
-    if (!mid_range(a)) return 1.0 / sqrt(a);
-    const double y = exact_f64(rsqrtf(seed_f32(a)));
-    const double e = fma(-(a * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
-// 1/a in FP64 the same way: FP32 reciprocal seed y, e = 1 - a y,
-// 1/a = y (1 + e + e^2 + O(e^3)). Outside FP32's normal range: 1 / a.
-__device__ __forceinline__ double rcp_fp64(double a) {
-    const double m = fabs(a);
-    if (!mid_range(m)) return 1.0 / a;
-    const double y = copysign(exact_f64(__frcp_rn(seed_f32(m))), a);
-    const double e = fma(-a, y, 1.0);
-    return fma(y * e, 1.0 + e, y);
-}
-
-// sqrt(a) for a >= 0: a / sqrt(a) and one correction of the product's rounding.
-__device__ __forceinline__ double sqrt_fp64(double a) {
-    if (!mid_range(a)) return sqrt(a);
-    const double r = rsqrt_fp64(a), s = a * r;
-    return fma(0.5 * r, fma(-s, s, a), s);
-}
 
 // ------------------------------------------------------ double-float numbers
 // The restart's eigen-solves of H^(m) and H^(m-1) run the reduction in

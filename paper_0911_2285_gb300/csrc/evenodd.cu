@@ -12,6 +12,7 @@
 // half index h = s >> 1 (Lx even, so each pair of sites 2h, 2h + 1 holds one site
 // of each parity); a half field is the chunk layout of common.cuh over V/2 sites.
 #include "dslash.cuh"
+#include "evenodd.cuh"
 #include "kernels.cuh"
 #include "reduce.cuh"
 
@@ -20,26 +21,6 @@ namespace {
 
 constexpr int EO_THREADS = 128;
 constexpr double EO_BREAK_TOL = 1e-14;
-
-// Full site index of half index h in parity P.
-__device__ __forceinline__ int eo_site(const Geom& g, int h, int P) {
-    const int s0 = 2 * h;
-    int r = s0 / g.L[0];
-    const int y = r % g.L[1];
-    r /= g.L[1];
-    const int z = r % g.L[2], t = r / g.L[2];
-    // x of s0 is even, so the parity of s0 is that of y + z + t
-    return s0 + ((((y + z + t) & 1) != P) ? 1 : 0);
-}
-
-// A half field read at full site indices (the neighbours of a site of the other parity).
-template <typename S> struct HalfIn {
-    const void* p;
-    int Vh;
-    template <typename C> __device__ __forceinline__ void load(int s, C (&v)[12]) const {
-        Field<S>::load(p, Vh, s >> 1, v);
-    }
-};
 
 int eo_blocks(int Vh) {
     int nb = (Vh + EO_THREADS - 1) / EO_THREADS;
@@ -246,14 +227,13 @@ __global__ void __launch_bounds__(THREADS, MINB) eo_pair2_kernel(Geom g, const v
     }
 }
 
-// FP64 Schur residual r = b_hat - A_hat x_hi of the slots that asked for it
-// (in-iteration, check_only = 0) or of every started slot (check_only = 1):
+// FP64 Schur residual r = b_hat - A_hat x_hi of every started slot (end of a solve):
 // stage 1 t = D_eo x_hi into the slot's FP64 stage buffer, stage 2 the residual.
 __global__ void __launch_bounds__(EO_THREADS) eo_res1_kernel(Geom g, const void* links64, SlotState* states,
-                                                            const SlotPtrs* ptrs, int check_only) {
+                                                            const SlotPtrs* ptrs) {
     const SlotState& st = states[blockIdx.y];
     const SlotPtrs& P = ptrs[blockIdx.y];
-    if (check_only ? st.status == ST_IDLE : (st.status != ST_RUNNING || !st.need_ru)) return;
+    if (st.status == ST_IDLE) return;
     const int Vh = g.V / 2;
     LinksD U{reinterpret_cast<const double2*>(links64), g.V};
     HalfIn<double> in{P.x_hi, Vh};
@@ -265,10 +245,10 @@ __global__ void __launch_bounds__(EO_THREADS) eo_res1_kernel(Geom g, const void*
 }
 
 __global__ void __launch_bounds__(EO_THREADS) eo_res2_kernel(Geom g, const void* links64, double kappa,
-                                                            SlotState* states, const SlotPtrs* ptrs, int check_only) {
+                                                            SlotState* states, const SlotPtrs* ptrs) {
     SlotState& st = states[blockIdx.y];
     const SlotPtrs& P = ptrs[blockIdx.y];
-    if (check_only ? st.status == ST_IDLE : (st.status != ST_RUNNING || !st.need_ru)) return;
+    if (st.status == ST_IDLE) return;
     const int Vh = g.V / 2;
     LinksD U{reinterpret_cast<const double2*>(links64), g.V};
     HalfIn<double> in{P.eo64, Vh};
@@ -290,7 +270,6 @@ __global__ void __launch_bounds__(EO_THREADS) eo_res2_kernel(Geom g, const void*
     if (reduce_slot<1>(P, CNT_RU, v, tot, gridDim.x, blockIdx.x) && threadIdx.x == 0) {
         st.true_rnorm = sqrt(tot[0].x);
         st.matvecs += 1;
-        if (!check_only && st.true_rnorm <= st.tol * st.bnorm) st.status = ST_CONVERGED;
     }
 }
 
@@ -351,10 +330,10 @@ cudaError_t launch_eo_pair(const Geom& g, const void* links, double kappa, int p
 }
 
 cudaError_t launch_eo_true_resid(const Geom& g, const void* links64, double kappa, SlotState* states,
-                                 const SlotPtrs* ptrs, int nslots, int check_only, cudaStream_t st) {
+                                 const SlotPtrs* ptrs, int nslots, cudaStream_t st) {
     const dim3 grid(eo_blocks(g.V / 2), nslots);
-    eo_res1_kernel<<<grid, EO_THREADS, 0, st>>>(g, links64, states, ptrs, check_only);
-    eo_res2_kernel<<<grid, EO_THREADS, 0, st>>>(g, links64, kappa, states, ptrs, check_only);
+    eo_res1_kernel<<<grid, EO_THREADS, 0, st>>>(g, links64, states, ptrs);
+    eo_res2_kernel<<<grid, EO_THREADS, 0, st>>>(g, links64, kappa, states, ptrs);
     count_launches(2);
     return cudaGetLastError();
 }

@@ -7,16 +7,15 @@
 // partial sums to a fixed slot, and the last block to finish adds them in
 // block order (same result alone or inside a batch).
 #include "dslash.cuh"
-#include "dfloat.cuh"
 #include "kernels.cuh"
 #include "reduce.cuh"
+#include "vec.cuh"
 
 namespace lqcd {
 namespace {
 
 constexpr int DS_THREADS = 128;   // operator kernels
 constexpr int BL_THREADS = 256;   // vector kernels
-constexpr double BREAK_TOL = 1e-14;
 
 inline int div_up(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 
@@ -238,67 +237,6 @@ __global__ void scale_fields_kernel(int b, void* Y, const double2* sc, size_t N)
 }
 
 // ------------------------------------------------------------ BiCG kernels
-// Vector units: two complex numbers (one float4 in FP32, two double2 in FP64).
-template <typename S> struct Unit;
-template <> struct Unit<float> {
-    float2 a, b;
-    __device__ __forceinline__ static Unit load(const void* p, size_t u) {
-        float4 t = reinterpret_cast<const float4*>(p)[u];
-        return Unit{make_float2(t.x, t.y), make_float2(t.z, t.w)};
-    }
-    __device__ __forceinline__ void store(void* p, size_t u) const {
-        reinterpret_cast<float4*>(p)[u] = make_float4(a.x, a.y, b.x, b.y);
-    }
-};
-template <> struct Unit<double> {
-    double2 a, b;
-    __device__ __forceinline__ static Unit load(const void* p, size_t u) {
-        const double2* d = reinterpret_cast<const double2*>(p);
-        return Unit{d[2 * u], d[2 * u + 1]};
-    }
-    __device__ __forceinline__ void store(void* p, size_t u) const {
-        double2* d = reinterpret_cast<double2*>(p);
-        d[2 * u] = a; d[2 * u + 1] = b;
-    }
-};
-
-// Compensated FP32 accumulation of a complex sum (Knuth's two-sum per term), for
-// the gamma5 variant's inner products rho = r^H gamma5 r and sigma = p^H gamma5 A p:
-// their terms have both signs and cancel down to about ||r||^2 / sqrt(N), so a
-// plain FP32 sum would lose three to four digits of them. The per-thread value
-// goes to FP64 block and cross-block sums.
-struct CompC {
-    float sx = 0.f, cx = 0.f, sy = 0.f, cy = 0.f;
-    __device__ __forceinline__ static void add1(float& s, float& c, float v) {
-        const float t = s + v, bp = t - s;
-        c += (s - (t - bp)) + (v - bp);
-        s = t;
-    }
-    __device__ __forceinline__ void add(float2 v) { add1(sx, cx, v.x); add1(sy, cy, v.y); }
-    __device__ __forceinline__ double2 value() const { return make_double2((double)sx + cx, (double)sy + cy); }
-};
-
-// Block and cross-block sum of (z, (a, b)) per slot: in the storage precision,
-// or (gamma5 variant with FP32 storage, compensated z) in FP64 throughout.
-template <typename S>
-__device__ __forceinline__ bool reduce2(const SlotPtrs& P, int kind, bool comp, const CompC& cz, const Acc<S>& acc,
-                                        double2 (&tot)[2], unsigned nblocks, unsigned bid) {
-    if (comp) {
-        double2 v[2] = {cz.value(), make_double2((double)acc.a, (double)acc.b)};
-        return reduce_slot<2>(P, kind, v, tot, nblocks, bid);
-    }
-    cplx<S> v[2];
-    acc.to(v);
-    return reduce_slot<2>(P, kind, v, tot, nblocks, bid);
-}
-
-// gamma5 = diag(1, 1, -1, -1) on a vector unit: units u < N/4 hold spins 0 and 1
-// (chunks q = 0..2 of the field layout), the rest spins 2 and 3.
-template <typename S> __device__ __forceinline__ Unit<S> g5u(Unit<S> v, size_t u, size_t N) {
-    if (u >= N / 4) { v.a = -v.a; v.b = -v.b; }
-    return v;
-}
-
 // Start: r0 = b - A x_hi (already in r_true, FP64), rhat0 = r0 (gamma5 r0 in the
 // gamma5 variant), p = r, phat = rhat, x_lo = 0; rho_0 = (rhat_0, r_0), ||r_0||,
 // ||b||  (Algorithm eigBiCG, steps 1-2).
@@ -634,6 +572,7 @@ __global__ void __launch_bounds__(BL_THREADS) update_kernel(SlotState* states, c
         st.x_owed = 1;
         if (!isfinite(st.rnorm_new) || !isfinite(st.rho_new.x) || !isfinite(st.rho_new.y)) {
             st.status = ST_BREAKDOWN;
+            st.live = 0;
         } else {
             // Reliable update (FP32 Krylov vectors): when the residual has dropped by
             // delta since the last update, or far below the largest residual seen
@@ -648,25 +587,19 @@ __global__ void __launch_bounds__(BL_THREADS) update_kernel(SlotState* states, c
             }
             if (st.rnorm_new > st.rmax) st.rmax = st.rnorm_new;
             if (st.delta > 0.0 && (st.rnorm_new < st.delta * st.r_ru || st.rnorm_new < 1e-3 * st.rmax)) st.need_ru = 1;
+            if (!st.need_ru) bicg_scalars(st, P);   // else the reliable update ends the iteration
         }
     }
 }
 
-// FP64 true residual r = b - A x_hi for slots that asked for it (x_lo has been
-// folded into x_hi just before).
-// check_only = 0: inside the iteration (converged if ||r|| <= tol ||b||);
-// check_only = 1: final report for every slot that was started.
+// FP64 true residual r = b - A x_hi at the end of a solve, for every slot that was
+// started (x_lo has been folded into x_hi just before).
 template <int THREADS, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB) true_resid_kernel(Geom g, const void* links64, double kappa,
-                                                                   SlotState* states, const SlotPtrs* ptrs,
-                                                                   int check_only) {
+                                                                   SlotState* states, const SlotPtrs* ptrs) {
     SlotState& st = states[blockIdx.y];
     const SlotPtrs& P = ptrs[blockIdx.y];
-    if (check_only) {
-        if (st.status == ST_IDLE) return;
-    } else if (st.status != ST_RUNNING || !st.need_ru) {
-        return;
-    }
+    if (st.status == ST_IDLE) return;
     LinksD U{reinterpret_cast<const double2*>(links64), g.V};
     FieldIn<double> in{P.x_hi, g.V};
     double2 v[1] = {make_double2(0, 0)};
@@ -686,235 +619,7 @@ __global__ void __launch_bounds__(THREADS, MINB) true_resid_kernel(Geom g, const
     if (reduce_slot<1>(P, CNT_RU, v, tot, gridDim.x, blockIdx.x) && threadIdx.x == 0) {
         st.true_rnorm = sqrt(tot[0].x);
         st.matvecs += 1;
-        if (!check_only && st.true_rnorm <= st.tol * st.bnorm) st.status = ST_CONVERGED;
     }
-}
-
-// The in-iteration reliable-update residual b - A x_hi with A x_hi in
-// double-float arithmetic (dfloat.cuh): same contract as true_resid_kernel
-// with check_only = 0.
-// One hop in double-float: each colour row of U h (or U^+ h) is formed and
-// added into the accumulator at once, and the link is read row by row, so
-// only a row of U and one colour of U h are live next to h and the sums.
-template <int MU, int SG>
-__device__ __forceinline__ void recon_row_df(dfc a, dfc b, int c, dfc (&acc)[12]) {
-    dfc l0, l1;   // M^+ (a, b)
-    if (MU == 0) { l0 = mul_i(b); l1 = mul_i(a); }
-    else if (MU == 1) { l0 = b; l1 = -a; }
-    else if (MU == 2) { l0 = mul_i(a); l1 = mul_mi(b); }
-    else { l0 = a; l1 = b; }
-    acc[c] = acc[c] + a;
-    acc[3 + c] = acc[3 + c] + b;
-    if (SG > 0) { acc[6 + c] = acc[6 + c] + l0; acc[9 + c] = acc[9 + c] + l1; }
-    else { acc[6 + c] = acc[6 + c] - l0; acc[9 + c] = acc[9 + c] - l1; }
-}
-template <int MU, bool BWD>
-__device__ __forceinline__ void hop_df(const Nbr& nb, const LinksDF& U, const FieldDF& in, int s, dfc (&acc)[12]) {
-    constexpr int SG = BWD ? +1 : -1;
-    dfc h[2][3];
-    {
-        dfc psi[12];
-        in.load(BWD ? nb.b[MU] : nb.f[MU], psi);
-        project<MU, SG>(psi, h);
-    }
-    const int ls = BWD ? nb.b[MU] : s;
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        dfc u[3];   // row r of U (forward) or column r (backward, conjugated below)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float4 t = __ldg(U.u + (size_t)(MU * 9 + (BWD ? 3 * c + r : 3 * r + c)) * U.V + ls);
-            u[c] = {{t.x, t.z}, {t.y, t.w}};
-        }
-        dfc o[2];
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            Dot2 re, im;
-            if (!BWD) {
-                re.first(u[0].x, h[a][0].x); re.add(-u[0].y, h[a][0].y);
-                im.first(u[0].x, h[a][0].y); im.add(u[0].y, h[a][0].x);
-#pragma unroll
-                for (int c = 1; c < 3; ++c) {
-                    re.add(u[c].x, h[a][c].x); re.add(-u[c].y, h[a][c].y);
-                    im.add(u[c].x, h[a][c].y); im.add(u[c].y, h[a][c].x);
-                }
-            } else {
-                re.first(u[0].x, h[a][0].x); re.add(u[0].y, h[a][0].y);
-                im.first(u[0].x, h[a][0].y); im.add(-u[0].y, h[a][0].x);
-#pragma unroll
-                for (int c = 1; c < 3; ++c) {
-                    re.add(u[c].x, h[a][c].x); re.add(u[c].y, h[a][c].y);
-                    im.add(u[c].x, h[a][c].y); im.add(-u[c].y, h[a][c].x);
-                }
-            }
-            o[a] = {re.done(), im.done()};
-        }
-        recon_row_df<MU, SG>(o[0], o[1], r, acc);
-    }
-}
-template <int THREADS, int MINB>
-__global__ void __launch_bounds__(THREADS, MINB) true_resid_df_kernel(Geom g, const float4* links_df, double kappa,
-                                                                      SlotState* states, const SlotPtrs* ptrs) {
-    SlotState& st = states[blockIdx.y];
-    const SlotPtrs& P = ptrs[blockIdx.y];
-    if (st.status != ST_RUNNING || !st.need_ru) return;
-    const LinksDF U{links_df, g.V};
-    const FieldDF in{P.x_df, g.V};
-    double2 v[1] = {make_double2(0, 0)};
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += gridDim.x * blockDim.x) {
-        const Nbr nb(g, s);
-        dfc acc[12];
-#pragma unroll
-        for (int c = 0; c < 12; ++c) acc[c] = {{0.f, 0.f}, {0.f, 0.f}};
-        hop_df<0, false>(nb, U, in, s, acc);
-        hop_df<0, true>(nb, U, in, s, acc);
-        hop_df<1, false>(nb, U, in, s, acc);
-        hop_df<1, true>(nb, U, in, s, acc);
-        hop_df<2, false>(nb, U, in, s, acc);
-        hop_df<2, true>(nb, U, in, s, acc);
-        hop_df<3, false>(nb, U, in, s, acc);
-        hop_df<3, true>(nb, U, in, s, acc);
-        double2 self[12], b[12];
-        Field<double>::load(P.x_hi, g.V, s, self);
-        Field<double>::load(P.b, g.V, s, b);
-#pragma unroll
-        for (int c = 0; c < 12; ++c) {
-            const double2 a = make_double2(df_value(acc[c].x), df_value(acc[c].y));
-            b[c] = b[c] - (self[c] - kappa * a);
-            v[0].x += cabs2(b[c]);
-        }
-        Field<double>::store(P.r_true, g.V, s, b);
-    }
-    double2 tot[1];
-    if (reduce_slot<1>(P, CNT_RU, v, tot, gridDim.x, blockIdx.x) && threadIdx.x == 0) {
-        st.true_rnorm = sqrt(tot[0].x);
-        st.matvecs += 1;
-        if (st.true_rnorm <= st.tol * st.bnorm) st.status = ST_CONVERGED;
-    }
-}
-
-// Reliable update, first half: x_hi += x_lo, x_lo = 0 for slots that asked for it.
-template <typename S>
-__global__ void __launch_bounds__(BL_THREADS) fold_ru_kernel(SlotState* states, const SlotPtrs* ptrs, size_t N) {
-    const SlotState& st = states[blockIdx.y];
-    const SlotPtrs& P = ptrs[blockIdx.y];
-    if (st.status != ST_RUNNING || !st.need_ru) return;
-    const size_t units = N / 2;
-    const cplx<S> al = cvt<S>(st.alpha);
-    Unit<S> zero{mk<S>(0, 0), mk<S>(0, 0)};
-    for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < units; u += (size_t)gridDim.x * blockDim.x) {
-        Unit<double> xh = Unit<double>::load(P.x_hi, u);
-        Unit<S> xl = Unit<S>::load(P.x_lo, u);
-        if (st.x_owed) {   // alpha p of this iteration's residual update
-            const Unit<S> p = Unit<S>::load(P.p, u);
-            xl.a = xl.a + al * p.a; xl.b = xl.b + al * p.b;
-        }
-        xh.a = xh.a + to_d(xl.a); xh.b = xh.b + to_d(xl.b);
-        xh.store(P.x_hi, u);
-        zero.store(P.x_lo, u);
-        if (P.x_df) {   // the double-float copy read by the reliable-update residual
-            const dfl ar = df_split(xh.a.x), ai = df_split(xh.a.y), br = df_split(xh.b.x), bi = df_split(xh.b.y);
-            P.x_df[2 * u] = make_float4(ar.h, ai.h, ar.l, ai.l);
-            P.x_df[2 * u + 1] = make_float4(br.h, bi.h, br.l, bi.l);
-        }
-    }
-}
-
-// Reliable update, second half: unless converged, the recursive residual r_j is
-// replaced by the true one and rho_j recomputed.
-template <typename S>
-__global__ void __launch_bounds__(BL_THREADS) replace_kernel(SlotState* states, const SlotPtrs* ptrs, size_t N) {
-    SlotState& st = states[blockIdx.y];
-    const SlotPtrs& P = ptrs[blockIdx.y];
-    if (!st.live || !st.need_ru || (st.status != ST_RUNNING && st.status != ST_CONVERGED)) return;
-    const bool run = st.status == ST_RUNNING;
-    void* rcur = slot_field<S>(P.V, next_slot(st), N);
-    void* hcur = slot_field<S>(P.W, next_slot(st), N);
-    cplx<S> rho = mk<S>(S(0), S(0));
-    CompC cz;   // gamma5 variant, FP32 storage
-    const bool comp = st.g5 && sizeof(S) == 4;
-    const size_t units = N / 2;
-    for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < units; u += (size_t)gridDim.x * blockDim.x) {
-        if (run) {
-            Unit<double> rt = Unit<double>::load(P.r_true, u);
-            Unit<S> r{cvt<S>(rt.a), cvt<S>(rt.b)};
-            r.store(rcur, u);
-            Unit<S> h;
-            if (st.g5) {   // the shadow residual follows: rhat = gamma5 r
-                h = g5u(r, u, N);
-                if (st.m > 0) h.store(hcur, u);
-            } else {
-                h = Unit<S>::load(hcur, u);
-            }
-            if (comp) {
-                if constexpr (sizeof(S) == 4) { cz.add(cdot(h.a, r.a)); cz.add(cdot(h.b, r.b)); }
-            } else {
-                rho = rho + cdot(h.a, r.a) + cdot(h.b, r.b);
-            }
-        }
-    }
-    double2 tot[1];
-    bool last;
-    if (comp) {
-        double2 v[1] = {cz.value()};
-        last = reduce_slot<1>(P, CNT_REPLACE, v, tot, gridDim.x, blockIdx.x);
-    } else {
-        cplx<S> v[1] = {rho};
-        last = reduce_slot<1>(P, CNT_REPLACE, v, tot, gridDim.x, blockIdx.x);
-    }
-    if (last && threadIdx.x == 0) {
-        if (run) {
-            st.rho_new = tot[0];
-            st.rnorm_new = st.true_rnorm;
-            st.rmax = st.true_rnorm;
-            st.r_ru = st.true_rnorm;
-        }
-        st.need_ru = 0;
-        st.ru_count += 1;
-        st.x_owed = 0;   // the fold added alpha p
-    }
-}
-
-// Scalar bookkeeping of one iteration (one thread per slot):
-// beta_{j-1} = rho_j / rho_{j-1}; window append v = r/||r||, w = (||r||/conj(rho)) rhat;
-// tridiagonal entries of H (Algorithm eigBiCG, step 3); iteration counters.
-__global__ void scalars_kernel(SlotState* states, const SlotPtrs* ptrs) {
-    if (threadIdx.x != 0) return;
-    SlotState& st = states[blockIdx.x];
-    const SlotPtrs& P = ptrs[blockIdx.x];
-    if (!st.live || st.stab) return;
-    if (st.status == ST_BREAKDOWN) { st.live = 0; return; }
-    const double2 beta = cdiv(st.rho_new, st.rho);
-    if (st.m > 0) {
-        const int k = st.vs;   // 0-based index of the appended vector
-        const int m = st.m;
-        P.vscale[k] = 1.0 / st.rnorm;
-        P.wscale[k] = cdiv(make_double2(st.rnorm, 0.0), conj_(st.rho));
-        const double2 inv_a = cdiv(make_double2(1.0, 0.0), st.alpha);
-        double2 diag = inv_a;
-        if (st.iter > 0) diag = diag + cdiv(st.beta_prev, st.alpha_prev);
-        P.H[k * m + k] = diag;
-        if (k + 1 < m) {
-            P.H[k * m + k + 1] = -(st.rnorm / st.rnorm_new) * cdiv(beta, st.alpha);
-            P.H[(k + 1) * m + k] = -(st.rnorm_new / st.rnorm) * inv_a;
-        }
-        st.vs = k + 1;
-    }
-    st.beta = beta;
-    st.alpha_prev = st.alpha;
-    st.beta_prev = beta;
-    st.rho = st.rho_new;
-    st.rnorm = st.rnorm_new;
-    st.iter += 1;
-    if (st.status == ST_RUNNING) {
-        if (st.iter >= st.maxiter) st.status = ST_NOCONV;
-        else if (!(cabs_(st.rho) >= BREAK_TOL * st.rhat_norm * st.rnorm)) st.status = ST_BREAKDOWN;
-    }
-    if (st.status != ST_RUNNING) st.live = 0;
-    // the direction update adds the owed alpha p; a slot that stops here keeps it
-    // owed for the final fold
-    if (st.status == ST_RUNNING) { st.x_dir = st.x_owed; st.x_owed = 0; }
-    else st.x_dir = 0;
 }
 
 // p_j = r_j + beta p_{j-1}, phat_j = rhat_j + conj(beta) phat_{j-1}.
@@ -1094,26 +799,9 @@ __global__ void __launch_bounds__(BL_THREADS) stab_update_kernel(SlotState* stat
             if (st.rnorm_new <= st.tol * st.bnorm) st.need_ru = 1;
             if (st.rnorm_new > st.rmax) st.rmax = st.rnorm_new;
             if (st.delta > 0.0 && (st.rnorm_new < st.delta * st.r_ru || st.rnorm_new < 1e-3 * st.rmax)) st.need_ru = 1;
+            if (!st.need_ru) stab_scalars(st);
         }
     }
-}
-
-// beta = (rho' / rho) (alpha / omega); counters; maxiter and breakdown (rho or omega).
-__global__ void stab_scalars_kernel(SlotState* states) {
-    if (threadIdx.x != 0) return;
-    SlotState& st = states[blockIdx.x];
-    if (!st.live || !st.stab) return;
-    if (st.status == ST_BREAKDOWN) { st.live = 0; return; }
-    st.iter += 1;
-    const bool om0 = cabs2(st.omega) == 0.0;
-    if (!om0) st.beta = cdiv(st.rho_new, st.rho) * cdiv(st.alpha, st.omega);
-    st.rho = st.rho_new;
-    st.rnorm = st.rnorm_new;
-    if (st.status == ST_RUNNING) {
-        if (st.iter >= st.maxiter) st.status = ST_NOCONV;
-        else if (om0 || !(cabs_(st.rho) >= BREAK_TOL * st.rhat_norm * st.rnorm)) st.status = ST_BREAKDOWN;
-    }
-    if (st.status != ST_RUNNING) st.live = 0;
 }
 
 // Fold x_lo into x_hi at the end of a solve (x = 0 for a zero source).
@@ -1296,15 +984,6 @@ __global__ void __launch_bounds__(WG_T * ((RMAX + WG_K - 1) / WG_K))
 
 }  // namespace
 
-// FP64 links [mu][9][V] double2 -> double-float float4 (h.re, h.im, l.re, l.im).
-__global__ void links_df_kernel(const double2* l64, float4* ldf, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const double2 v = l64[i];
-        const dfl r = df_split(v.x), m = df_split(v.y);
-        ldf[i] = make_float4(r.h, m.h, r.l, m.l);
-    }
-}
-
 // ------------------------------------------------------------------ launchers
 static Geom geom_of(const Geom& g) { return g; }
 
@@ -1422,12 +1101,6 @@ cudaError_t launch_norms(int b, const void* Y, int yp, size_t N, double* out, do
     else norms_kernel<float><<<grid, BL_THREADS, 0, st>>>(Y, N, scratch);
     norms_reduce_kernel<<<(b + 63) / 64, 64, 0, st>>>(b, nb, scratch, out);
     count_launches(2);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_links_df(const double2* l64, float4* ldf, size_t n, cudaStream_t st) {
-    links_df_kernel<<<1216, 256, 0, st>>>(l64, ldf, n);
-    count_launches(1);
     return cudaGetLastError();
 }
 
@@ -1567,50 +1240,20 @@ cudaError_t launch_bicg_update(int prec, SlotState* states, const SlotPtrs* ptrs
 // pipe) decides; the library times them at init.
 template <int THREADS, int MINB>
 static void true_resid_launch(const Geom& g, const void* links64, double kappa, SlotState* states,
-                              const SlotPtrs* ptrs, int nslots, int check_only, cudaStream_t s) {
+                              const SlotPtrs* ptrs, int nslots, cudaStream_t s) {
     int nb = div_up((size_t)g.V, THREADS);
     if (nb > PARTIAL_STRIDE / 2) nb = PARTIAL_STRIDE / 2;
-    true_resid_kernel<THREADS, MINB><<<dim3(nb, nslots), THREADS, 0, s>>>(g, links64, kappa, states, ptrs, check_only);
+    true_resid_kernel<THREADS, MINB><<<dim3(nb, nslots), THREADS, 0, s>>>(g, links64, kappa, states, ptrs);
 }
-int true_resid_variants() { return 6; }
-static void launch_true_resid(int variant, const Geom& g, const void* links64, const float4* links_df,
-                              double kappa, SlotState* states, const SlotPtrs* ptrs, int nslots, int check_only,
-                              cudaStream_t s) {
-    if ((variant == RU_DF || variant == RU_DF + 1) && !check_only && links_df) {
-        int nb = div_up((size_t)g.V, 128);
-        if (nb > PARTIAL_STRIDE / 2) nb = PARTIAL_STRIDE / 2;
-        if (variant == RU_DF)
-            true_resid_df_kernel<128, 4><<<dim3(nb, nslots), 128, 0, s>>>(g, links_df, kappa, states, ptrs);
-        else
-            true_resid_df_kernel<128, 2><<<dim3(nb, nslots), 128, 0, s>>>(g, links_df, kappa, states, ptrs);
-        return;
-    }
+int true_resid_variants() { return 4; }
+cudaError_t launch_true_resid(int variant, const Geom& g, const void* links64, double kappa, SlotState* states,
+                              const SlotPtrs* ptrs, int nslots, cudaStream_t s) {
     switch (variant) {
-        case 1: true_resid_launch<128, 3>(g, links64, kappa, states, ptrs, nslots, check_only, s); break;
-        case 2: true_resid_launch<128, 4>(g, links64, kappa, states, ptrs, nslots, check_only, s); break;
-        case 3: true_resid_launch<64, 6>(g, links64, kappa, states, ptrs, nslots, check_only, s); break;
-        default: true_resid_launch<128, 1>(g, links64, kappa, states, ptrs, nslots, check_only, s); break;
+        case 1: true_resid_launch<128, 3>(g, links64, kappa, states, ptrs, nslots, s); break;
+        case 2: true_resid_launch<128, 4>(g, links64, kappa, states, ptrs, nslots, s); break;
+        case 3: true_resid_launch<64, 6>(g, links64, kappa, states, ptrs, nslots, s); break;
+        default: true_resid_launch<128, 1>(g, links64, kappa, states, ptrs, nslots, s); break;
     }
-}
-
-cudaError_t launch_bicg_ru(const Geom& g, const void* links64, double kappa, int prec, SlotState* states,
-                           const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s, int ru_variant,
-                           const float4* links_df, int eo) {
-    dim3 g2(blas_blocks(N / 2), nslots);
-    if (prec == 0) fold_ru_kernel<double><<<g2, BL_THREADS, 0, s>>>(states, ptrs, N);
-    else fold_ru_kernel<float><<<g2, BL_THREADS, 0, s>>>(states, ptrs, N);
-    count_launches(1);
-    if (eo) {
-        cudaError_t e = launch_eo_true_resid(g, links64, kappa, states, ptrs, nslots, 0, s);
-        if (e != cudaSuccess) return e;
-    } else {
-        launch_true_resid(ru_variant, g, links64, links_df, kappa, states, ptrs, nslots, 0, s);
-        count_launches(1);
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (prec == 0) replace_kernel<double><<<g2, BL_THREADS, 0, s>>>(states, ptrs, N);
-    else replace_kernel<float><<<g2, BL_THREADS, 0, s>>>(states, ptrs, N);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1643,18 +1286,6 @@ cudaError_t launch_stab_step(const Geom& g, const void* links, double kappa, int
     return cudaGetLastError();
 }
 
-cudaError_t launch_stab_scalars(SlotState* states, int nslots, cudaStream_t s) {
-    stab_scalars_kernel<<<nslots, 32, 0, s>>>(states);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_bicg_scalars(SlotState* states, const SlotPtrs* ptrs, int nslots, cudaStream_t s) {
-    scalars_kernel<<<nslots, 32, 0, s>>>(states, ptrs);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_bicg_direction(int prec, SlotState* states, const SlotPtrs* ptrs, int nslots, size_t N,
                                   cudaStream_t s) {
     dim3 grid(blas_blocks(N / 2), nslots);
@@ -1672,10 +1303,8 @@ cudaError_t launch_bicg_finish(const Geom& g, const void* links64, double kappa,
     count_launches(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (eo) return launch_eo_true_resid(g, links64, kappa, states, ptrs, nslots, 1, s);
-    launch_true_resid(ru_variant >= RU_DF ? 0 : ru_variant, g, links64, nullptr, kappa, states, ptrs, nslots, 1, s);
-    count_launches(1);
-    return cudaGetLastError();
+    if (eo) return launch_eo_true_resid(g, links64, kappa, states, ptrs, nslots, s);
+    return launch_true_resid(ru_variant, g, links64, kappa, states, ptrs, nslots, s);
 }
 
 template <typename S, int RMAX>

@@ -130,24 +130,30 @@ bool matvec_g5_variant_ok(const Geom& g, int v);
 cudaError_t launch_bicg_matvec_g5(const Geom& g, const void* links, double kappa, int prec,
                                   SlotState* st_, const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant);
 cudaError_t launch_bicg_update(int prec, SlotState* st_, const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s);
-// ru_variant: true-residual kernel shape (0 .. true_resid_variants()-1, timed at init);
-// RU_DF and RU_DF + 1 evaluate A x_hi in double-float arithmetic (needs links_df
-// and the slots' x_df); the final residual of launch_bicg_finish is always native FP64.
-constexpr int RU_DF = 4;
+// FP64 residual of the started slots at the end of a solve, in one of
+// true_resid_variants() kernel shapes (timed at init).
 int true_resid_variants();
-// eo: the even-odd Schur residual (FP64) instead of the full-lattice one.
-cudaError_t launch_bicg_ru(const Geom& g, const void* links64, double kappa, int prec,
-                           SlotState* st_, const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s,
-                           int ru_variant = 0, const float4* links_df = nullptr, int eo = 0);
+cudaError_t launch_true_resid(int variant, const Geom& g, const void* links64, double kappa, SlotState* st_,
+                              const SlotPtrs* ptrs, int nslots, cudaStream_t s);
+// Reliable update of the slots that asked for it (reliable.cu): x_hi += x_lo, the
+// true residual b - A x_hi, and unless it meets the tolerance the recursive residual
+// is replaced by it; ends the iteration of these slots (scalars). One cooperative
+// launch. links_df != null: A x_hi in double-float arithmetic (needs the slots'
+// x_df), else FP64; eo: the even-odd Schur residual (FP64). err: device word set to
+// 1 if a bounded wait gave up. max_blocks: ru_max_blocks().
+cudaError_t launch_bicg_ru(const Geom& g, const void* links64, double kappa, int prec, SlotState* st_,
+                           const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s, const float4* links_df, int eo,
+                           int max_blocks, int* err);
+// Blocks of the reliable-update kernel that the current device can hold at once.
+cudaError_t ru_max_blocks(int prec, int df, int eo, int* blocks);
+cudaError_t set_wait_cycles_ru(long long cycles);
 // FP64 links -> double-float links (n complex elements).
 cudaError_t launch_links_df(const double2* l64, float4* ldf, size_t n, cudaStream_t st);
-cudaError_t launch_bicg_scalars(SlotState* st_, const SlotPtrs* ptrs, int nslots, cudaStream_t s);
 // BiCGStab step over the slots with stab set (direction, v = A p with alpha, s,
-// t = A s with omega, x and r update with rho and the reliable-update flags),
-// then (after launch_bicg_ru) the scalars: beta, counters, maxiter, breakdown.
+// t = A s with omega, x and r update with rho, the reliable-update flags and, where
+// none is due, the scalars: beta, counters, maxiter, breakdown).
 cudaError_t launch_stab_step(const Geom& g, const void* links, double kappa, int prec, SlotState* st_,
                              const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s);
-cudaError_t launch_stab_scalars(SlotState* st_, int nslots, cudaStream_t s);
 cudaError_t launch_bicg_direction(int prec, SlotState* st_, const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s);
 cudaError_t launch_bicg_finish(const Geom& g, const void* links64, double kappa, int prec,
                                SlotState* st_, const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s,
@@ -212,9 +218,9 @@ cudaError_t launch_eo_reconstruct(const Geom& g, const void* links64, double kap
 // BiCG operator pair on A_hat over the slots (two stages through eo_t, eo_th) with sigma and alpha.
 cudaError_t launch_eo_pair(const Geom& g, const void* links, double kappa, int prec, SlotState* states,
                            const SlotPtrs* ptrs, int nslots, cudaStream_t st);
-// FP64 Schur residual b_hat - A_hat x_hi (through eo64): in-iteration (check_only 0) or final.
+// FP64 Schur residual b_hat - A_hat x_hi (through eo64) at the end of a solve.
 cudaError_t launch_eo_true_resid(const Geom& g, const void* links64, double kappa, SlotState* states,
-                                 const SlotPtrs* ptrs, int nslots, int check_only, cudaStream_t st);
+                                 const SlotPtrs* ptrs, int nslots, cudaStream_t st);
 
 // Bound of the device-side waits (SM clock cycles) of the kernels of gemm_tc.cu
 // and dslash_tiled.cu on the current device; cycles <= 0 restores the default.

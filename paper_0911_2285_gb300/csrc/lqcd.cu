@@ -157,7 +157,8 @@ struct lqcd_ctx {
 
     int dslash_variant = 0;         // operator-kernel shape (autotuned at init); TILED = plane streaming
     int use_tc = 1;                 // FP32 projections and restart products on the tensor cores
-    int ru_variant = 0;             // FP64 true-residual kernel shape (timed at init)
+    int ru_variant = 0;             // kernel shape of the final FP64 residual (timed at init)
+    int ru_blocks = 1;              // co-resident blocks of the reliable-update kernel
     TileGeom tgeo[MAX_SLOTS + 1] = {};
     bool tile_ok[MAX_SLOTS + 1] = {};
     long long deflations_discarded = 0;   // oblique projections undone (deflate_range)
@@ -596,6 +597,8 @@ extern "C" lqcd_status lqcd_eigbicg_init(lqcd_ctx** out, const lqcd_params* para
         if (e == cudaErrorInvalidValue) { cudaGetLastError(); e = cudaSuccess; }
         if (e != cudaSuccess) { set_error("prepare_staged", e); return fail(LQCD_ERR_CUDA); }
     }
+    e = ru_max_blocks(c->kprec, c->links_df != nullptr && !c->eo, c->eo ? 1 : 0, &c->ru_blocks);
+    if (e != cudaSuccess) { set_error("ru_max_blocks", e); return fail(LQCD_ERR_CUDA); }
     st = c->p.no_autotune ? LQCD_OK : autotune(c);
     if (st != LQCD_OK) return fail(st);
     c->kbatch = c->kmax;
@@ -1092,6 +1095,12 @@ cudaError_t launch_matvec(lqcd_ctx* c, int nslots, int variant) {
                               variant == TILED ? 0 : variant);
 }
 
+// The reliable update of an iteration (a no-op for slots that need none).
+cudaError_t launch_ru(lqcd_ctx* c, int nslots) {
+    return launch_bicg_ru(c->g, c->links64, c->p.kappa, c->kprec, c->d_state, c->d_ptrs, nslots, c->N, c->stream,
+                          c->links_df, c->eo ? 1 : 0, c->ru_blocks, c->d_err);
+}
+
 // One chunk of CHECK_EVERY iterations for nslots slots (graph body).
 // Kernel groups of an iteration chunk (bit mask): BiCG iteration, its eigBiCG
 // window (restart), BiCGStab iteration. Each kernel skips the slots of the
@@ -1111,16 +1120,12 @@ lqcd_status enqueue_chunk(lqcd_ctx* c, int nslots, int kinds) {
                     CK(launch_window_gemm(c->kprec, 2 * c->nev, c->d_state, c->d_ptrs, nslots, c->N, c->stream));
             }
             CK(launch_bicg_update(c->kprec, c->d_state, c->d_ptrs, nslots, c->N, c->stream));
-            CK(launch_bicg_ru(c->g, c->links64, c->p.kappa, c->kprec, c->d_state, c->d_ptrs, nslots, c->N,
-                              c->stream, c->ru_variant, c->links_df, c->eo ? 1 : 0));
-            CK(launch_bicg_scalars(c->d_state, c->d_ptrs, nslots, c->stream));
+            CK(launch_ru(c, nslots));
             CK(launch_bicg_direction(c->kprec, c->d_state, c->d_ptrs, nslots, c->N, c->stream));
         }
         if (kinds & CH_STAB) {
             CK(launch_stab_step(c->g, links, c->p.kappa, c->kprec, c->d_state, c->d_ptrs, nslots, c->N, c->stream));
-            CK(launch_bicg_ru(c->g, c->links64, c->p.kappa, c->kprec, c->d_state, c->d_ptrs, nslots, c->N,
-                              c->stream, c->ru_variant, c->links_df, c->eo ? 1 : 0));
-            CK(launch_stab_scalars(c->d_state, nslots, c->stream));
+            CK(launch_ru(c, nslots));
         }
     }
     return LQCD_OK;
@@ -1684,12 +1689,8 @@ static lqcd_status time_kernel_impl(lqcd_ctx* c, int kernel, int k, int reps, do
         return LQCD_ERR_ARG;
     if (kernel == TIME_TILED && !c->tile_ok[k]) return LQCD_ERR_ARG;
     if (c->eo && kernel >= 10) return LQCD_ERR_ARG;   // one operator shape
+    const int resid_shape = kernel >= 40 && kernel < 40 + true_resid_variants() ? kernel - 40 : -1;
     if (kernel >= 10 && kernel < 10 + matvec_variants() && !shape_ok(c, kernel - 10)) return LQCD_ERR_ARG;
-    const int ru_saved = c->ru_variant;
-    if (kernel >= 40 && kernel < 40 + true_resid_variants()) {   // reliable update with FP64 shape v
-        c->ru_variant = kernel - 40;
-        kernel = 3;
-    }
     // Slots 0..k-1 iterate with fixed scalars on whatever their buffers hold.
     std::vector<SlotState> tmpl(c->kmax);
     for (int s = 0; s < c->kmax; ++s) {
@@ -1713,13 +1714,13 @@ static lqcd_status time_kernel_impl(lqcd_ctx* c, int kernel, int k, int reps, do
     for (int r = 0; r < reps; ++r) {
         CK(cudaMemcpyAsync(c->d_state, tmpl.data(), sizeof(SlotState) * c->kmax, cudaMemcpyHostToDevice, c->stream));
         CK(cudaEventRecord(e0, c->stream));
-        if (kernel == 0) CK(launch_matvec(c, k, c->dslash_variant));
+        if (resid_shape >= 0) CK(launch_true_resid(resid_shape, c->g, c->links64, c->p.kappa, c->d_state, c->d_ptrs, k, c->stream));
+        else if (kernel == 0) CK(launch_matvec(c, k, c->dslash_variant));
         else if (kernel == TIME_TILED) CK(launch_matvec(c, k, TILED));
         else if (kernel >= 10) CK(launch_matvec(c, k, kernel - 10));
         else if (kernel == 1) CK(launch_bicg_update(c->kprec, c->d_state, c->d_ptrs, k, c->N, c->stream));
         else if (kernel == 2) CK(launch_bicg_direction(c->kprec, c->d_state, c->d_ptrs, k, c->N, c->stream));
-        else CK(launch_bicg_ru(c->g, c->links64, c->p.kappa, c->kprec, c->d_state, c->d_ptrs, k, c->N, c->stream,
-                               c->ru_variant, c->links_df, c->eo ? 1 : 0));
+        else CK(launch_ru(c, k));
         CK(cudaEventRecord(e1, c->stream));
         CK(cudaEventSynchronize(e1));
         float ms = 0.f;
@@ -1728,7 +1729,6 @@ static lqcd_status time_kernel_impl(lqcd_ctx* c, int kernel, int k, int reps, do
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    c->ru_variant = ru_saved;
     // leave the slots idle
     for (int s = 0; s < c->kmax; ++s) { tmpl[s].status = ST_IDLE; tmpl[s].live = 0; }
     CK(cudaMemcpyAsync(c->d_state, tmpl.data(), sizeof(SlotState) * c->kmax, cudaMemcpyHostToDevice, c->stream));
@@ -1788,11 +1788,10 @@ extern "C" lqcd_status lqcd_set_dslash_variant(lqcd_ctx* c, int variant) {
 static lqcd_status autotune(lqcd_ctx* c) {
     Range nvtx_("autotune operator shapes");
     if (c->eo) return LQCD_OK;   // the even-odd operator and its FP64 residual have one shape each
-    {   // FP64 true-residual shape
+    {   // shape of the final FP64 residual
         double best_ru = 1e300;
         for (int v = 0; v < true_resid_variants(); ++v) {
             double ms = 0.0;
-            if (v >= RU_DF && !c->links_df) continue;
             lqcd_status s = time_kernel_impl(c, 40 + v, 1, 1, &ms);
             if (s != LQCD_OK) return s;
             s = time_kernel_impl(c, 40 + v, 1, 2, &ms);
@@ -2191,6 +2190,7 @@ __device__ int g_flag_status;   // status word of lqcd_wait_flag
 extern "C" lqcd_status lqcd_set_wait_limit(long long cycles) {
     CK(set_wait_cycles_tc(cycles));
     CK(set_wait_cycles_tiled(cycles));
+    CK(set_wait_cycles_ru(cycles));
     return LQCD_OK;
 }
 

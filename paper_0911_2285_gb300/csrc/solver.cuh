@@ -77,8 +77,9 @@ struct SlotPtrs {
     const double* bnorm_ref;   // if set: ||b|| of the full system (the Schur system's tolerance reference)
 };
 
-enum CounterId { CNT_MATVEC = 0, CNT_UPDATE = 1, CNT_RU = 2, CNT_REPLACE = 3, CNT_START = 4,
-                 CNT_GEMM_V = 5, CNT_GEMM_W = 6, CNT_GROUP = 7, CNT_COUNT = 8 };
+// CNT_BAR and CNT_GEN of slot 0: arrivals and generation of the reliable update's grid barrier.
+enum CounterId { CNT_MATVEC = 0, CNT_UPDATE = 1, CNT_RU = 2, CNT_BAR = 3, CNT_START = 4,
+                 CNT_GEMM_V = 5, CNT_GEMM_W = 6, CNT_GROUP = 7, CNT_GEN = 8, CNT_COUNT = 9 };
 
 // Slot of the current residual r_{j-1} at the start of an iteration.
 __device__ __forceinline__ int cur_slot(const SlotState& st) { return st.m > 0 ? st.vs : 0; }
