@@ -16,6 +16,7 @@ namespace {
 
 constexpr int DS_THREADS = 128;   // operator kernels
 constexpr int BL_THREADS = 256;   // vector kernels
+constexpr int G5_STALL = 200;     // iterations without a reliable update after which the gamma5 variant starts over
 
 inline int div_up(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 
@@ -587,6 +588,12 @@ __global__ void __launch_bounds__(BL_THREADS) update_kernel(SlotState* states, c
             }
             if (st.rnorm_new > st.rmax) st.rmax = st.rnorm_new;
             if (st.delta > 0.0 && (st.rnorm_new < st.delta * st.r_ru || st.rnorm_new < 1e-3 * st.rmax)) st.need_ru = 1;
+            // gamma5 variant with FP32 vectors: its shadow recursion can lose its
+            // biorthogonality for good, which rounding decides (about one deflated solve
+            // in twelve on a near-free 4^4 field, whatever the kernels); a residual that
+            // has not earned a reliable update in G5_STALL iterations starts over from
+            // the true residual with a fresh direction.
+            if (st.g5 && st.delta > 0.0 && st.iter - st.ru_iter >= G5_STALL) st.need_ru = st.fresh_dir = 1;
             if (!st.need_ru) bicg_scalars(st, P);   // else the reliable update ends the iteration
         }
     }

@@ -335,6 +335,7 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
             }
             st.need_ru = 0;
             st.ru_count += 1;
+            st.ru_iter = st.iter + 1;
             st.x_owed = 0;   // the fold added alpha p
             if (st.stab) stab_scalars(st);
             else bicg_scalars(st, P);

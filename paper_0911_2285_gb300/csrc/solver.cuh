@@ -33,6 +33,8 @@ struct SlotState {
     int status;           // SlotStatus
     int need_ru;          // 1: recompute the FP64 residual in this iteration
     int ru_count;
+    int ru_iter;          // iteration of the last reliable update (or the start)
+    int fresh_dir;        // 1: the next direction starts over (beta = 0)
     int restarts;
     int restart_r;        // vectors kept by the restart in this iteration (0 = none)
     int matvecs;

@@ -89,7 +89,8 @@ __device__ __forceinline__ void bicg_scalars(SlotState& st, const SlotPtrs& P) {
         }
         st.vs = k + 1;
     }
-    st.beta = beta;
+    st.beta = st.fresh_dir ? make_double2(0.0, 0.0) : beta;
+    st.fresh_dir = 0;
     st.alpha_prev = st.alpha;
     st.beta_prev = beta;
     st.rho = st.rho_new;
