@@ -66,15 +66,21 @@ __device__ __forceinline__ dfl df_fast_sum(float h, float l) {   // |l| small ag
     const float s = h + l;
     return {s, l - (s - h)};
 }
-// 1/sqrt(a), a.h inside [1e-28, 1e28]: FP32 seed and one third-order step whose
-// residual e = 1 - a y^2 keeps every product's rounding error.
+// 1/sqrt(a), a.h inside [1e-28, 1e28], to about 2^-49: FP32 seed y and one
+// third-order step. e = 1 - a y^2 is kept as an exact part d (1 minus the rounded
+// a.h y^2) and the small rest, and y d/2 with its rounding error: one FP32 number
+// for e would leave 2^-47, which the thousands of rotations of a solve add up.
 __device__ __forceinline__ dfl df_rsqrt(dfl a) {
     const float y = rsqrtf(a.h);
     const float t = y * y, tl = fmaf(y, y, -t);
-    float e = fmaf(-a.h, t, 1.f);
-    e = fmaf(-a.l, t, e);
-    e = fmaf(-a.h, tl, e);
-    return df_fast_sum(y, y * (e * fmaf(0.375f, e, 0.5f)));
+    const float p = a.h * t, pl = fmaf(a.h, t, -p);
+    const float d = 1.f - p;   // exact: p is within 2^-20 of 1
+    const float rest = -fmaf(a.h, tl, fmaf(a.l, t, pl));
+    const float hd = 0.5f * d, m = y * hd, ml = fmaf(y, hd, -m);
+    const float e = d + rest;
+    const float low = fmaf(y, fmaf(0.375f * e, e, 0.5f * rest), ml);
+    const float h = y + m;
+    return df_fast_sum(h, (m - (h - y)) + low);
 }
 // 1/a the same way.
 __device__ __forceinline__ dfl df_rcp(dfl a) {
@@ -111,11 +117,8 @@ struct NumD {
         __device__ __forceinline__ C value() const { return s; }
     };
     static __device__ __forceinline__ R abs2(C a) { return fma(a.y, a.y, a.x * a.x); }
-    static __device__ __forceinline__ R add(R a, R b) { return a + b; }
-    static __device__ __forceinline__ double rvalue(R a) { return a; }
     static __device__ __forceinline__ R rfrom(double a) { return a; }
-    static __device__ __forceinline__ R rzero() { return 0.0; }
-    static __device__ __forceinline__ R shfl_xor(R a, int o) { return __shfl_xor_sync(FULL, a, o); }
+    static __device__ __forceinline__ bool is_zero(C a) { return a.x == 0.0 && a.y == 0.0; }
     static __device__ __forceinline__ bool negligible(C sub, C d0, C d1, double anorm) {
         double t = cabs1(d0) + cabs1(d1);
         if (t == 0.0) t = anorm;
@@ -126,7 +129,7 @@ struct NumD {
     // cy = conj(y)/n, n = sqrt(|x|^2 + |y|^2).
     static __device__ __forceinline__ void givens(C x, C y, C& cx, C& cy) {
         const double n2 = abs2(x) + abs2(y);
-        if (!mid_range(n2) && n2 == 0.0) { cx = one(); cy = zero(); return; }
+        if (!wide_range(n2) && n2 == 0.0) { cx = one(); cy = zero(); return; }
         const double inv = rsqrt_fp64(n2);
         cx = make_double2(inv * x.x, -(inv * x.y));
         cy = make_double2(inv * y.x, -(inv * y.y));
@@ -140,32 +143,18 @@ struct NumF {
     static __device__ __forceinline__ C one() { return {{1.f, 0.f}, {0.f, 0.f}}; }
     static __device__ __forceinline__ C from(double2 a) { return dc_from(a); }
     static __device__ __forceinline__ double2 to(C a) { return dc_to(a); }
-    static __device__ __forceinline__ C lin2(C u, C a, C v, C b) {
-        Dot2 re, im;
-        re.first(u.x, a.x); re.add(-u.y, a.y); re.add(v.x, b.x); re.add(-v.y, b.y);
-        im.first(u.x, a.y); im.add(u.y, a.x); im.add(v.x, b.y); im.add(v.y, b.x);
-        return {re.done(), im.done()};
-    }
+    // Every product and sum normalised: running (s, c) sums would take 30 % fewer
+    // instructions, but cost half a bit in the residuals of the small eigenpairs.
     static __device__ __forceinline__ C mul(C a, C b) {
-        Dot2 re, im;
-        re.first(a.x, b.x); re.add(-a.y, b.y);
-        im.first(a.x, b.y); im.add(a.y, b.x);
-        return {re.done(), im.done()};
+        return {df_mul(a.x, b.x) - df_mul(a.y, b.y), df_mul(a.x, b.y) + df_mul(a.y, b.x)};
     }
-    static __device__ __forceinline__ C fms(C c, C a, C b) {
-        Dot2 re{c.x.h, c.x.l}, im{c.y.h, c.y.l};
-        re.add(-a.x, b.x); re.add(a.y, b.y);
-        im.add(-a.x, b.y); im.add(-a.y, b.x);
-        return {re.done(), im.done()};
-    }
+    static __device__ __forceinline__ C lin2(C u, C a, C v, C b) { return mul(u, a) + mul(v, b); }
+    static __device__ __forceinline__ C fms(C c, C a, C b) { return c - mul(a, b); }
     static __device__ __forceinline__ C scale(R s, C a) { return {df_mul(s, a.x), df_mul(s, a.y)}; }
     struct Sum {
-        Dot2 re{0.f, 0.f}, im{0.f, 0.f};
-        __device__ __forceinline__ void add(C a, C b) {
-            re.add(a.x, b.x); re.add(-a.y, b.y);
-            im.add(a.x, b.y); im.add(a.y, b.x);
-        }
-        __device__ __forceinline__ C value() const { return {re.done(), im.done()}; }
+        C s = {{0.f, 0.f}, {0.f, 0.f}};
+        __device__ __forceinline__ void add(C a, C b) { s = s + mul(a, b); }
+        __device__ __forceinline__ C value() const { return s; }
     };
     static __device__ __forceinline__ R abs2(C a) {
         Dot2 s;
@@ -173,13 +162,8 @@ struct NumF {
         s.add(a.y, a.y);
         return s.done();
     }
-    static __device__ __forceinline__ R add(R a, R b) { return a + b; }
-    static __device__ __forceinline__ double rvalue(R a) { return df_value(a); }
     static __device__ __forceinline__ R rfrom(double a) { return df_split(a); }
-    static __device__ __forceinline__ R rzero() { return {0.f, 0.f}; }
-    static __device__ __forceinline__ R shfl_xor(R a, int o) {
-        return {__shfl_xor_sync(FULL, a.h, o), __shfl_xor_sync(FULL, a.l, o)};
-    }
+    static __device__ __forceinline__ bool is_zero(C a) { return a.x.h == 0.f && a.y.h == 0.f; }
     static constexpr float EPS_DF = 1.4e-14f;   // about four units of double-float rounding
     static __device__ __forceinline__ float abs1(C a) { return fabsf(a.x.h) + fabsf(a.y.h); }
     static __device__ __forceinline__ bool negligible(C sub, C d0, C d1, double anorm) {
@@ -187,18 +171,19 @@ struct NumF {
         if (t == 0.f) t = (float)anorm;
         return abs1(sub) <= EPS_DF * t;
     }
-    static __device__ __forceinline__ double wide_abs2(C a) { return df_value(abs2(a)); }
+    static __device__ __forceinline__ double wide_abs2(C a) { return NumD::abs2(dc_to(a)); }
     static __device__ __forceinline__ void givens(C x, C y, C& cx, C& cy) {
         Dot2 s;
         s.first(x.x, x.x); s.add(x.y, x.y); s.add(y.x, y.x); s.add(y.y, y.y);
         const dfl n2 = s.done();
-        dfl inv;
-        if (df_seed_ok(n2.h)) {
-            inv = df_rsqrt(n2);
-        } else {
-            if (n2.h == 0.f) { cx = one(); cy = zero(); return; }
-            inv = df_split(rsqrt_fp64(df_value(n2)));
+        if (!df_seed_ok(n2.h)) {   // squares near the ends of FP32's range: in FP64
+            double2 dx, dy;
+            NumD::givens(dc_to(x), dc_to(y), dx, dy);
+            cx = dc_from(dx);
+            cy = dc_from(dy);
+            return;
         }
+        const dfl inv = df_rsqrt(n2);
         cx = {df_mul(inv, x.x), -df_mul(inv, x.y)};
         cy = {df_mul(inv, y.x), -df_mul(inv, y.y)};
     }
@@ -305,23 +290,17 @@ __device__ int schur(double2* A64, double2* Q64, int n, int lda, double2* v64, d
     // columns need no work. Warp 0 forms the reflection, a column element per lane.
     for (int k = 0; k + 2 < n; ++k) {
         if (warp == 0) {
-            R nrm2 = M::rzero(), tail = M::rzero();
             int last = k + 1;
-            for (int i = k + 1 + lane; i < n; i += 32) {
-                const R a2 = M::abs2(A[i * lda + k]);
-                nrm2 = M::add(nrm2, a2);
-                if (i >= k + 2) tail = M::add(tail, a2);
-                if (M::rvalue(a2) != 0.0) last = i;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                nrm2 = M::add(nrm2, M::shfl_xor(nrm2, o));
-                tail = M::add(tail, M::shfl_xor(tail, o));
-                last = max(last, __shfl_xor_sync(FULL, last, o));
-            }
-            const bool work = M::rvalue(tail) > 0.0;
+            for (int i = k + 1 + lane; i < n; i += 32)
+                if (!M::is_zero(A[i * lda + k])) last = i;
+            last = __reduce_max_sync(FULL, last);
+            const bool work = last > k + 1;
             if (work) {   // v = x + e^{i theta} ||x|| e1, tau = 2/||v||^2
-                const double alpha = sqrt_fp64(M::rvalue(nrm2));
+                // the norm in FP64: squares of small entries leave FP32's range
+                double nrm2 = 0.0;
+                for (int i = k + 1 + lane; i <= last; i += 32) nrm2 += NumD::abs2(M::to(A[i * lda + k]));
+                nrm2 = warp_sum(nrm2);
+                const double alpha = sqrt_fp64(nrm2);
                 const double2 x0 = M::to(A[(k + 1) * lda + k]);
                 const double a0 = NumD::abs2(x0);
                 double2 ph = cone();

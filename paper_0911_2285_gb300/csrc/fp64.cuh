@@ -22,55 +22,96 @@ __device__ __forceinline__ double exact_f64(float a) {
     return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
 }
 
-// FP32 to FP64, exact (infinities and NaNs kept); subnormals (below 1.2e-38) give
-// zero. Without the conversion instruction even as a rare branch: the compiler
-// would turn the branch into a select and issue it always.
+// FP32 to FP64, exact over FP32's whole range (subnormals scaled up first). Without
+// the conversion instruction even as a rare branch: the compiler would turn the
+// branch into a select and issue it always.
 __device__ __forceinline__ double widen(float a) {
-    const unsigned b = __float_as_uint(a), m = b & 0x7fffffffu;
-    const unsigned up = m >= 0x7f800000u ? (1792u << 20) : (896u << 20);
-    const bool zero = m < 0x00800000u;
+    const unsigned ma = __float_as_uint(a) & 0x7fffffffu;
+    const bool sub = ma < 0x00800000u;
+    const unsigned b = __float_as_uint(sub ? a * 16777216.f : a), m = b & 0x7fffffffu;
+    const unsigned up = ma >= 0x7f800000u ? (1792u << 20) : sub ? (872u << 20) : (896u << 20);
+    const bool zero = m == 0u;
     return __hiloint2double((int)((b & 0x80000000u) | (zero ? 0u : (m >> 3) + up)), zero ? 0 : (int)(b << 29));
 }
-// FP64 to FP32, to nearest (ties away from zero); below 2^-126 zero, from FP32's
-// largest number up infinity, NaN kept.
+// FP64 to FP32, to nearest (ties away from zero; subnormal results rounded twice);
+// from FP32's largest number up infinity, NaN kept.
 __device__ __forceinline__ float narrow(double a) {
     const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a), sign = hi & 0x80000000u;
+    const bool sub = (hi & 0x7fffffffu) < (897u << 20);         // below 2^-126: by way of 2^64 a
     const unsigned l2 = lo + 0x10000000u;                       // half a unit of FP32's last place
-    const unsigned h2 = (hi & 0x7fffffffu) + (l2 < lo ? 1u : 0u);
+    const unsigned h2 = (hi & 0x7fffffffu) + (l2 < lo ? 1u : 0u) + (sub ? (64u << 20) : 0u);
     unsigned r = ((h2 - (896u << 20)) << 3) | (l2 >> 29);
     if (h2 < (897u << 20)) r = 0u;
     if (h2 >= (1151u << 20)) r = 0x7f800000u;
     if ((hi & 0x7fffffffu) + (lo != 0u ? 1u : 0u) > 0x7ff00000u) r = 0x7fffffffu;   // NaN
-    return __uint_as_float(sign | r);
+    return __uint_as_float(sign | r) * (sub ? 5.42101086242752217e-20f : 1.f);
 }
 __device__ __forceinline__ float2 narrow(double2 a) { return make_float2(narrow(a.x), narrow(a.y)); }
 __device__ __forceinline__ double2 widen(float2 a) { return make_double2(widen(a.x), widen(a.y)); }
+// FP64 to storage precision S and back.
+template <typename S> __device__ __forceinline__ cplx<S> nar(double2 a) {
+    if constexpr (sizeof(S) == 4) return narrow(a);
+    else return a;
+}
+__device__ __forceinline__ double2 wid(float2 a) { return widen(a); }
+__device__ __forceinline__ double2 wid(double2 a) { return a; }
 
-// 1/sqrt(a) for a > 0 in FP64: inside FP32's normal range an FP32 reciprocal
+// 2^e with the exponent field f = e + 1023, 0 < f < 2047; a times 2^e by its exponent.
+__device__ __forceinline__ double pow2_field(int f) { return __hiloint2double(f << 20, 0); }
+__device__ __forceinline__ double shift_exp(double a, int e) {
+    return __hiloint2double(__double2hiint(a) + e * (1 << 20), __double2loint(a));
+}
+// a positive with an exponent that the routines below may move by half or negate.
+__device__ __forceinline__ bool wide_range(double a) { return ((unsigned)__double2hiint(a) >> 20) - 64u < 1918u; }
+
+// 1/sqrt(a) for a > 0 in FP64: a scaled by 4^k into [1, 4), an FP32 reciprocal
 // square root y (relative error about 2^-21) and one step of third order: with
-// e = 1 - a y^2, 1/sqrt(a) = y (1 + e/2 + 3 e^2/8 + O(e^3)). Outside: 1 / sqrt(a).
+// e = 1 - a y^2, 1/sqrt(a) = y (1 + e/2 + 3 e^2/8 + O(e^3)). Near the ends of
+// FP64's range: 1 / sqrt(a).
 __device__ __forceinline__ double rsqrt_fp64(double a) {
-    if (!mid_range(a)) return 1.0 / sqrt(a);
-    const double y = exact_f64(rsqrtf(seed_f32(a)));
-    const double e = fma(-(a * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
+    if (!wide_range(a)) return 1.0 / sqrt(a);
+    const int k = ((__double2hiint(a) >> 20) - 1023) & ~1;
+    const double m = shift_exp(a, -k);
+    const double y = exact_f64(rsqrtf(seed_f32(m)));
+    const double e = fma(-(m * y), y, 1.0);
+    return shift_exp(fma(y * e, fma(0.375, e, 0.5), y), -(k / 2));
 }
 
-// 1/a in FP64 the same way: FP32 reciprocal seed y, e = 1 - a y,
-// 1/a = y (1 + e + e^2 + O(e^3)). Outside FP32's normal range: 1 / a.
+// 1/a in FP64 the same way: mantissa in [1, 2), FP32 reciprocal seed y, e = 1 - a y,
+// 1/a = y (1 + e + e^2 + O(e^3)).
 __device__ __forceinline__ double rcp_fp64(double a) {
-    const double m = fabs(a);
-    if (!mid_range(m)) return 1.0 / a;
-    const double y = copysign(exact_f64(__frcp_rn(seed_f32(m))), a);
-    const double e = fma(-a, y, 1.0);
-    return fma(y * e, 1.0 + e, y);
+    const double p = fabs(a);
+    if (!wide_range(p)) return 1.0 / a;
+    const int k = (__double2hiint(p) >> 20) - 1023;
+    const double m = shift_exp(p, -k);
+    const double y = exact_f64(__frcp_rn(seed_f32(m)));
+    const double e = fma(-m, y, 1.0);
+    return copysign(shift_exp(fma(y * e, 1.0 + e, y), -k), a);
 }
 
 // sqrt(a) for a >= 0: a / sqrt(a) and one correction of the product's rounding.
 __device__ __forceinline__ double sqrt_fp64(double a) {
-    if (!mid_range(a)) return sqrt(a);
+    if (!wide_range(a)) return sqrt(a);
     const double r = rsqrt_fp64(a), s = a * r;
     return fma(0.5 * r, fma(-s, s, a), s);
+}
+
+// a / b: the larger part of b scaled to [1, 2), one reciprocal of |b|^2 (Smith's
+// division takes three dependent FP64 divisions). Near the ends of the range: Smith.
+__device__ __forceinline__ double2 cdiv_fp64(double2 a, double2 b) {
+    const int f = max(__double2hiint(b.x) & 0x7ff00000, __double2hiint(b.y) & 0x7ff00000) >> 20;
+    if (f < 64 || f > 1982) return cdiv(a, b);
+    const double up = pow2_field(2046 - f);   // 2^(1023 - f)
+    const double2 s = make_double2(up * b.x, up * b.y);
+    const double r = rcp_fp64(fma(s.y, s.y, s.x * s.x)) * up;
+    const double2 t = make_double2(r * s.x, -(r * s.y));
+    return make_double2(fma(-a.y, t.y, a.x * t.x), fma(a.y, t.x, a.x * t.y));
+}
+
+// |z| >= tol s1 s2 (s1, s2 >= 0), without the square root of |z|; false for NaN.
+__device__ __forceinline__ bool abs_at_least(double2 z, double tol, double s1, double s2) {
+    const double t = tol * s1 * s2;
+    return fma(z.y, z.y, z.x * z.x) >= t * t && !(z.x == 0.0 && z.y == 0.0 && t > 0.0);
 }
 
 }  // namespace lqcd
