@@ -51,6 +51,28 @@ template <typename C> __host__ __device__ __forceinline__ C cdot(C a, C b) {
 template <typename C> __host__ __device__ __forceinline__ C mulc(C a, C b) {
     C r; r.x = a.x * b.x + a.y * b.y; r.y = a.y * b.x - a.x * b.y; return r;
 }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+// c + a b, c - a b, c + conj(a) b, c + |a|^2. In FP64, whose pipe bounds the kernels
+// that use them, as four (two) multiply-adds; a product followed by a sum takes six
+// (three) instructions. FP32 kernels are bound by memory and keep the plain form.
+__device__ __forceinline__ float2 cfma(float2 c, float2 a, float2 b) { return c + a * b; }
+__device__ __forceinline__ float2 cfms(float2 c, float2 a, float2 b) { return c - a * b; }
+__device__ __forceinline__ float2 cdot_acc(float2 c, float2 a, float2 b) { return c + cdot(a, b); }
+__device__ __forceinline__ float abs2_acc(float c, float2 a) { return c + (a.x * a.x + a.y * a.y); }
+__device__ __forceinline__ double2 cfma(double2 c, double2 a, double2 b) {
+    return make_double2(fma(-a.y, b.y, fma(a.x, b.x, c.x)), fma(a.y, b.x, fma(a.x, b.y, c.y)));
+}
+__device__ __forceinline__ double2 cfms(double2 c, double2 a, double2 b) {
+    return make_double2(fma(a.y, b.y, fma(-a.x, b.x, c.x)), fma(-a.y, b.x, fma(-a.x, b.y, c.y)));
+}
+__device__ __forceinline__ double2 cdot_acc(double2 c, double2 a, double2 b) {
+    return make_double2(fma(a.y, b.y, fma(a.x, b.x, c.x)), fma(-a.y, b.x, fma(a.x, b.y, c.y)));
+}
+__device__ __forceinline__ double abs2_acc(double c, double2 a) { return fma(a.y, a.y, fma(a.x, a.x, c)); }
+// c + |a|^2 + |b|^2
+__device__ __forceinline__ float abs2_two(float c, float2 a, float2 b) { return c + ((a.x * a.x + a.y * a.y) + (b.x * b.x + b.y * b.y)); }
+__device__ __forceinline__ double abs2_two(double c, double2 a, double2 b) { return abs2_acc(abs2_acc(c, a), b); }
 __host__ __device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 __host__ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
     // Smith's algorithm for a / b.

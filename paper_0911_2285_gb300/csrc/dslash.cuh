@@ -74,8 +74,9 @@ __device__ __forceinline__ void project(const C (&psi)[12], C (&h)[2][3]) {
     }
 }
 
-// acc += (uh, sg M_mu^+ uh)
-template <int MU, int SG, typename C>
+// acc += (uh, sg M_mu^+ uh); SET: acc = instead (24 FP64 additions to zero less in
+// kernels that the FP64 pipe bounds).
+template <int MU, int SG, bool SET = false, typename C>
 __device__ __forceinline__ void reconstruct(const C (&uh)[2][3], C (&acc)[12]) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -85,6 +86,13 @@ __device__ __forceinline__ void reconstruct(const C (&uh)[2][3], C (&acc)[12]) {
         else if (MU == 1) { l0 = b; l1 = -a; }
         else if (MU == 2) { l0 = mul_i(a); l1 = mul_mi(b); }
         else { l0 = a; l1 = b; }
+        if (SET) {
+            acc[c] = a;
+            acc[3 + c] = b;
+            acc[6 + c] = SG > 0 ? l0 : -l0;
+            acc[9 + c] = SG > 0 ? l1 : -l1;
+            continue;
+        }
         acc[c] = acc[c] + a;
         acc[3 + c] = acc[3 + c] + b;
         if (SG > 0) { acc[6 + c] = acc[6 + c] + l0; acc[9 + c] = acc[9 + c] + l1; }
@@ -94,9 +102,6 @@ __device__ __forceinline__ void reconstruct(const C (&uh)[2][3], C (&acc)[12]) {
 
 // Fused multiply-add chains (one rounding per term, no separate product and
 // sum instructions): o = u h and o = u^+ h for the two spin rows of h.
-__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
-
 template <typename C>
 __device__ __forceinline__ void su3_mul(const C (&u)[3][3], const C (&h)[2][3], C (&o)[2][3]) {
 #pragma unroll
@@ -172,7 +177,7 @@ __device__ __forceinline__ void hop_dir(const Nbr& nb, const LK& U, const IN& in
         project<MU, SF>(psi, h);
         U.load(MU, s, u);
         su3_mul(u, h, uh);
-        reconstruct<MU, SF>(uh, acc);
+        reconstruct<MU, SF, MU == 0 && sizeof(T) == 8>(uh, acc);
     }
     {
         int sb = nb.b[MU];

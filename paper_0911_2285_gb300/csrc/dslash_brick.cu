@@ -27,7 +27,6 @@ namespace lqcd {
 namespace {
 
 constexpr int BR_THREADS = 256;
-constexpr double BR_BREAK_TOL = 1e-14;
 
 __device__ __forceinline__ void stcs4(void* base, size_t i, float4 v) {
     __stcs(reinterpret_cast<float4*>(base) + i, v);
@@ -235,15 +234,7 @@ __global__ void __launch_bounds__(BR_THREADS, MINB)
         z = warp_sum(z);
         ab = warp_sum(ab);
         if (lane == 0) {
-            st.sigma = z;
-            st.phat_norm = sqrt(ab.x);
-            st.ap_norm = sqrt(ab.y);
-            st.matvecs += 2;
-            if (!(cabs_(st.sigma) >= BR_BREAK_TOL * st.phat_norm * st.ap_norm) || cabs2(st.sigma) == 0.0) {
-                st.status = ST_BREAKDOWN;
-            } else {
-                st.alpha = cdiv(st.rho, st.sigma);
-            }
+            finish_sigma(st, z, ab.x, ab.y, 2);
         }
     }
 }

@@ -38,7 +38,6 @@ namespace lqcd {
 namespace {
 
 constexpr int SG_THREADS = 256;   // one thread per site of the brick
-constexpr double SG_BREAK_TOL = 1e-14;
 
 __device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* tmap, int c0, int c1, int c2, int c3,
                                             int c4, uint64_t* bar) {
@@ -342,15 +341,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         z = warp_sum(z);
         ab = warp_sum(ab);
         if (lane == 0) {
-            st.sigma = z;
-            st.phat_norm = sqrt(ab.x);
-            st.ap_norm = sqrt(ab.y);
-            st.matvecs += 2;
-            if (!(cabs_(st.sigma) >= SG_BREAK_TOL * st.phat_norm * st.ap_norm) || cabs2(st.sigma) == 0.0) {
-                st.status = ST_BREAKDOWN;
-            } else {
-                st.alpha = cdiv(st.rho, st.sigma);
-            }
+            finish_sigma(st, z, ab.x, ab.y, 2);
         }
     }
 }

@@ -224,15 +224,7 @@ __global__ void __launch_bounds__(TILE_MAX_THREADS, 1)
     const unsigned nblk = (unsigned)(tg.nyb * Lz * tg.nseg);
     const unsigned myblk = (unsigned)(yb + tg.nyb * (z + Lz * seg));
     if (reduce_slot<2>(P, CNT_MATVEC, v, tot, nblk, myblk) && threadIdx.x == 0) {
-        st.sigma = tot[0];
-        st.phat_norm = sqrt(tot[1].x);
-        st.ap_norm = sqrt(tot[1].y);
-        st.matvecs += 2;
-        if (!(cabs_(st.sigma) >= 1e-14 * st.phat_norm * st.ap_norm) || cabs2(st.sigma) == 0.0) {
-            st.status = ST_BREAKDOWN;
-        } else {
-            st.alpha = cdiv(st.rho, st.sigma);
-        }
+        finish_sigma(st, tot[0], tot[1].x, tot[1].y, 2);
     }
 }
 

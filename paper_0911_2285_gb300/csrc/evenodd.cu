@@ -20,7 +20,6 @@ namespace lqcd {
 namespace {
 
 constexpr int EO_THREADS = 128;
-constexpr double EO_BREAK_TOL = 1e-14;
 
 int eo_blocks(int Vh) {
     int nb = (Vh + EO_THREADS - 1) / EO_THREADS;
@@ -206,9 +205,9 @@ __global__ void __launch_bounds__(THREADS, MINB) eo_pair2_kernel(Geom g, const v
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
             b[c] = self[c] - k2 * b[c];
-            sacc.z = sacc.z + cdot(self[c], a[c]);
-            sacc.a += abs2(self[c]);
-            sacc.b += abs2(a[c]);
+            sacc.z = cdot_acc(sacc.z, self[c], a[c]);
+            sacc.a = abs2_acc(sacc.a, self[c]);
+            sacc.b = abs2_acc(sacc.b, a[c]);
         }
         Field<S>::store(P.Ahp[par], Vh, h, b);
     }
@@ -216,14 +215,7 @@ __global__ void __launch_bounds__(THREADS, MINB) eo_pair2_kernel(Geom g, const v
     sacc.to(v);
     double2 tot[2];
     if (reduce_slot<2>(P, CNT_MATVEC, v, tot, nsb, sblock) && threadIdx.x == 0) {
-        st.sigma = tot[0];
-        st.phat_norm = sqrt(tot[1].x);
-        st.ap_norm = sqrt(tot[1].y);
-        st.matvecs += 2;
-        if (!(cabs_(st.sigma) >= EO_BREAK_TOL * st.phat_norm * st.ap_norm) || cabs2(st.sigma) == 0.0)
-            st.status = ST_BREAKDOWN;
-        else
-            st.alpha = cdiv(st.rho, st.sigma);
+        finish_sigma(st, tot[0], tot[1].x, tot[1].y, 2);
     }
 }
 

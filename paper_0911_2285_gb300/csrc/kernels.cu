@@ -20,6 +20,13 @@ constexpr int G5_STALL = 200;     // iterations without a reliable update after 
 
 inline int div_up(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 
+// Threads per block of the FP64 site and vector kernels: the FP64 pipe of an SM serves
+// 2 lanes per clock, so what matters is how many SMs take part. Below two blocks of
+// the full size per SM, one-warp blocks spread the same warps over the chip: operator
+// pair on 4^4 (16 warps) 42 us on 4 SMs.
+constexpr int SMALL_GRID = 2 * 152;
+int site_threads(size_t sites, int jobs, int full) { return (sites + full - 1) / full * jobs < SMALL_GRID ? 32 : full; }
+
 int blas_blocks(size_t units) {
     int nb = div_up(units, BL_THREADS);
     if (nb > 1216) nb = 1216;   // 8 blocks of 256 per SM on 152 SMs
@@ -257,7 +264,7 @@ __global__ void __launch_bounds__(BL_THREADS) start_kernel(SlotState* states, co
     for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < units; u += (size_t)gridDim.x * blockDim.x) {
         Unit<double> rt = Unit<double>::load(P.r_true, u);
         Unit<double> bb = Unit<double>::load(P.b, u);
-        Unit<S> r{cvt<S>(rt.a), cvt<S>(rt.b)};
+        Unit<S> r{nar<S>(rt.a), nar<S>(rt.b)};
         r.store(P.V, u);
         r.store(P.p, u);
         Unit<S> h = r;
@@ -272,16 +279,16 @@ __global__ void __launch_bounds__(BL_THREADS) start_kernel(SlotState* states, co
         if (comp) {
             if constexpr (sizeof(S) == 4) { cz.add(cdot(h.a, r.a)); cz.add(cdot(h.b, r.b)); }
         } else {
-            acc.z = acc.z + cdot(h.a, r.a) + cdot(h.b, r.b);
+            acc.z = cdot_acc(cdot_acc(acc.z, h.a, r.a), h.b, r.b);
         }
-        acc.a += abs2(r.a) + abs2(r.b);
+        acc.a = abs2_two(acc.a, r.a, r.b);
         acc.b += (S)(cabs2(bb.a) + cabs2(bb.b));
     }
     double2 tot[2];
     if (reduce2<S>(P, CNT_START, comp, cz, acc, tot, gridDim.x, blockIdx.x) && threadIdx.x == 0) {
         st.rho = tot[0];
-        st.rnorm = sqrt(tot[1].x);
-        st.bnorm = P.bnorm_ref ? *P.bnorm_ref : sqrt(tot[1].y);   // even-odd: ||b|| of the full system
+        st.rnorm = sqrt_fp64(tot[1].x);
+        st.bnorm = P.bnorm_ref ? *P.bnorm_ref : sqrt_fp64(tot[1].y);   // even-odd: ||b|| of the full system
         st.rhat_norm = st.rnorm;
         st.rmax = st.rnorm;
         st.r_ru = st.rnorm;
@@ -292,7 +299,7 @@ __global__ void __launch_bounds__(BL_THREADS) start_kernel(SlotState* states, co
         if (st.rnorm <= st.tol * st.bnorm) { st.status = ST_CONVERGED; st.live = 0; }
         // rho_0 = (rhat_0, r_0) must not vanish (e.g. the gamma5 shadow start on a
         // source whose upper and lower spin halves have equal norms)
-        else if (!(cabs_(st.rho) >= BREAK_TOL * st.rhat_norm * st.rnorm)) { st.status = ST_BREAKDOWN; st.live = 0; }
+        else if (!abs_at_least(st.rho, BREAK_TOL, st.rhat_norm, st.rnorm)) { st.status = ST_BREAKDOWN; st.live = 0; }
     }
     (void)sizeof(C);
 }
@@ -370,9 +377,9 @@ __global__ void __launch_bounds__(THREADS, MINB) matvec_kernel(Geom g, const voi
 #pragma unroll
             for (int c = 0; c < 12; ++c) {
                 b[c] = self[c] - k * b[c];
-                sacc.z = sacc.z + cdot(self[c], a[c]);
-                sacc.a += abs2(self[c]);
-                sacc.b += abs2(a[c]);
+                sacc.z = cdot_acc(sacc.z, self[c], a[c]);
+                sacc.a = abs2_acc(sacc.a, self[c]);
+                sacc.b = abs2_acc(sacc.b, a[c]);
             }
             Field<S>::store(P.Ahp[par], g.V, s, b);
         }
@@ -396,9 +403,9 @@ __global__ void __launch_bounds__(THREADS, MINB) matvec_kernel(Geom g, const voi
                 for (int c = 0; c < 12; ++c) {
                     const C ph = c < 6 ? self_p[c] : -self_p[c];
                     if constexpr (sizeof(S) == 4) scomp.add(cdot(ph, acc[c]));
-                    else sacc.z = sacc.z + cdot(ph, acc[c]);
-                    sacc.a += abs2(ph);
-                    sacc.b += abs2(acc[c]);
+                    else sacc.z = cdot_acc(sacc.z, ph, acc[c]);
+                    sacc.a = abs2_acc(sacc.a, ph);
+                    sacc.b = abs2_acc(sacc.b, acc[c]);
                 }
                 if (win) {
 #pragma unroll
@@ -410,9 +417,9 @@ __global__ void __launch_bounds__(THREADS, MINB) matvec_kernel(Geom g, const voi
                 Field<S>::load(P.phat, g.V, s, ph);
 #pragma unroll
                 for (int c = 0; c < 12; ++c) {
-                    sacc.z = sacc.z + cdot(ph[c], acc[c]);
-                    sacc.a += abs2(ph[c]);
-                    sacc.b += abs2(acc[c]);
+                    sacc.z = cdot_acc(sacc.z, ph[c], acc[c]);
+                    sacc.a = abs2_acc(sacc.a, ph[c]);
+                    sacc.b = abs2_acc(sacc.b, acc[c]);
                 }
             }
         }
@@ -420,15 +427,7 @@ __global__ void __launch_bounds__(THREADS, MINB) matvec_kernel(Geom g, const voi
     }
     double2 tot[2];
     if (reduce2<S>(P, CNT_MATVEC, G5 && sizeof(S) == 4, scomp, sacc, tot, nsb, sblock) && threadIdx.x == 0) {
-        st.sigma = tot[0];
-        st.phat_norm = sqrt(tot[1].x);
-        st.ap_norm = sqrt(tot[1].y);
-        st.matvecs += G5 ? 1 : 2;   // the gamma5 variant applies A only
-        if (!(cabs_(st.sigma) >= BREAK_TOL * st.phat_norm * st.ap_norm) || cabs2(st.sigma) == 0.0) {
-            st.status = ST_BREAKDOWN;
-        } else {
-            st.alpha = cdiv(st.rho, st.sigma);
-        }
+        finish_sigma(st, tot[0], tot[1].x, tot[1].y, G5 ? 1 : 2);   // the gamma5 variant applies A only
     }
 }
 
@@ -473,9 +472,9 @@ __global__ void __launch_bounds__(32 * JPB, MINB)
                 Field<float>::load(P.phat, g.V, s, ph);
 #pragma unroll
                 for (int c = 0; c < 12; ++c) {
-                    sacc.z = sacc.z + cdot(ph[c], acc[c]);
-                    sacc.a += abs2(ph[c]);
-                    sacc.b += abs2(acc[c]);
+                    sacc.z = cdot_acc(sacc.z, ph[c], acc[c]);
+                    sacc.a = abs2_acc(sacc.a, ph[c]);
+                    sacc.b = abs2_acc(sacc.b, acc[c]);
                 }
             }
         }
@@ -504,15 +503,7 @@ __global__ void __launch_bounds__(32 * JPB, MINB)
         z = warp_sum(z);
         ab = warp_sum(ab);
         if (lane == 0) {
-            st.sigma = z;
-            st.phat_norm = sqrt(ab.x);
-            st.ap_norm = sqrt(ab.y);
-            st.matvecs += 2;
-            if (!(cabs_(st.sigma) >= BREAK_TOL * st.phat_norm * st.ap_norm) || cabs2(st.sigma) == 0.0) {
-                st.status = ST_BREAKDOWN;
-            } else {
-                st.alpha = cdiv(st.rho, st.sigma);
-            }
+            finish_sigma(st, z, ab.x, ab.y, 2);
         }
     }
 }
@@ -543,12 +534,12 @@ __global__ void __launch_bounds__(BL_THREADS) update_kernel(SlotState* states, c
         const bool win = st.m > 0;
         for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < units; u += (size_t)gridDim.x * blockDim.x) {
             Unit<S> r = Unit<S>::load(rin, u), a = Unit<S>::load(ap, u);
-            r.a = r.a - al * a.a; r.b = r.b - al * a.b;
+            r.a = cfms(r.a, al, a.a); r.b = cfms(r.b, al, a.b);
             r.store(rout, u);
             const Unit<S> h = g5u(r, u, N);
             if (win) h.store(hout, u);
             if constexpr (sizeof(S) == 4) { cz.add(cdot(h.a, r.a)); cz.add(cdot(h.b, r.b)); }
-            else acc.z = acc.z + cdot(h.a, r.a) + cdot(h.b, r.b);
+            else acc.z = cdot_acc(cdot_acc(acc.z, h.a, r.a), h.b, r.b);
             acc.a += abs2(r.a) + abs2(r.b);
         }
         acc.b = acc.a;
@@ -556,20 +547,20 @@ __global__ void __launch_bounds__(BL_THREADS) update_kernel(SlotState* states, c
         for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < units; u += (size_t)gridDim.x * blockDim.x) {
             Unit<S> r = Unit<S>::load(rin, u), a = Unit<S>::load(ap, u);
             Unit<S> h = Unit<S>::load(hin, u), ah = Unit<S>::load(ahp, u);
-            r.a = r.a - al * a.a; r.b = r.b - al * a.b;
-            h.a = h.a - alc * ah.a; h.b = h.b - alc * ah.b;
+            r.a = cfms(r.a, al, a.a); r.b = cfms(r.b, al, a.b);
+            h.a = cfms(h.a, alc, ah.a); h.b = cfms(h.b, alc, ah.b);
             r.store(rout, u);
             h.store(hout, u);
-            acc.z = acc.z + cdot(h.a, r.a) + cdot(h.b, r.b);
-            acc.a += abs2(r.a) + abs2(r.b);
-            acc.b += abs2(h.a) + abs2(h.b);
+            acc.z = cdot_acc(cdot_acc(acc.z, h.a, r.a), h.b, r.b);
+            acc.a = abs2_two(acc.a, r.a, r.b);
+            acc.b = abs2_two(acc.b, h.a, h.b);
         }
     }
     double2 tot[2];
     if (reduce2<S>(P, CNT_UPDATE, comp, cz, acc, tot, gridDim.x, blockIdx.x) && threadIdx.x == 0) {
         st.rho_new = tot[0];
-        st.rnorm_new = sqrt(tot[1].x);
-        st.rhat_norm = sqrt(tot[1].y);
+        st.rnorm_new = sqrt_fp64(tot[1].x);
+        st.rhat_norm = sqrt_fp64(tot[1].y);
         st.x_owed = 1;
         if (!isfinite(st.rnorm_new) || !isfinite(st.rho_new.x) || !isfinite(st.rho_new.y)) {
             st.status = ST_BREAKDOWN;
@@ -617,14 +608,14 @@ __global__ void __launch_bounds__(THREADS, MINB) true_resid_kernel(Geom g, const
         Field<double>::load(P.b, g.V, s, b);
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
-            acc[c] = b[c] - (self[c] - kappa * acc[c]);
-            v[0].x += cabs2(acc[c]);
+            acc[c] = b[c] - make_double2(fma(-kappa, acc[c].x, self[c].x), fma(-kappa, acc[c].y, self[c].y));
+            v[0].x = abs2_acc(v[0].x, acc[c]);
         }
         Field<double>::store(P.r_true, g.V, s, acc);
     }
     double2 tot[1];
     if (reduce_slot<1>(P, CNT_RU, v, tot, gridDim.x, blockIdx.x) && threadIdx.x == 0) {
-        st.true_rnorm = sqrt(tot[0].x);
+        st.true_rnorm = sqrt_fp64(tot[0].x);
         st.matvecs += 1;
     }
 }
@@ -648,13 +639,13 @@ __global__ void __launch_bounds__(BL_THREADS) direction_kernel(SlotState* states
         if (!g5) { ph = Unit<S>::load(P.phat, u); hh = Unit<S>::load(h, u); }
         if (addx) {   // x_lo += alpha p_{j-1} (owed by the residual update)
             Unit<S> x = Unit<S>::load(P.x_lo, u);
-            x.a = x.a + al * p.a; x.b = x.b + al * p.b;
+            x.a = cfma(x.a, al, p.a); x.b = cfma(x.b, al, p.b);
             x.store(P.x_lo, u);
         }
-        p.a = rr.a + be * p.a; p.b = rr.b + be * p.b;
+        p.a = cfma(rr.a, be, p.a); p.b = cfma(rr.b, be, p.b);
         p.store(P.p, u);
         if (!g5) {
-            ph.a = hh.a + bec * ph.a; ph.b = hh.b + bec * ph.b;
+            ph.a = cfma(hh.a, bec, ph.a); ph.b = cfma(hh.b, bec, ph.b);
             ph.store(P.phat, u);
         }
     }
@@ -683,8 +674,8 @@ __global__ void __launch_bounds__(BL_THREADS) stab_dir_kernel(SlotState* states,
         Unit<S> r = Unit<S>::load(P.V, u);
         if (!first) {
             const Unit<S> p = Unit<S>::load(P.p, u), v = Unit<S>::load(P.Ap[0], u);
-            r.a = r.a + be * (p.a - om * v.a);
-            r.b = r.b + be * (p.b - om * v.b);
+            r.a = cfma(r.a, be, cfms(p.a, om, v.a));
+            r.b = cfma(r.b, be, cfms(p.b, om, v.b));
         }
         r.store(P.p, u);
     }
@@ -719,16 +710,16 @@ __global__ void __launch_bounds__(THREADS, MINB) stab_matvec_kernel(Geom g, cons
             Field<S>::load(P.W, g.V, s, h);
 #pragma unroll
             for (int c = 0; c < 12; ++c) {
-                acc.z = acc.z + cdot(h[c], o[c]);
-                acc.a += abs2(h[c]);
-                acc.b += abs2(o[c]);
+                acc.z = cdot_acc(acc.z, h[c], o[c]);
+                acc.a = abs2_acc(acc.a, h[c]);
+                acc.b = abs2_acc(acc.b, o[c]);
             }
         } else {
 #pragma unroll
             for (int c = 0; c < 12; ++c) {
-                acc.z = acc.z + cdot(o[c], self[c]);
-                acc.a += abs2(o[c]);
-                acc.b += abs2(self[c]);
+                acc.z = cdot_acc(acc.z, o[c], self[c]);
+                acc.a = abs2_acc(acc.a, o[c]);
+                acc.b = abs2_acc(acc.b, self[c]);
             }
         }
     }
@@ -736,19 +727,13 @@ __global__ void __launch_bounds__(THREADS, MINB) stab_matvec_kernel(Geom g, cons
     acc.to(v);
     double2 tot[2];
     if (reduce_slot<2>(P, CNT_MATVEC, v, tot, nsb, sblock) && threadIdx.x == 0) {
-        st.matvecs += 1;
         if (PHASE == 1) {
-            st.sigma = tot[0];
-            st.phat_norm = sqrt(tot[1].x);
-            st.ap_norm = sqrt(tot[1].y);
-            if (!(cabs_(st.sigma) >= BREAK_TOL * st.phat_norm * st.ap_norm) || cabs2(st.sigma) == 0.0)
-                st.status = ST_BREAKDOWN;
-            else
-                st.alpha = cdiv(st.rho, st.sigma);
+            finish_sigma(st, tot[0], tot[1].x, tot[1].y, 1);
         } else {
+            st.matvecs += 1;
             st.ts = tot[0];
             st.tt = tot[1].x;
-            st.omega = st.tt > 0.0 ? cdiv(st.ts, make_double2(st.tt, 0.0)) : make_double2(0.0, 0.0);
+            st.omega = st.tt > 0.0 ? rcp_fp64(st.tt) * st.ts : make_double2(0.0, 0.0);
         }
     }
 }
@@ -764,8 +749,8 @@ __global__ void __launch_bounds__(BL_THREADS) stab_s_kernel(SlotState* states, c
     for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < units; u += (size_t)gridDim.x * blockDim.x) {
         Unit<S> r = Unit<S>::load(P.V, u);
         const Unit<S> v = Unit<S>::load(P.Ap[0], u);
-        r.a = r.a - al * v.a;
-        r.b = r.b - al * v.b;
+        r.a = cfms(r.a, al, v.a);
+        r.b = cfms(r.b, al, v.b);
         r.store(P.phat, u);
     }
 }
@@ -785,20 +770,20 @@ __global__ void __launch_bounds__(BL_THREADS) stab_update_kernel(SlotState* stat
         Unit<S> x = Unit<S>::load(P.x_lo, u);
         const Unit<S> p = Unit<S>::load(P.p, u), sv = Unit<S>::load(P.phat, u), t = Unit<S>::load(P.Ahp[0], u);
         const Unit<S> h = Unit<S>::load(P.W, u);
-        x.a = x.a + al * p.a + om * sv.a;
-        x.b = x.b + al * p.b + om * sv.b;
+        x.a = cfma(cfma(x.a, al, p.a), om, sv.a);
+        x.b = cfma(cfma(x.b, al, p.b), om, sv.b);
         x.store(P.x_lo, u);
-        Unit<S> r{sv.a - om * t.a, sv.b - om * t.b};
+        Unit<S> r{cfms(sv.a, om, t.a), cfms(sv.b, om, t.b)};
         r.store(P.V, u);
-        acc.z = acc.z + cdot(h.a, r.a) + cdot(h.b, r.b);
-        acc.a += abs2(r.a) + abs2(r.b);
+        acc.z = cdot_acc(cdot_acc(acc.z, h.a, r.a), h.b, r.b);
+        acc.a = abs2_two(acc.a, r.a, r.b);
     }
     cplx<S> v[2];
     acc.to(v);
     double2 tot[2];
     if (reduce_slot<2>(P, CNT_UPDATE, v, tot, gridDim.x, blockIdx.x) && threadIdx.x == 0) {
         st.rho_new = tot[0];
-        st.rnorm_new = sqrt(tot[1].x);
+        st.rnorm_new = sqrt_fp64(tot[1].x);
         st.x_owed = 0;   // x is complete after this step
         if (!isfinite(st.rnorm_new) || !isfinite(st.rho_new.x) || !isfinite(st.rho_new.y)) {
             st.status = ST_BREAKDOWN;
@@ -827,10 +812,10 @@ __global__ void fold_kernel(SlotState* states, const SlotPtrs* ptrs, size_t N) {
         Unit<S> xl = Unit<S>::load(P.x_lo, u);
         if (owed) {
             const Unit<S> p = Unit<S>::load(P.p, u);
-            xl.a = xl.a + al * p.a; xl.b = xl.b + al * p.b;
+            xl.a = cfma(xl.a, al, p.a); xl.b = cfma(xl.b, al, p.b);
         }
         if (zero_src) { xh.a = make_double2(0, 0); xh.b = make_double2(0, 0); }
-        else { xh.a = xh.a + to_d(xl.a); xh.b = xh.b + to_d(xl.b); }
+        else { xh.a = xh.a + wid(xl.a); xh.b = xh.b + wid(xl.b); }
         xh.store(P.x_hi, u);
         zero.store(P.x_lo, u);
     }
@@ -1001,10 +986,12 @@ void set_launches(long long n) { g_launches = n; }
 
 cudaError_t launch_apply(const Geom& g, const void* links, double kappa, int precision, const ApplyJob* d_jobs,
                          int njobs, int residual, cudaStream_t st) {
-    const int grid = ds_blocks(g.V) * njobs;   // jobs fastest: they share each block's links
+    int grid = ds_blocks(g.V) * njobs;   // jobs fastest: they share each block's links
     if (precision == 0) {
-        if (residual) apply_kernel<double, true><<<grid, DS_THREADS, 0, st>>>(geom_of(g), links, kappa, d_jobs, njobs);
-        else apply_kernel<double, false><<<grid, DS_THREADS, 0, st>>>(geom_of(g), links, kappa, d_jobs, njobs);
+        const int t = site_threads(g.V, njobs, DS_THREADS);
+        if (t == 32) grid = div_up(g.V, 32) * njobs;
+        if (residual) apply_kernel<double, true><<<grid, t, 0, st>>>(geom_of(g), links, kappa, d_jobs, njobs);
+        else apply_kernel<double, false><<<grid, t, 0, st>>>(geom_of(g), links, kappa, d_jobs, njobs);
     } else {
         if (residual) return cudaErrorInvalidValue;
         apply_kernel<float, false><<<grid, DS_THREADS, 0, st>>>(geom_of(g), links, kappa, d_jobs, njobs);
@@ -1167,7 +1154,8 @@ cudaError_t launch_bicg_matvec(const Geom& g, const void* links, double kappa, i
     if (prec != 0 && variant >= 25 && variant < 30)   // 4-D bricks, every slot per block (dslash_brick.cu)
         return launch_matvec_brick(g, links, kappa, states, ptrs, nslots, s, variant);
     if (prec == 0) {
-        matvec_launch<double, 128, 1, false>(g, links, kappa, states, ptrs, nslots, s);
+        if (site_threads(g.V, 2 * nslots, 128) == 32) matvec_launch<double, 32, 8, false>(g, links, kappa, states, ptrs, nslots, s);
+        else matvec_launch<double, 128, 1, false>(g, links, kappa, states, ptrs, nslots, s);
     } else {
         switch (variant) {
             case 1: matvec_launch<float, 128, 6, false>(g, links, kappa, states, ptrs, nslots, s); break;
@@ -1215,7 +1203,8 @@ bool matvec_g5_variant_ok(const Geom& g, int v) {
 cudaError_t launch_bicg_matvec_g5(const Geom& g, const void* links, double kappa, int prec, SlotState* states,
                                   const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant) {
     if (prec == 0) {
-        matvec_launch<double, 128, 1, false, 0, 1, true>(g, links, kappa, states, ptrs, nslots, s);
+        if (site_threads(g.V, nslots, 128) == 32) matvec_launch<double, 32, 8, false, 0, 1, true>(g, links, kappa, states, ptrs, nslots, s);
+        else matvec_launch<double, 128, 1, false, 0, 1, true>(g, links, kappa, states, ptrs, nslots, s);
     } else {
         switch (variant) {
             case 1: matvec_launch<float, 128, 6, false, 0, 1, true>(g, links, kappa, states, ptrs, nslots, s); break;
@@ -1236,7 +1225,8 @@ cudaError_t launch_bicg_matvec_g5(const Geom& g, const void* links, double kappa
 
 cudaError_t launch_bicg_update(int prec, SlotState* states, const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s) {
     dim3 grid(blas_blocks(N / 2), nslots);
-    if (prec == 0) update_kernel<double><<<grid, BL_THREADS, 0, s>>>(states, ptrs, N);
+    const int t = site_threads(N / 2, nslots, BL_THREADS);
+    if (prec == 0) update_kernel<double><<<t == 32 ? dim3(blas_blocks(N / 2 * (BL_THREADS / 32)), nslots) : grid, t, 0, s>>>(states, ptrs, N);
     else update_kernel<float><<<grid, BL_THREADS, 0, s>>>(states, ptrs, N);
     count_launches(1);
     return cudaGetLastError();
@@ -1296,7 +1286,8 @@ cudaError_t launch_stab_step(const Geom& g, const void* links, double kappa, int
 cudaError_t launch_bicg_direction(int prec, SlotState* states, const SlotPtrs* ptrs, int nslots, size_t N,
                                   cudaStream_t s) {
     dim3 grid(blas_blocks(N / 2), nslots);
-    if (prec == 0) direction_kernel<double><<<grid, BL_THREADS, 0, s>>>(states, ptrs, N);
+    const int t = site_threads(N / 2, nslots, BL_THREADS);
+    if (prec == 0) direction_kernel<double><<<t == 32 ? dim3(blas_blocks(N / 2 * (BL_THREADS / 32)), nslots) : grid, t, 0, s>>>(states, ptrs, N);
     else direction_kernel<float><<<grid, BL_THREADS, 0, s>>>(states, ptrs, N);
     count_launches(1);
     return cudaGetLastError();

@@ -1,5 +1,6 @@
 // Per-slot two-level reductions shared by the lattice kernels.
 #pragma once
+#include "fp64.cuh"
 #include "kernels.cuh"
 
 namespace lqcd {
@@ -25,17 +26,38 @@ __device__ bool reduce_slot(const SlotPtrs& P, int kind, C (&v)[NV], double2 (&t
     }
     bool last = last_block(P.counters + kind, nblocks);
     if (last) {
-        // the last block adds the partials in block order (deterministic)
-        double2 acc[NV];
+        // The last block adds the partials in a fixed order (deterministic): thread t
+        // takes the real number t % (2 NV) of every block whose index is
+        // t / (2 NV) modulo the threads per number, then a fixed tree. One FP64 sum
+        // per thread and step: an FP64 addition takes 64 cycles here, and the tail of
+        // each reduction is a chain of them.
+        constexpr int NR = 2 * NV;
+        static_assert(NR == 2 || NR == 4, "numbers per block");
+        const int q = threadIdx.x % NR, per = blockDim.x / NR;
+        const double* pd = reinterpret_cast<const double*>(pp);
+        double a0 = 0.0, a1 = 0.0;
+        unsigned b = threadIdx.x / NR;
+        for (; b + per < nblocks; b += 2 * per) {
+            a0 += __ldcg(pd + (size_t)b * NR + q);
+            a1 += __ldcg(pd + (size_t)(b + per) * NR + q);
+        }
+        if (b < nblocks) a0 += __ldcg(pd + (size_t)b * NR + q);
+        a0 += a1;
 #pragma unroll
-        for (int i = 0; i < NV; ++i) acc[i] = make_double2(0.0, 0.0);
-        for (unsigned b = threadIdx.x; b < nblocks; b += blockDim.x)
+        for (int o = 16; o >= NR; o >>= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        double* sd = reinterpret_cast<double*>(smd);
+        if (lane < NR) sd[w * NR + lane] = a0;
+        __syncthreads();
+        if (w == 0) {
+            // lane l: number l % NR of warp l / NR (at most 8 warps x 4 numbers)
+            double t = lane < nw * NR ? sd[lane] : 0.0;
 #pragma unroll
-            for (int i = 0; i < NV; ++i) acc[i] = acc[i] + __ldcg(pp + (size_t)b * NV + i);
-        // fixed-order tree over threads
-        block_sum<NV>(acc, smd);
+            for (int o = 16; o >= NR; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
 #pragma unroll
-        for (int i = 0; i < NV; ++i) tot[i] = acc[i];
+            for (int i = 0; i < NV; ++i)
+                tot[i] = make_double2(__shfl_sync(0xffffffffu, t, 2 * i), __shfl_sync(0xffffffffu, t, 2 * i + 1));
+        }
     }
     return last;
 }
@@ -52,5 +74,19 @@ template <typename S> struct Acc {
 };
 template <typename C> __device__ __forceinline__ auto abs2(C a) -> decltype(a.x) { return a.x * a.x + a.y * a.y; }
 
+constexpr double BREAK_TOL = 1e-14;
+
+// End of an operator launch for one slot (one thread): sigma = (phat, A p), the scales
+// of its breakdown test (p2 = |phat|^2, ap2 = |A p|^2) and alpha = rho / sigma.
+static __device__ __noinline__ void finish_sigma(SlotState& st, double2 sigma, double p2, double ap2, int products) {
+    st.sigma = sigma;
+    st.phat_norm = sqrt_fp64(p2);
+    st.ap_norm = sqrt_fp64(ap2);
+    st.matvecs += products;
+    if (!abs_at_least(sigma, BREAK_TOL, st.phat_norm, st.ap_norm) || (sigma.x == 0.0 && sigma.y == 0.0))
+        st.status = ST_BREAKDOWN;
+    else
+        st.alpha = cdiv_fp64(st.rho, sigma);
+}
 
 }  // namespace lqcd

@@ -201,10 +201,9 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
             Unit<S> xl = Unit<S>::load(P.x_lo, u);
             if (owed) {   // alpha p of this iteration's residual update
                 const Unit<S> p = Unit<S>::load(P.p, u);
-                xl.a = xl.a + al * p.a; xl.b = xl.b + al * p.b;
+                xl.a = cfma(xl.a, al, p.a); xl.b = cfma(xl.b, al, p.b);
             }
-            if constexpr (sizeof(S) == 4) { xh.a = xh.a + widen(xl.a); xh.b = xh.b + widen(xl.b); }
-            else { xh.a = xh.a + xl.a; xh.b = xh.b + xl.b; }
+            xh.a = xh.a + wid(xl.a); xh.b = xh.b + wid(xl.b);
             xh.store(P.x_hi, u);
             zero.store(P.x_lo, u);
             if (MODE == RU_DF) {   // the double-float copy that the residual reads
@@ -274,14 +273,14 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
                 LiveField{P.x_hi, Vs}.load(s, self);
                 LiveField{P.b, Vs}.load(s, r);
 #pragma unroll
-                for (int c = 0; c < 12; ++c) r[c] = r[c] - (self[c] - kk * acc[c]);
+                for (int c = 0; c < 12; ++c)
+                    r[c] = r[c] - make_double2(fma(-kk, acc[c].x, self[c].x), fma(-kk, acc[c].y, self[c].y));
             }
             cplx<S> rs[12], hs[12];
 #pragma unroll
             for (int c = 0; c < 12; ++c) {
                 nrm = fma(r[c].x, r[c].x, fma(r[c].y, r[c].y, nrm));
-                if constexpr (sizeof(S) == 4) rs[c] = narrow(r[c]);
-                else rs[c] = r[c];
+                rs[c] = nar<S>(r[c]);
             }
             Field<S>::store(rcur, Vs, s, rs);
             if (g5) {   // the shadow residual follows: rhat = gamma5 r
@@ -298,7 +297,7 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
                 }
             } else {
 #pragma unroll
-                for (int c = 0; c < 12; ++c) rho = rho + cdot(hs[c], rs[c]);
+                for (int c = 0; c < 12; ++c) rho = cdot_acc(rho, hs[c], rs[c]);
             }
         }
         double2 v[2] = {comp ? cz.value() : to_d(rho), make_double2(nrm, 0.0)};
@@ -323,7 +322,7 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
         }
         block_sum<2>(v, smd);
         if (threadIdx.x == 0) {
-            st.true_rnorm = sqrt(v[1].x);
+            st.true_rnorm = sqrt_fp64(v[1].x);
             st.matvecs += 1;
             if (st.true_rnorm <= st.tol * st.bnorm) {
                 st.status = ST_CONVERGED;

@@ -5,8 +5,6 @@
 
 namespace lqcd {
 
-constexpr double BREAK_TOL = 1e-14;
-
 // Vector units: two complex numbers (one float4 in FP32, two double2 in FP64).
 template <typename S> struct Unit;
 template <> struct Unit<float> {
@@ -72,20 +70,22 @@ template <typename S> __device__ __forceinline__ Unit<S> g5u(Unit<S> v, size_t u
 // update, or after the reliable update where one was asked for):
 // beta_{j-1} = rho_j / rho_{j-1}; window append v = r/||r||, w = (||r||/conj(rho)) rhat;
 // tridiagonal entries of H (Algorithm eigBiCG, step 3); iteration counters.
-__device__ __forceinline__ void bicg_scalars(SlotState& st, const SlotPtrs& P) {
-    const double2 beta = cdiv(st.rho_new, st.rho);
+// Not inlined: its registers would cut the occupancy of the vector kernels whose last
+// block calls it.
+static __device__ __noinline__ void bicg_scalars(SlotState& st, const SlotPtrs& P) {
+    const double2 beta = cdiv_fp64(st.rho_new, st.rho);
     if (st.m > 0) {
         const int k = st.vs;   // 0-based index of the appended vector
         const int m = st.m;
-        P.vscale[k] = 1.0 / st.rnorm;
-        P.wscale[k] = cdiv(make_double2(st.rnorm, 0.0), conj_(st.rho));
-        const double2 inv_a = cdiv(make_double2(1.0, 0.0), st.alpha);
+        P.vscale[k] = rcp_fp64(st.rnorm);
+        P.wscale[k] = cdiv_fp64(make_double2(st.rnorm, 0.0), conj_(st.rho));
+        const double2 inv_a = cdiv_fp64(make_double2(1.0, 0.0), st.alpha);
         double2 diag = inv_a;
-        if (st.iter > 0) diag = diag + cdiv(st.beta_prev, st.alpha_prev);
+        if (st.iter > 0) diag = diag + cdiv_fp64(st.beta_prev, st.alpha_prev);
         P.H[k * m + k] = diag;
         if (k + 1 < m) {
-            P.H[k * m + k + 1] = -(st.rnorm / st.rnorm_new) * cdiv(beta, st.alpha);
-            P.H[(k + 1) * m + k] = -(st.rnorm_new / st.rnorm) * inv_a;
+            P.H[k * m + k + 1] = -(st.rnorm * rcp_fp64(st.rnorm_new)) * cdiv_fp64(beta, st.alpha);
+            P.H[(k + 1) * m + k] = -(st.rnorm_new * P.vscale[k]) * inv_a;
         }
         st.vs = k + 1;
     }
@@ -98,7 +98,7 @@ __device__ __forceinline__ void bicg_scalars(SlotState& st, const SlotPtrs& P) {
     st.iter += 1;
     if (st.status == ST_RUNNING) {
         if (st.iter >= st.maxiter) st.status = ST_NOCONV;
-        else if (!(cabs_(st.rho) >= BREAK_TOL * st.rhat_norm * st.rnorm)) st.status = ST_BREAKDOWN;
+        else if (!abs_at_least(st.rho, BREAK_TOL, st.rhat_norm, st.rnorm)) st.status = ST_BREAKDOWN;
     }
     if (st.status != ST_RUNNING) st.live = 0;
     // the direction update adds the owed alpha p; a slot that stops here keeps it
@@ -108,15 +108,15 @@ __device__ __forceinline__ void bicg_scalars(SlotState& st, const SlotPtrs& P) {
 }
 
 // beta = (rho' / rho) (alpha / omega); counters; maxiter and breakdown (rho or omega).
-__device__ __forceinline__ void stab_scalars(SlotState& st) {
+static __device__ __noinline__ void stab_scalars(SlotState& st) {
     st.iter += 1;
     const bool om0 = cabs2(st.omega) == 0.0;
-    if (!om0) st.beta = cdiv(st.rho_new, st.rho) * cdiv(st.alpha, st.omega);
+    if (!om0) st.beta = cdiv_fp64(st.rho_new, st.rho) * cdiv_fp64(st.alpha, st.omega);
     st.rho = st.rho_new;
     st.rnorm = st.rnorm_new;
     if (st.status == ST_RUNNING) {
         if (st.iter >= st.maxiter) st.status = ST_NOCONV;
-        else if (om0 || !(cabs_(st.rho) >= BREAK_TOL * st.rhat_norm * st.rnorm)) st.status = ST_BREAKDOWN;
+        else if (om0 || !abs_at_least(st.rho, BREAK_TOL, st.rhat_norm, st.rnorm)) st.status = ST_BREAKDOWN;
     }
     if (st.status != ST_RUNNING) st.live = 0;
 }
