@@ -295,10 +295,10 @@ long long lqcd_kernel_launches(void);
 lqcd_status lqcd_time_kernel(lqcd_ctx *ctx, int kernel, int k, int reps, double *avg_ms);
 
 /* Implementation switch (no counterpart in the paper): on != 0 (the default)
- * runs the FP32 Galerkin projections (U_l^H r, growth blocks) and the FP32
- * restart window product V <- V Yc, W <- W Zc on the tensor cores (3xTF32
- * tcgen05 MMAs) where the shapes allow (m <= 64, 2 nev <= 24, 12 V a multiple
- * of 128); on = 0 uses the CUDA-core kernels. Results agree to FP32 rounding,
+ * runs the FP32 Galerkin projections (U_l^H r, growth blocks) on the TMA-staged
+ * kernel and the FP32 restart window product V <- V Yc, W <- W Zc on the tensor
+ * cores (3xTF32 tcgen05 MMAs) where the shapes allow (m <= 64, 2 nev <= 24,
+ * 12 V a multiple of 128); on = 0 uses the other kernels. Results agree to FP32 rounding,
  * not bit for bit. Waits for the context's stream; LQCD_ERR_STATE while
  * serving requests are in flight. */
 lqcd_status lqcd_set_tensor_cores(lqcd_ctx *ctx, int on);
@@ -331,9 +331,10 @@ lqcd_status lqcd_apply_pair(lqcd_ctx *ctx, int variant, int k, const double *p, 
  * U_l^H r and U_l^H A U_r): C[i*b + j] = sum_e conj(X_i(e)) Y_j(e) for i < a,
  * j < b.  X, Y: DEVICE pointers to a (resp. b) consecutive fields of n complex
  * FP32 numbers (re, im interleaved, 16-byte aligned).  C: HOST, a*b complex
- * (2ab doubles).  path 0 = CUDA cores (FP32 products, FP64 block sums),
- * path 1 = tensor cores (3xTF32 tcgen05 MMAs, FP32 runs summed in FP64;
- * needs 2n divisible by 32 and a <= 512, else LQCD_ERR_ARG).  With reps > 0
+ * (2ab doubles).  path 0 = fields read by every block that needs them (FP32
+ * products, FP32 block sums), path 1 = fields staged in shared memory by TMA
+ * (FP32 products, or 3xTF32 tcgen05 MMAs for large a and b; FP32 runs of 32
+ * elements, then FP64; needs 2n divisible by 32 and a <= 512, else LQCD_ERR_ARG).  With reps > 0
  * the call is repeated reps more times and *avg_ms receives the mean device
  * time of one call.  Allocates its scratch; synchronises the device. */
 lqcd_status lqcd_field_dots(int a, const float *X, int b, const float *Y, long long n, int path, int reps,

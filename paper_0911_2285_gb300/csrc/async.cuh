@@ -46,6 +46,7 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, unsigned parity) {
 }
 // Wait for the phase of the given parity to complete, at most wait_cycles().
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
+    if (mbar_test(bar, parity)) return true;   // before the limit is read: that load takes longer than most waits
     const long long t0 = clock64(), lim = wait_cycles();
     while (!mbar_test(bar, parity))
         if (clock64() - t0 > lim) return false;

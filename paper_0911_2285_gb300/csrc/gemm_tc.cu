@@ -7,8 +7,11 @@
 // Real form: with x' = (re x, im x) interleaved along K (K = 2N reals),
 //   Re C_ij = x'_i . y'_j,   Im C_ij = x'_i . z_j,  z = (im y, -re y),
 // so one real GEMM of the a x K matrix X' against the 2b x K matrix [Y'; Z]
-// gives both parts (M = 128 rows of X per CTA tile, N = 16 = 8 Y columns and
-// their Z twins, FP32 accumulators in tensor memory).
+// gives both parts (M = 128 rows of X per CTA tile, N = 48 = 24 Y columns and
+// their Z twins, FP32 accumulators in tensor memory). Its time is that of a full
+// tile, 4.3 ms at N = 10.6 M for any a <= 128 and b <= 24 (moving the split tiles
+// through shared memory), so it serves the large blocks; the others go to the FP32
+// form of launch_dots.
 //
 // Precision: 3xTF32. Each operand v is split into big = tf32(v) and
 // small = v - big, and the tile product is big.big + big.small + small.big,
@@ -39,34 +42,31 @@ namespace {
 
 constexpr int TC_KT = 32;        // reals per row per K-tile (128 bytes)
 constexpr int TC_M = 128;        // X rows per CTA tile
-constexpr int TC_NB = 8;         // Y fields per launch, narrow form (N = 2 * TC_NB)
-constexpr int TC_NB_WIDE = 24;   // wide form (N = 48): one launch serves up to 24 Y fields, so X is
-                                 // read once and each MMA instruction does three times the work
+constexpr int TC_NB = 24;        // Y fields per launch (N = 2 * TC_NB = 48 columns)
 constexpr int TC_STAGES = 5;
 constexpr int TC_FLUSH = 2;      // K-tiles per FP32 accumulation run in tensor memory
 constexpr int TC_XW = 8;         // split (transform) warps
 constexpr int TC_THREADS = 32 * (2 + TC_XW);
 constexpr int TC_NBUF = 4;       // accumulator sets in flight (runs the readers may lag behind)
 constexpr int TC_SUPER = 16;     // runs summed in FP32 before an FP64 add
-// tensor-memory columns: TC_NBUF runs x (big.big, correction) x 2 NB columns, as a power of two
+// tensor-memory columns: TC_NBUF runs x (big.big, correction) x 2 TC_NB columns, as a power of two
 __host__ __device__ constexpr unsigned tc_tmem_cols(int nb) {
     return (unsigned)(TC_NBUF * 2 * 2 * nb) <= 128u ? 128u : (unsigned)(TC_NBUF * 2 * 2 * nb) <= 256u ? 256u : 512u;
 }
 
-template <int NB> struct __align__(1024) TcStage {
+struct __align__(1024) TcStage {
     float xa[TC_M * TC_KT];      // TMA X tile, then its TF32 big part in place
     float xs[TC_M * TC_KT];      // small part of X
-    float yb[2 * NB * TC_KT];    // rows 0..NB-1: TMA Y tile -> big part; rows NB..2NB-1: big part of Z
-    float ys[2 * NB * TC_KT];    // small parts of Y and Z
+    float yb[2 * TC_NB * TC_KT];    // rows 0..TC_NB-1: TMA Y tile -> big part; rows TC_NB..2TC_NB-1: big part of Z
+    float ys[2 * TC_NB * TC_KT];    // small parts of Y and Z
 };
-static_assert(sizeof(TcStage<TC_NB>) % 1024 == 0, "stage must keep 1024-byte alignment");
-static_assert(sizeof(TcStage<TC_NB_WIDE>) % 1024 == 0, "stage must keep 1024-byte alignment");
+static_assert(sizeof(TcStage) % 1024 == 0, "stage must keep 1024-byte alignment");
 struct TcBars {
     uint64_t full[TC_STAGES], ready[TC_STAGES], empty[TC_STAGES], accfull[TC_NBUF], accempty[TC_NBUF];
     unsigned tmem;
     int abort;
 };
-template <int NB> constexpr size_t tc_smem() { return TC_STAGES * sizeof(TcStage<NB>) + 1024 /*align slack*/ + sizeof(TcBars); }
+constexpr size_t tc_smem() { return TC_STAGES * sizeof(TcStage) + 1024 /*align slack*/ + sizeof(TcBars); }
 
 __device__ __forceinline__ void split4(float4 v, float4& big, float4& small) {
     big = make_float4(to_tf32(v.x), to_tf32(v.y), to_tf32(v.z), to_tf32(v.w));
@@ -77,6 +77,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 // Bounded wait that also gives up once another role has aborted.
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, unsigned parity, volatile int* abort) {
+    if (mbar_test(bar, parity)) return true;   // before the limit is read: that load takes longer than most waits
     const long long t0 = clock64(), lim = wait_cycles();
     while (!mbar_test(bar, parity)) {
         if (*abort) return false;
@@ -90,15 +91,13 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, unsigned parity, vo
 // TF32 big/small parts, and warps 2-5 (one per tensor-memory lane quarter)
 // also move each finished accumulation run into their FP64 sums.
 // Grid (split-K CTAs, row tiles of 128). part: [gridDim.y][gridDim.x][128][16] FP64.
-// NB: Y fields per launch (N = 2 NB columns: the Y fields and their Z twins).
-template <int NB>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     dots_tc_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap my, int box_rows,
                    long long tiles, double* part, int* err) {
-    constexpr int NC = 2 * NB;                       // accumulator columns
-    constexpr unsigned TMEM_COLS = tc_tmem_cols(NB);
+    constexpr int NC = 2 * TC_NB;                       // accumulator columns
+    constexpr unsigned TMEM_COLS = tc_tmem_cols(TC_NB);
     extern __shared__ unsigned char smem_raw[];
-    using Stage = TcStage<NB>;
+    using Stage = TcStage;
     Stage* st = reinterpret_cast<Stage*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     TcBars* B = reinterpret_cast<TcBars*>(st + TC_STAGES);
     volatile int* abort = &B->abort;
@@ -108,7 +107,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const long long t1 = (long long)(blockIdx.x + 1) * tiles / gridDim.x;
     const int n = (int)(t1 - t0);
     const int ngroups = (n + TC_FLUSH - 1) / TC_FLUSH;
-    const unsigned tx = (unsigned)(box_rows + NB) * TC_KT * 4;
+    const unsigned tx = (unsigned)(box_rows + TC_NB) * TC_KT * 4;
 
     if (tid == 0) {
         for (int s = 0; s < TC_STAGES; ++s) {
@@ -240,7 +239,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 xa[p] = big;
                 xs[p] = small;
             }
-            for (int yt = xt; yt < NB * TC_KT / 4; yt += 32 * TC_XW) {   // Y and its Z twin
+            for (int yt = xt; yt < TC_NB * TC_KT / 4; yt += 32 * TC_XW) {   // Y and its Z twin
                 float4* yb = reinterpret_cast<float4*>(S.yb);
                 float4* ys = reinterpret_cast<float4*>(S.ys);
                 const float4 y = yb[yt];
@@ -249,8 +248,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 yb[yt] = big;
                 ys[yt] = small;
                 split4(make_float4(y.y, -y.x, y.w, -y.z), big, small);
-                yb[NB * TC_KT / 4 + yt] = big;
-                ys[NB * TC_KT / 4 + yt] = small;
+                yb[TC_NB * TC_KT / 4 + yt] = big;
+                ys[TC_NB * TC_KT / 4 + yt] = small;
             }
             fence_proxy_async();
             __syncwarp();
@@ -619,23 +618,21 @@ bool encode_tensor_map_f32(void* map, const void* base, int rank, const uint64_t
                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool tensor_maps_available() { return get_encode() == cudaSuccess; }
+
 bool dots_tc_supported(int a, const void* X, const void* Y, size_t N) {
     return a > 0 && a <= 4 * TC_M && N > 0 && (2 * N) % TC_KT == 0 && ((uintptr_t)X & 15) == 0 &&
            ((uintptr_t)Y & 15) == 0 && get_encode() == cudaSuccess;
 }
 
 size_t dots_tc_scratch_doubles(int a) {
-    return (size_t)((a + TC_M - 1) / TC_M) * num_sms() * TC_M * 2 * TC_NB_WIDE;
+    return (size_t)((a + TC_M - 1) / TC_M) * num_sms() * TC_M * 2 * TC_NB;
 }
 
 cudaError_t prepare_dots_tc() {
     std::call_once(g_prepare_once, [] {
-        g_prepare_err = cudaFuncSetAttribute((const void*)dots_tc_kernel<TC_NB>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem<TC_NB>());
-        if (g_prepare_err == cudaSuccess)
-            g_prepare_err = cudaFuncSetAttribute((const void*)dots_tc_kernel<TC_NB_WIDE>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)tc_smem<TC_NB_WIDE>());
+        g_prepare_err = cudaFuncSetAttribute((const void*)dots_tc_kernel,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem());
         if (g_prepare_err == cudaSuccess)
             g_prepare_err = cudaFuncSetAttribute((const void*)restart_tc_kernel,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RT_SMEM);
@@ -686,9 +683,7 @@ cudaError_t launch_dots_tc(int a, const void* X, size_t x_stride, int b, const v
     const int ty = (a + TC_M - 1) / TC_M;
     int nblk = num_sms();
     if (nblk > tiles) nblk = (int)tiles;
-    // up to 8 Y fields per launch in the narrow form (N = 16), more in the wide one
-    // (N = 48), which reads X once for 24 fields
-    const int nb = b > TC_NB ? TC_NB_WIDE : TC_NB;
+    const int nb = TC_NB;
     if ((size_t)ty * nblk * TC_M * 2 * nb > scratch_doubles) return cudaErrorInvalidValue;
     const int box_rows = ty > 1 ? TC_M : (a + 7) / 8 * 8;
     CUtensorMap mx;
@@ -698,12 +693,7 @@ cudaError_t launch_dots_tc(int a, const void* X, size_t x_stride, int b, const v
         CUtensorMap my;
         const char* Yj = reinterpret_cast<const char*>(Y) + (size_t)j0 * y_stride;
         if (!encode_rows(&my, Yj, N, bb, y_stride, nb)) return cudaErrorInvalidValue;
-        if (nb == TC_NB)
-            dots_tc_kernel<TC_NB><<<dim3(nblk, ty), TC_THREADS, tc_smem<TC_NB>(), st>>>(mx, my, box_rows, tiles,
-                                                                                     scratch, err);
-        else
-            dots_tc_kernel<TC_NB_WIDE><<<dim3(nblk, ty), TC_THREADS, tc_smem<TC_NB_WIDE>(), st>>>(
-                mx, my, box_rows, tiles, scratch, err);
+        dots_tc_kernel<<<dim3(nblk, ty), TC_THREADS, tc_smem(), st>>>(mx, my, box_rows, tiles, scratch, err);
         count_launches(1);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -1034,12 +1034,17 @@ cudaError_t launch_convert(const void* src, int sp, void* dst, int dp, size_t n,
 
 cudaError_t launch_multidot(int a, const void* X, int xp, int b, const void* Y, int yp, size_t N, double2* Cm,
                             int ldc, int conj_store, double2* scratch, size_t scratch_elems, cudaStream_t st,
-                            int* err, int tensor_cores) {
+                            int* err, int staged) {
     if (a <= 0 || b <= 0) return cudaSuccess;
-    if (tensor_cores && xp == 1 && yp == 1 && dots_tc_supported(a, X, Y, N) &&
-        dots_tc_scratch_doubles(a) <= 2 * scratch_elems)
+    // The tensor-core form takes a tile of 128 X against 24 Y fields whatever part of it is
+    // filled (4.3 ms at N = 10.6 M), the FP32 form 1.35 ms per 80 X and 8 Y fields: 128 x 24
+    // cost as much as 252 x 8.
+    if (staged && xp == 1 && yp == 1 && div_up(b, 8) * a > 252 * div_up(a, 128) * div_up(b, 24) &&
+        dots_tc_supported(a, X, Y, N) && dots_tc_scratch_doubles(a) <= 2 * scratch_elems)
         return launch_dots_tc(a, X, N * 8, b, Y, N * 8, N, Cm, ldc, conj_store, reinterpret_cast<double*>(scratch),
                               2 * scratch_elems, err, st);
+    if (staged && err && xp == 1 && yp == 1 && dots_supported(a, X, Y, N) && dots_scratch(a, b, N) <= scratch_elems)
+        return launch_dots(a, X, b, Y, N, Cm, ldc, conj_store, scratch, scratch_elems, err, st);
     for (int j0 = 0; j0 < b; j0 += MD_BMAX) {
         const int bb = b - j0 < MD_BMAX ? b - j0 : MD_BMAX;
         const int nby = div_up(a, MD_TI);

@@ -55,23 +55,27 @@ cudaError_t launch_convert(const void* src, int src_prec, void* dst, int dst_pre
 // conj_store: store conj(C) transposed, C[j*ldc + i] instead.
 cudaError_t launch_multidot(int a, const void* X, int xprec, int b, const void* Y, int yprec,
                             size_t N, double2* C, int ldc, int conj_store, double2* scratch,
-                            size_t scratch_elems, cudaStream_t st, int* err = nullptr, int tensor_cores = 1);
-// tensor_cores = 1: FP32 x FP32 products go to the tensor-core path where the shape allows.
-// Tensor-core form of launch_multidot for FP32 X and Y (gemm_tc.cu): 3xTF32
-// tcgen05 MMAs, split-K over the SMs, partials summed in FP64. Fields of X
-// (resp. Y) are x_stride (y_stride) bytes apart. scratch: dots_tc_scratch_doubles(a)
-// doubles. err: device word set to 1 if a bounded wait gave up.
+                            size_t scratch_elems, cudaStream_t st, int* err = nullptr, int staged = 1);
+// staged = 1: FP32 x FP32 products go to launch_dots (dots.cu: TMA-staged FP32 products)
+// or launch_dots_tc (gemm_tc.cu: 3xTF32 tcgen05 MMAs, split-K over the SMs, partials
+// summed in FP64) where the shape allows. X and Y are consecutive fields. scratch:
+// dots_scratch(a, b, N) double2, dots_tc_scratch_doubles(a) doubles. err: device word
+// set to 1 if a bounded wait gave up.
+bool dots_supported(int a, const void* X, const void* Y, size_t N);
+size_t dots_scratch(int a, int b, size_t N);
+cudaError_t launch_dots(int a, const void* X, int b, const void* Y, size_t N, double2* C, int ldc, int conj_store,
+                        double2* scratch, size_t scratch_elems, int* err, cudaStream_t st);
 bool dots_tc_supported(int a, const void* X, const void* Y, size_t N);
+size_t dots_tc_scratch_doubles(int a);
+cudaError_t launch_dots_tc(int a, const void* X, size_t x_stride, int b, const void* Y, size_t y_stride, size_t N,
+                           double2* C, int ldc, int conj_store, double* scratch, size_t scratch_doubles, int* err,
+                           cudaStream_t st);
+cudaError_t set_wait_cycles_dots(long long cycles);
 // Tensor-core form of the FP32 restart window product (gemm_tc.cu), same
 // contract as launch_window_gemm; supported for m <= 64, 2 nev <= 24, N % 128 == 0.
 bool restart_tc_supported(int m, int two_nev, size_t N);
 cudaError_t launch_restart_tc(SlotState* states, const SlotPtrs* ptrs, int nslots, size_t N, int* err,
                               cudaStream_t st);
-size_t dots_tc_scratch_doubles(int a);
-cudaError_t prepare_dots_tc();
-cudaError_t launch_dots_tc(int a, const void* X, size_t x_stride, int b, const void* Y, size_t y_stride, size_t N,
-                           double2* C, int ldc, int conj_store, double* scratch, size_t scratch_doubles, int* err,
-                           cudaStream_t st);
 // overwrite = 0: Y_j += sum_i X_i D[i*ldd + j];  overwrite = 1: Y_j = sum_i X_i D[i*ldd + j].
 // The arithmetic is FP32 when X is FP32 (the sum is added to an FP64 Y in FP64),
 // unless fp64_arith is set and Y is FP64 (coefficients with large, cancelling
@@ -106,6 +110,7 @@ int matvec_variants();
 bool matvec_variant_ok(const Geom& g, int v);
 // Tiled tensor map (FP32 elements, no swizzle, rank <= 5) into the 128-byte
 // CUtensorMap at map; dims innermost first, strides in bytes (rank - 1 of them).
+bool tensor_maps_available();
 bool encode_tensor_map_f32(void* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
                            const uint32_t* box);
 // Operator pair with links and spinor tiles staged in shared memory by TMA

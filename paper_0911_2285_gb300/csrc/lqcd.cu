@@ -156,7 +156,7 @@ struct lqcd_ctx {
     double2* dconst = nullptr;      // constants
 
     int dslash_variant = 0;         // operator-kernel shape (autotuned at init); TILED = plane streaming
-    int use_tc = 1;                 // FP32 projections and restart products on the tensor cores
+    int use_tc = 1;                 // FP32 projections staged by TMA, restart products on the tensor cores
     int ru_variant = 0;             // kernel shape of the final FP64 residual (timed at init)
     int ru_blocks = 1;              // co-resident blocks of the reliable-update kernel
     TileGeom tgeo[MAX_SLOTS + 1] = {};
@@ -1602,10 +1602,10 @@ extern "C" lqcd_status lqcd_field_dots(int a, const float* X, int b, const float
         return LQCD_ERR_ARG;
     const size_t N = (size_t)n;
     if (path == 1 && !dots_tc_supported(a, X, Y, N)) {
-        g_last_error = "tensor-core path needs 2n % 32 == 0, a <= 512 and 16-byte aligned fields";
+        g_last_error = "staged path needs 2n % 32 == 0, a <= 512 and 16-byte aligned fields";
         return LQCD_ERR_ARG;
     }
-    const size_t md_elems = std::max((size_t)((a + 3) / 4) * 1216 * 32, dots_tc_scratch_doubles(a) / 2 + 1);
+    const size_t md_elems = std::max((size_t)((a + 3) / 4) * 1216 * 32, std::max(dots_scratch(a, b, N), dots_tc_scratch_doubles(a) / 2 + 1));
     double2 *scratch = nullptr, *dC = nullptr;
     int* derr = nullptr;
     lqcd_status ret = LQCD_OK;
@@ -1636,7 +1636,7 @@ extern "C" lqcd_status lqcd_field_dots(int a, const float* X, int b, const float
         if (e == cudaSuccess) e = cudaMemcpy(C, dC, (size_t)a * b * 16, cudaMemcpyDeviceToHost);
         if (e == cudaSuccess) e = cudaMemcpy(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) { set_error("field dots", e); ret = LQCD_ERR_CUDA; }
-        else if (herr) { g_last_error = "tensor-core dots: a bounded wait timed out"; ret = LQCD_ERR_TIMEOUT; }
+        else if (herr) { g_last_error = "staged inner products: a bounded wait timed out"; ret = LQCD_ERR_TIMEOUT; }
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
     }
@@ -2191,6 +2191,7 @@ extern "C" lqcd_status lqcd_set_wait_limit(long long cycles) {
     CK(set_wait_cycles_tc(cycles));
     CK(set_wait_cycles_tiled(cycles));
     CK(set_wait_cycles_ru(cycles));
+    CK(set_wait_cycles_dots(cycles));
     return LQCD_OK;
 }
 
