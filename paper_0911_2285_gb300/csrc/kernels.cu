@@ -40,26 +40,34 @@ int ds_blocks(int V) {
 }
 
 // ------------------------------------------------------------------- apply
-// r = b - A x with FP64 x, b, r and the hop in FP32 arithmetic on FP32 links:
-// the starting and deflation residuals of the mixed-precision solver, which
-// are consumed in FP32 (the reliable updates and the final residual use
-// FP64-class arithmetic). jobs: in = x, aux = b, out = r.
+// r = b - A x with FP64 x and b and the hop in FP32 arithmetic on FP32 links: the
+// starting and deflation residuals of the mixed-precision solver, which are consumed
+// in FP32 (the reliable updates and the final residual use FP64-class arithmetic).
+// x32: x rounded to FP32; SO: storage of r. nf consecutive fields.
+// What bounds it: rounding each of the eight neighbours from FP64 costs 16 conversions
+// per number on the FP64 pipe (26 operations with the rest: 480 us for 8 fields of
+// 16^3 x 32); from x32 four FP64 operations are left (86 us on that pipe), and bytes:
+// x, b and x32 read once, r written, 48 to 56 per number. Measured 480 -> 184 us
+// and 52 for x32.
+template <typename SO>
 __global__ void __launch_bounds__(DS_THREADS) residual32_kernel(Geom g, const float4* links, double kappa,
-                                                                const ApplyJob* jobs, int njobs) {
-    const int jid = blockIdx.x % njobs, sblock = blockIdx.x / njobs, nsb = gridDim.x / njobs;
-    const ApplyJob jb = jobs[jid];
+                                                                const double2* x, const float2* x32, const double2* b,
+                                                                cplx<SO>* r, int nf) {
+    const int jid = blockIdx.x % nf, sblock = blockIdx.x / nf, nsb = gridDim.x / nf;   // fields fastest: shared links
+    const size_t off = (size_t)jid * 12 * g.V;
     LinksF U{links, g.V};
-    FieldIn<double> in{jb.in, g.V};
+    FieldIn<float> in{x32 + off, g.V};
     const double k = kappa;
     for (int s = sblock * blockDim.x + threadIdx.x; s < g.V; s += nsb * blockDim.x) {
         float2 acc[12];
         hop_site<false, float>(g, U, in, s, acc);
-        double2 x[12], b[12];
-        Field<double>::load(jb.in, g.V, s, x);
-        Field<double>::load(jb.aux, g.V, s, b);
+        double2 xs[12], bs[12];
+        Field<double>::load(x + off, g.V, s, xs);
+        Field<double>::load(b + off, g.V, s, bs);
+        cplx<SO> out[12];
 #pragma unroll
-        for (int c = 0; c < 12; ++c) b[c] = b[c] - (x[c] - k * to_d(acc[c]));
-        Field<double>::store(jb.out, g.V, s, b);
+        for (int c = 0; c < 12; ++c) out[c] = nar<SO>(bs[c] - (xs[c] - k * widen(acc[c])));
+        Field<SO>::store(r + off, g.V, s, out);
     }
 }
 
@@ -116,7 +124,7 @@ __global__ void unpack_kernel(const void* dev, double2* aos, int V, int k) {
 template <typename SI, typename SO>
 __global__ void convert_kernel(const void* src, void* dst, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        st_elem<SO>(dst, i, cvt<SO>(to_d(ld_elem<SI>(src, i))));
+        st_elem<SO>(dst, i, nar<SO>(wid(ld_elem<SI>(src, i))));
 }
 
 // ------------------------------------------------------------- multidot
@@ -209,6 +217,57 @@ __global__ void __launch_bounds__(BL_THREADS) vupdate_kernel(int a, const void* 
                 double2 upd = to_d(acc[j]);
                 if (!overwrite) upd = upd + to_d(ld_elem<SY>(yj, e));   // add in the target precision
                 st_elem<SY>(yj, e, cvt<SY>(upd));
+            }
+    }
+}
+
+// The same with FP32 X and FP32 sums, added to an FP64 Y in FP64. A thread takes two
+// consecutive elements, so a coefficient read from shared memory (two Y fields per
+// 16-byte load) serves 16 multiply-adds, and four X loads are in flight. Bound: X once
+// and Y twice over memory (40 x 8 on 16^3 x 32: 0.5 + 0.4 GB, 133 us) against 54 us of
+// multiply-adds; with one element per thread and conversions on the FP64 pipe 325 us,
+// measured 223. N even.
+template <typename SY>
+__global__ void __launch_bounds__(BL_THREADS) vupdate32_kernel(int a, const float4* X, const double2* D, int ldd, int b,
+                                                               void* Y, int overwrite, size_t N) {
+    __shared__ float4 Ds[MAX_SMALL * MD_BMAX / 2];
+    for (int q = threadIdx.x; q < a * (MD_BMAX / 2); q += blockDim.x) {
+        const int i = q / (MD_BMAX / 2), j = 2 * (q % (MD_BMAX / 2));
+        const double2 z = make_double2(0.0, 0.0);
+        const double2 d0 = j < b ? D[(size_t)i * ldd + j] : z, d1 = j + 1 < b ? D[(size_t)i * ldd + j + 1] : z;
+        Ds[q] = make_float4((float)d0.x, (float)d0.y, (float)d1.x, (float)d1.y);
+    }
+    __syncthreads();
+    const size_t units = N / 2;
+    for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < units; u += (size_t)gridDim.x * blockDim.x) {
+        float2 acc[MD_BMAX][2];
+#pragma unroll
+        for (int j = 0; j < MD_BMAX; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int i = 0; i < a; ++i) {
+            const float4 x = X[(size_t)i * units + u];
+            const float2 x0 = make_float2(x.x, x.y), x1 = make_float2(x.z, x.w);
+#pragma unroll
+            for (int p = 0; p < MD_BMAX / 2; ++p)
+                if (2 * p < b) {
+                    const float4 d = Ds[i * (MD_BMAX / 2) + p];
+                    const float2 d0 = make_float2(d.x, d.y), d1 = make_float2(d.z, d.w);
+                    acc[2 * p][0] = acc[2 * p][0] + x0 * d0;
+                    acc[2 * p][1] = acc[2 * p][1] + x1 * d0;
+                    acc[2 * p + 1][0] = acc[2 * p + 1][0] + x0 * d1;
+                    acc[2 * p + 1][1] = acc[2 * p + 1][1] + x1 * d1;
+                }
+        }
+#pragma unroll
+        for (int j = 0; j < MD_BMAX; ++j)
+            if (j < b) {
+                cplx<SY>* y = reinterpret_cast<cplx<SY>*>(Y) + (size_t)j * N + 2 * u;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    double2 v = widen(acc[j][h]);
+                    if (!overwrite) v = v + wid(y[h]);
+                    y[h] = nar<SY>(v);
+                }
             }
     }
 }
@@ -1000,10 +1059,15 @@ cudaError_t launch_apply(const Geom& g, const void* links, double kappa, int pre
     return cudaGetLastError();
 }
 
-cudaError_t launch_residual32(const Geom& g, const void* links32, double kappa, const ApplyJob* d_jobs, int njobs,
-                              cudaStream_t st) {
-    const int grid = ds_blocks(g.V) * njobs;
-    residual32_kernel<<<grid, DS_THREADS, 0, st>>>(g, reinterpret_cast<const float4*>(links32), kappa, d_jobs, njobs);
+cudaError_t launch_residual32(const Geom& g, const void* links32, double kappa, const double2* x, void* x32,
+                              const double2* b, void* r, int rprec, int nf, cudaStream_t st) {
+    cudaError_t e = launch_convert(x, 0, x32, 1, (size_t)nf * 12 * g.V, st);
+    if (e != cudaSuccess) return e;
+    const int grid = ds_blocks(g.V) * nf;
+    const float4* U = reinterpret_cast<const float4*>(links32);
+    const float2* xs = reinterpret_cast<const float2*>(x32);
+    if (rprec) residual32_kernel<float><<<grid, DS_THREADS, 0, st>>>(g, U, kappa, x, xs, b, reinterpret_cast<float2*>(r), nf);
+    else residual32_kernel<double><<<grid, DS_THREADS, 0, st>>>(g, U, kappa, x, xs, b, reinterpret_cast<double2*>(r), nf);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1071,15 +1135,16 @@ cudaError_t launch_multidot(int a, const void* X, int xp, int b, const void* Y, 
 
 cudaError_t launch_vupdate(int a, const void* X, int xp, const double2* D, int ldd, int b, void* Y, int yp,
                            int overwrite, size_t N, cudaStream_t st, int fp64_arith) {
-    if (a > MAX_SMALL) return cudaErrorInvalidValue;
+    if (a > MAX_SMALL || N % 2) return cudaErrorInvalidValue;   // fields hold 12 numbers per site
     for (int j0 = 0; j0 < b; j0 += MD_BMAX) {
         const int bb = b - j0 < MD_BMAX ? b - j0 : MD_BMAX;
         char* Yj = reinterpret_cast<char*>(Y) + (size_t)j0 * N * (yp == 0 ? 16 : 8);
         const double2* Dj = D + j0;
         int nb = blas_blocks(N);
-        if (xp == 1 && yp == 1) vupdate_kernel<float, float, float><<<nb, BL_THREADS, 0, st>>>(a, X, Dj, ldd, bb, Yj, overwrite, N);
+        const float4* X4 = reinterpret_cast<const float4*>(X);
+        if (xp == 1 && yp == 1) vupdate32_kernel<float><<<blas_blocks(N / 2), BL_THREADS, 0, st>>>(a, X4, Dj, ldd, bb, Yj, overwrite, N);
         else if (xp == 1 && yp == 0 && fp64_arith) vupdate_kernel<float, double, double><<<nb, BL_THREADS, 0, st>>>(a, X, Dj, ldd, bb, Yj, overwrite, N);
-        else if (xp == 1 && yp == 0) vupdate_kernel<float, double, float><<<nb, BL_THREADS, 0, st>>>(a, X, Dj, ldd, bb, Yj, overwrite, N);
+        else if (xp == 1 && yp == 0) vupdate32_kernel<double><<<blas_blocks(N / 2), BL_THREADS, 0, st>>>(a, X4, Dj, ldd, bb, Yj, overwrite, N);
         else if (xp == 0 && yp == 1) vupdate_kernel<double, float, double><<<nb, BL_THREADS, 0, st>>>(a, X, Dj, ldd, bb, Yj, overwrite, N);
         else vupdate_kernel<double, double, double><<<nb, BL_THREADS, 0, st>>>(a, X, Dj, ldd, bb, Yj, overwrite, N);
         count_launches(1);

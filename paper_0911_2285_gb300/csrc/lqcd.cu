@@ -730,26 +730,19 @@ lqcd_status apply_fields(lqcd_ctx* c, int prec, int dagger, int nf, const void* 
     return LQCD_OK;
 }
 
-// r = b - A x for nf FP64 fields (consecutive slots): FP32 hop arithmetic in
-// mixed precision (the result feeds FP32 work), FP64 otherwise or when precise
-// is set (a residual far below ||A|| ||x||, e.g. after a first solve leg, where
-// FP32 hop rounding would swamp it).
-lqcd_status residual_fields(lqcd_ctx* c, int nf, const double2* x, double2* r, const double2* b,
-                            bool precise = false) {
-    if (!c->kprec || precise || c->eo) return apply_fields(c, 0, 0, nf, x, c->dbytes, r, c->dbytes, b);
-    std::vector<ApplyJob> jobs(2 * c->kmax);
-    for (int j0 = 0; j0 < nf; j0 += 2 * c->kmax) {
-        const int nb = std::min(2 * c->kmax, nf - j0);
-        for (int j = 0; j < nb; ++j) {
-            jobs[j].in = x + (size_t)(j0 + j) * c->N;
-            jobs[j].out = r + (size_t)(j0 + j) * c->N;
-            jobs[j].aux = b + (size_t)(j0 + j) * c->N;
-            jobs[j].dagger = 0;
-        }
-        CK(cudaMemcpyAsync(c->d_jobs, jobs.data(), sizeof(ApplyJob) * nb, cudaMemcpyHostToDevice, c->stream));
-        CK(launch_residual32(c->g, c->links32, c->p.kappa, c->d_jobs, nb, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
-    }
+bool residual_in_fp32(const lqcd_ctx* c, bool precise) { return c->kprec && !precise && !c->eo; }
+
+// r = b - A x_hi for slots s0 .. s0+nf-1: FP32 hop arithmetic in mixed precision (the
+// result feeds FP32 work; x_lo of these slots is overwritten by x_hi in FP32), FP64
+// otherwise or when precise is set (a residual far below ||A|| ||x||, e.g. after a
+// first solve leg, where FP32 hop rounding would swamp it). r goes to rt, in FP64
+// or, with fp32 set (only where residual_in_fp32), as consecutive FP32 fields.
+lqcd_status residual_fields(lqcd_ctx* c, int s0, int nf, bool precise = false, bool fp32 = false) {
+    const double2* x = c->x_hi_all + (size_t)s0 * c->N;
+    const double2* b = c->b_all + (size_t)s0 * c->N;
+    double2* r = c->rt_all + (size_t)s0 * c->N;
+    if (!residual_in_fp32(c, precise)) return apply_fields(c, 0, 0, nf, x, c->dbytes, r, c->dbytes, b);
+    CK(launch_residual32(c->g, c->links32, c->p.kappa, x, c->krylov(c->x_lo_all, s0), b, r, fp32 ? 1 : 0, nf, c->stream));
     return LQCD_OK;
 }
 
@@ -849,8 +842,8 @@ lqcd_status deflate_range(lqcd_ctx* c, int s0, int k, bool precise = false, bool
     const bool guard = first && c->p.gamma5;
     double2* xh = c->x_hi_all + (size_t)s0 * c->N;
     double2* rt = c->rt_all + (size_t)s0 * c->N;
-    const double2* bs = c->b_all + (size_t)s0 * c->N;
-    lqcd_status s = residual_fields(c, k, xh, rt, bs, precise);
+    const bool direct = residual_in_fp32(c, precise) && !guard;   // the guard's norms take the FP64 residual
+    lqcd_status s = residual_fields(c, s0, k, precise, direct);
     if (s != LQCD_OK) return s;
     double2* scr = c->dsmall + (size_t)MAX_SMALL * MAX_SMALL * 6;   // norms before / after, reverting C
     double* nrm = reinterpret_cast<double*>(scr);
@@ -858,18 +851,17 @@ lqcd_status deflate_range(lqcd_ctx* c, int s0, int k, bool precise = false, bool
     if (guard) CK(launch_norms(k, rt, 0, c->N, nrm, c->mdscratch, c->mdscratch_elems, c->stream));
     double2* C = c->dsmall;   // n x k, ld k
     const void* R = rt;
-    int rp = 0;
-    if (c->kprec) {   // FP32 projections: convert the residuals first (into these slots' x_lo)
+    if (c->kprec && !direct) {   // FP32 projections: convert the residuals first (into these slots' x_lo)
         void* xl = c->krylov(c->x_lo_all, s0);
         CK(launch_convert(rt, 0, xl, 1, (size_t)k * c->N, c->stream));
         R = xl;
-        rp = 1;
     }
+    const int rp = c->kprec;
     CK(launch_multidot(n, c->Ul, c->kprec, k, R, rp, c->N, C, k, 0, c->mdscratch, c->mdscratch_elems, c->stream, c->d_err, c->use_tc));
     CK(launch_lu_solve(n, c->Hlu, c->n_def_max, c->Hpiv, 0, k, C, k, c->stream));
     CK(launch_vupdate(n, c->Ur, c->kprec, C, k, k, xh, 0, 0, c->N, c->stream));
     if (!guard) return LQCD_OK;
-    s = residual_fields(c, k, xh, rt, bs, precise);
+    s = residual_fields(c, s0, k, precise);
     if (s != LQCD_OK) return s;
     CK(launch_norms(k, rt, 0, c->N, nrm + MAX_SLOTS, c->mdscratch, c->mdscratch_elems, c->stream));
     double hn[2 * MAX_SLOTS];
@@ -891,7 +883,7 @@ lqcd_status deflate_range(lqcd_ctx* c, int s0, int k, bool precise = false, bool
             }
         CK(cudaMemcpyAsync(Crev, hc.data(), sizeof(double2) * n * k, cudaMemcpyHostToDevice, c->stream));
         CK(launch_vupdate(n, c->Ur, c->kprec, Crev, k, k, xh, 0, 0, c->N, c->stream));
-        s = residual_fields(c, k, xh, rt, bs, precise);
+        s = residual_fields(c, s0, k, precise);
         if (s != LQCD_OK) return s;
         for (int j = 0; j < k; ++j) c->deflations_discarded += bad[j] ? 1 : 0;
     }
@@ -1178,7 +1170,7 @@ lqcd_status solve_slots(lqcd_ctx* c, int k, int windowed, double tol, bool rec_s
     }
     CK(cudaMemcpyAsync(c->d_state, c->h_state, sizeof(SlotState) * c->kmax, cudaMemcpyHostToDevice, c->stream));
     // r0 = b - A x0 (FP64), then the Krylov start vectors
-    lqcd_status s = residual_fields(c, k, c->x_hi_all, c->rt_all, c->b_all, precise);
+    lqcd_status s = residual_fields(c, 0, k, precise);
     if (s != LQCD_OK) return s;
     CK(launch_bicg_start(c->g, c->links64, c->p.kappa, c->kprec, c->d_state, c->d_ptrs, k, c->N, c->stream));
     while (true) {
@@ -1957,8 +1949,7 @@ lqcd_status begin_slot(lqcd_ctx* c, int s, lqcd_mode md, double tol, bool window
     st.g5 = c->p.gamma5;
     st.stab = stab && !windowed ? 1 : 0;
     CK(cudaMemcpyAsync(c->d_state + s, &st, sizeof(SlotState), cudaMemcpyHostToDevice, c->stream));
-    lqcd_status r = residual_fields(c, 1, c->x_hi_all + (size_t)s * c->N, c->rt_all + (size_t)s * c->N,
-                                    c->b_all + (size_t)s * c->N, precise);
+    lqcd_status r = residual_fields(c, s, 1, precise);
     if (r != LQCD_OK) return r;
     CK(launch_bicg_start(c->g, c->links64, c->p.kappa, c->kprec, c->d_state + s, c->d_ptrs + s, 1, c->N, c->stream));
     return LQCD_OK;
