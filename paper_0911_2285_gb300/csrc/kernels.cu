@@ -71,54 +71,82 @@ __global__ void __launch_bounds__(DS_THREADS) residual32_kernel(Geom g, const fl
     }
 }
 
+// nf consecutive fields, fields fastest in the grid: they share each block's links.
 template <typename S, bool RES>
 __global__ void __launch_bounds__(DS_THREADS) apply_kernel(Geom g, const void* links, double kappa,
-                                                           const ApplyJob* jobs, int njobs) {
+                                                           const void* src, void* dst, const double2* aux, int dagger,
+                                                           int nf) {
     using C = cplx<S>;
-    const int jid = blockIdx.x % njobs, sblock = blockIdx.x / njobs, nsb = gridDim.x / njobs;
-    const ApplyJob jb = jobs[jid];
+    const int jid = blockIdx.x % nf, sblock = blockIdx.x / nf, nsb = gridDim.x / nf;
+    const size_t off = (size_t)jid * 12 * g.V;
     typename LinkSel<S>::type U{reinterpret_cast<decltype(U.u)>(links), g.V};
-    FieldIn<S> in{jb.in, g.V};
+    FieldIn<S> in{reinterpret_cast<const C*>(src) + off, g.V};
     const S k = (S)kappa;
     for (int s = sblock * blockDim.x + threadIdx.x; s < g.V; s += nsb * blockDim.x) {
         C acc[12], self[12];
-        if (jb.dagger) hop_site<true, S>(g, U, in, s, acc);
+        if (dagger) hop_site<true, S>(g, U, in, s, acc);
         else hop_site<false, S>(g, U, in, s, acc);
         in.load(s, self);
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = self[c] - k * acc[c];
         if (RES) {
             double2 b[12];
-            Field<double>::load(jb.aux, g.V, s, b);
+            Field<double>::load(aux + off, g.V, s, b);
 #pragma unroll
             for (int c = 0; c < 12; ++c) acc[c] = cvt<S>(b[c] - to_d(acc[c]));
         }
-        Field<S>::store(jb.out, g.V, s, acc);
+        Field<S>::store(reinterpret_cast<C*>(dst) + off, g.V, s, acc);
     }
 }
 
 // -------------------------------------------------------------- pack/unpack
 // Host layout AoS [site][12] complex128 <-> device chunk layout.
+// A block turns PK_SITES sites of one field through shared memory, so that both sides
+// are read and written in whole lines (a site is 13 units apart there: no conflicts).
+// Bound by bytes: 24 or 32 per number; the conversions run on the integer pipe (two per
+// number on the FP64 pipe take as long as the bytes). Element by element, with 64-bit
+// divisions and 16-byte pieces, 4 fields of 24^3 x 64 took 181 us in and 171 out, now
+// 141 and 154 (1.0 GB each way).
+constexpr int PK_SITES = BL_THREADS / 2;
 template <typename S>
-__global__ void pack_kernel(const double2* aos, void* dev, int V, int k) {
-    const size_t total = (size_t)V * 12 * k;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t f = i / ((size_t)V * 12);
-        const size_t r = i % ((size_t)V * 12);
-        const int s = (int)(r / 12), c = (int)(r % 12);
-        const size_t e = f * (size_t)V * 12 + ((size_t)(c >> 1) * V + s) * 2 + (c & 1);
-        st_elem<S>(dev, e, cvt<S>(aos[i]));
+__global__ void __launch_bounds__(BL_THREADS) pack_kernel(const double2* aos, cplx<S>* dev, int V) {
+    __shared__ double2 sm[PK_SITES * 13];
+    const int s0 = blockIdx.x * PK_SITES, ns = V - s0 < PK_SITES ? V - s0 : PK_SITES, t = threadIdx.x;
+    const size_t f = (size_t)blockIdx.y * V * 12;
+    const double2* src = aos + f + (size_t)s0 * 12;
+    double2 v[6];
+#pragma unroll
+    for (int r = 0; r < 6; ++r)
+        if (r * BL_THREADS + t < ns * 12) v[r] = src[r * BL_THREADS + t];
+#pragma unroll
+    for (int r = 0; r < 6; ++r) {
+        const int i = r * BL_THREADS + t;
+        if (i < ns * 12) sm[i / 12 * 13 + i % 12] = v[r];
     }
+    __syncthreads();
+    if (t >= 2 * ns) return;
+#pragma unroll
+    for (int h = 0; h < 6; ++h)
+        dev[f + ((size_t)h * V + s0) * 2 + t] = nar<S>(sm[(t >> 1) * 13 + 2 * h + (t & 1)]);
 }
 template <typename S>
-__global__ void unpack_kernel(const void* dev, double2* aos, int V, int k) {
-    const size_t total = (size_t)V * 12 * k;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t f = i / ((size_t)V * 12);
-        const size_t r = i % ((size_t)V * 12);
-        const int s = (int)(r / 12), c = (int)(r % 12);
-        const size_t e = f * (size_t)V * 12 + ((size_t)(c >> 1) * V + s) * 2 + (c & 1);
-        aos[i] = to_d(ld_elem<S>(dev, e));
+__global__ void __launch_bounds__(BL_THREADS) unpack_kernel(const cplx<S>* dev, double2* aos, int V) {
+    __shared__ double2 sm[PK_SITES * 13];
+    const int s0 = blockIdx.x * PK_SITES, ns = V - s0 < PK_SITES ? V - s0 : PK_SITES, t = threadIdx.x;
+    const size_t f = (size_t)blockIdx.y * V * 12;
+    if (t < 2 * ns) {
+        cplx<S> v[6];
+#pragma unroll
+        for (int h = 0; h < 6; ++h) v[h] = dev[f + ((size_t)h * V + s0) * 2 + t];
+#pragma unroll
+        for (int h = 0; h < 6; ++h) sm[(t >> 1) * 13 + 2 * h + (t & 1)] = wid(v[h]);
+    }
+    __syncthreads();
+    double2* dst = aos + f + (size_t)s0 * 12;
+#pragma unroll
+    for (int r = 0; r < 6; ++r) {
+        const int i = r * BL_THREADS + t;
+        if (i < ns * 12) dst[i] = sm[i / 12 * 13 + i % 12];
     }
 }
 template <typename SI, typename SO>
@@ -1043,17 +1071,17 @@ void count_launches(long long n) { g_launches += n; }
 long long launches_so_far() { return g_launches; }
 void set_launches(long long n) { g_launches = n; }
 
-cudaError_t launch_apply(const Geom& g, const void* links, double kappa, int precision, const ApplyJob* d_jobs,
-                         int njobs, int residual, cudaStream_t st) {
-    int grid = ds_blocks(g.V) * njobs;   // jobs fastest: they share each block's links
+cudaError_t launch_apply(const Geom& g, const void* links, double kappa, int precision, const void* in, void* out,
+                         const double2* aux, int dagger, int nf, cudaStream_t st) {
+    int grid = ds_blocks(g.V) * nf;
     if (precision == 0) {
-        const int t = site_threads(g.V, njobs, DS_THREADS);
-        if (t == 32) grid = div_up(g.V, 32) * njobs;
-        if (residual) apply_kernel<double, true><<<grid, t, 0, st>>>(geom_of(g), links, kappa, d_jobs, njobs);
-        else apply_kernel<double, false><<<grid, t, 0, st>>>(geom_of(g), links, kappa, d_jobs, njobs);
+        const int t = site_threads(g.V, nf, DS_THREADS);
+        if (t == 32) grid = div_up(g.V, 32) * nf;
+        if (aux) apply_kernel<double, true><<<grid, t, 0, st>>>(geom_of(g), links, kappa, in, out, aux, dagger, nf);
+        else apply_kernel<double, false><<<grid, t, 0, st>>>(geom_of(g), links, kappa, in, out, aux, dagger, nf);
     } else {
-        if (residual) return cudaErrorInvalidValue;
-        apply_kernel<float, false><<<grid, DS_THREADS, 0, st>>>(geom_of(g), links, kappa, d_jobs, njobs);
+        if (aux) return cudaErrorInvalidValue;
+        apply_kernel<float, false><<<grid, DS_THREADS, 0, st>>>(geom_of(g), links, kappa, in, out, aux, dagger, nf);
     }
     count_launches(1);
     return cudaGetLastError();
@@ -1073,16 +1101,18 @@ cudaError_t launch_residual32(const Geom& g, const void* links32, double kappa, 
 }
 
 cudaError_t launch_pack(const double* aos, void* dev, int V, int k, int precision, cudaStream_t st) {
-    int nb = blas_blocks((size_t)V * 12 * k);
-    if (precision == 0) pack_kernel<double><<<nb, BL_THREADS, 0, st>>>(reinterpret_cast<const double2*>(aos), dev, V, k);
-    else pack_kernel<float><<<nb, BL_THREADS, 0, st>>>(reinterpret_cast<const double2*>(aos), dev, V, k);
+    const dim3 grid(div_up(V, PK_SITES), k);
+    const double2* src = reinterpret_cast<const double2*>(aos);
+    if (precision == 0) pack_kernel<double><<<grid, BL_THREADS, 0, st>>>(src, reinterpret_cast<double2*>(dev), V);
+    else pack_kernel<float><<<grid, BL_THREADS, 0, st>>>(src, reinterpret_cast<float2*>(dev), V);
     count_launches(1);
     return cudaGetLastError();
 }
 cudaError_t launch_unpack(const void* dev, double* aos, int V, int k, int precision, cudaStream_t st) {
-    int nb = blas_blocks((size_t)V * 12 * k);
-    if (precision == 0) unpack_kernel<double><<<nb, BL_THREADS, 0, st>>>(dev, reinterpret_cast<double2*>(aos), V, k);
-    else unpack_kernel<float><<<nb, BL_THREADS, 0, st>>>(dev, reinterpret_cast<double2*>(aos), V, k);
+    const dim3 grid(div_up(V, PK_SITES), k);
+    double2* dst = reinterpret_cast<double2*>(aos);
+    if (precision == 0) unpack_kernel<double><<<grid, BL_THREADS, 0, st>>>(reinterpret_cast<const double2*>(dev), dst, V);
+    else unpack_kernel<float><<<grid, BL_THREADS, 0, st>>>(reinterpret_cast<const float2*>(dev), dst, V);
     count_launches(1);
     return cudaGetLastError();
 }

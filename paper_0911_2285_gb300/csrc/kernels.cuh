@@ -30,16 +30,11 @@ struct EoJob {
     int dagger;
 };
 
-struct ApplyJob {            // out = A in, A^+ in, or aux - A in
-    const void* in;
-    void* out;
-    const void* aux;         // FP64 b for the residual form
-    int dagger;
-};
-
-// precision: 0 = FP64 storage/arith (FP64 links), 1 = FP32 storage/arith (FP32 links)
-cudaError_t launch_apply(const Geom& g, const void* links, double kappa, int precision,
-                         const ApplyJob* d_jobs, int njobs, int residual, cudaStream_t st);
+// out_j = A in_j (A^+ in_j when dagger; aux_j - A in_j when aux, FP64 only) for nf
+// consecutive fields. precision: 0 = FP64 storage/arith (FP64 links), 1 = FP32
+// storage/arith (FP32 links).
+cudaError_t launch_apply(const Geom& g, const void* links, double kappa, int precision, const void* in, void* out,
+                         const double2* aux, int dagger, int nf, cudaStream_t st);
 
 // r = b - A x for nf consecutive FP64 fields with the hop in FP32 on FP32 links; x32:
 // FP32 scratch of nf fields (receives x); rprec: storage of r (0 = FP64, 1 = FP32).

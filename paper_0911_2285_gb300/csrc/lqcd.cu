@@ -126,7 +126,6 @@ struct lqcd_ctx {
     int* ritz_n = nullptr;          // per slot: number of final Ritz pairs
     double2* mdscratch = nullptr;
     size_t mdscratch_elems = 0;
-    ApplyJob* d_jobs = nullptr;
     double2* staging = nullptr;     // kmax FP64 full fields (host AoS I/O)
     // even-odd (Schur complement) operator: the solver works on the odd half
     // lattice (N = 6 V); sources and solutions stay full fields (Nfull = 12 V)
@@ -503,7 +502,6 @@ extern "C" lqcd_status lqcd_eigbicg_init(lqcd_ctx** out, const lqcd_params* para
     AL(c->ritz_all, (size_t)MAX_SLOTS * RITZ_STRIDE * 16);
     AL(c->ritz_n, MAX_SLOTS * sizeof(int));
     AL(c->mdscratch, c->mdscratch_elems * 16);
-    AL(c->d_jobs, sizeof(ApplyJob) * 2 * K);
     AL(c->staging, K * c->Nfull * 16);
     if (c->eo) {
         AL(c->bfull_all, K * c->Nfull * 16);
@@ -687,8 +685,8 @@ lqcd_status download(lqcd_ctx* c, const void* src, int prec, int k, double* dst,
 // out_j = A in_j (or A^+, or b_j - A in_j) for nf device fields in precision prec:
 // the solver's operator (A_hat on the odd half lattice in an even-odd context),
 // or with full = true the full-lattice A (fields of Nfull complex).
-lqcd_status apply_fields(lqcd_ctx* c, int prec, int dagger, int nf, const void* in, size_t in_stride, void* out,
-                         size_t out_stride, const double2* aux, bool full = false) {
+lqcd_status apply_fields(lqcd_ctx* c, int prec, int dagger, int nf, const void* in, void* out, const double2* aux,
+                         bool full = false) {
     const void* links = prec ? (const void*)c->links32 : (const void*)c->links64;
     if (prec && !c->links32) return LQCD_ERR_ARG;
     if (c->eo && !full) {   // two stages through the half-field scratch
@@ -697,10 +695,10 @@ lqcd_status apply_fields(lqcd_ctx* c, int prec, int dagger, int nf, const void* 
         for (int j0 = 0; j0 < nf; j0 += 2 * c->kmax) {
             const int nb = std::min(2 * c->kmax, nf - j0);
             for (int j = 0; j < nb; ++j) {
-                const char* fin = reinterpret_cast<const char*>(in) + (j0 + j) * in_stride;
+                const char* fin = reinterpret_cast<const char*>(in) + (j0 + j) * sb;
                 char* scr = c->eo_scr + (size_t)j * sb;
                 st1[j] = EoJob{fin, nullptr, scr, nullptr, dagger};
-                st2[j] = EoJob{scr, fin, reinterpret_cast<char*>(out) + (j0 + j) * out_stride,
+                st2[j] = EoJob{scr, fin, reinterpret_cast<char*>(out) + (j0 + j) * sb,
                                aux ? aux + (size_t)(j0 + j) * c->N : nullptr, dagger};
             }
             CK(cudaMemcpyAsync(c->d_eojobs, st1.data(), sizeof(EoJob) * nb, cudaMemcpyHostToDevice, c->stream));
@@ -712,21 +710,7 @@ lqcd_status apply_fields(lqcd_ctx* c, int prec, int dagger, int nf, const void* 
         }
         return LQCD_OK;
     }
-    const size_t an = full ? c->Nfull : c->N;
-    std::vector<ApplyJob> jobs(2 * c->kmax);
-    for (int j0 = 0; j0 < nf; j0 += 2 * c->kmax) {
-        const int nb = std::min(2 * c->kmax, nf - j0);
-        for (int j = 0; j < nb; ++j) {
-            jobs[j].in = reinterpret_cast<const char*>(in) + (j0 + j) * in_stride;
-            jobs[j].out = reinterpret_cast<char*>(out) + (j0 + j) * out_stride;
-            jobs[j].aux = aux ? aux + (size_t)(j0 + j) * an : nullptr;
-            jobs[j].dagger = dagger;
-        }
-        CK(cudaMemcpyAsync(c->d_jobs, jobs.data(), sizeof(ApplyJob) * nb, cudaMemcpyHostToDevice, c->stream));
-        CK(launch_apply(c->g, links, c->p.kappa, prec, c->d_jobs, nb, aux != nullptr, c->stream));
-        // the job table is reused: wait before overwriting it
-        CK(cudaStreamSynchronize(c->stream));
-    }
+    CK(launch_apply(c->g, links, c->p.kappa, prec, in, out, aux, dagger, nf, c->stream));
     return LQCD_OK;
 }
 
@@ -741,7 +725,7 @@ lqcd_status residual_fields(lqcd_ctx* c, int s0, int nf, bool precise = false, b
     const double2* x = c->x_hi_all + (size_t)s0 * c->N;
     const double2* b = c->b_all + (size_t)s0 * c->N;
     double2* r = c->rt_all + (size_t)s0 * c->N;
-    if (!residual_in_fp32(c, precise)) return apply_fields(c, 0, 0, nf, x, c->dbytes, r, c->dbytes, b);
+    if (!residual_in_fp32(c, precise)) return apply_fields(c, 0, 0, nf, x, r, b);
     CK(launch_residual32(c->g, c->links32, c->p.kappa, x, c->krylov(c->x_lo_all, s0), b, r, fp32 ? 1 : 0, nf, c->stream));
     return LQCD_OK;
 }
@@ -780,7 +764,7 @@ lqcd_status store_solutions(lqcd_ctx* c, int s0, int k, double* x, int on_device
     CK(launch_eo_reconstruct(c->g, c->links64, c->p.kappa, bf, c->x_hi_all + (size_t)s0 * c->N, xf, k, c->stream));
     if (resid) {
         double2* rf = reinterpret_cast<double2*>(c->eo_scr);   // room for kmax full FP64 fields
-        lqcd_status s = apply_fields(c, 0, 0, k, xf, c->Nfull * 16, rf, c->Nfull * 16, bf, true);
+        lqcd_status s = apply_fields(c, 0, 0, k, xf, rf, bf, true);
         if (s != LQCD_OK) return s;
         double* rn = reinterpret_cast<double*>(c->dsmall);
         CK(launch_norms(k, rf, 0, c->Nfull, rn, c->mdscratch, c->mdscratch_elems, c->stream));
@@ -809,10 +793,9 @@ extern "C" lqcd_status lqcd_apply(lqcd_ctx* c, int dagger, lqcd_precision prec, 
         const int kb = std::min(c->kmax, k - j0);
         void* fin = pr ? (void*)c->x_lo_all : (void*)c->x_hi_all;
         void* fout = pr ? (void*)c->vw_base : (void*)c->rt_all;
-        const size_t fb = c->N * (pr ? 8 : 16);
         lqcd_status s = upload(c, in + (size_t)j0 * 2 * c->N, kb, fin, pr, on_device);
         if (s != LQCD_OK) return s;
-        s = apply_fields(c, pr, dagger ? 1 : 0, kb, fin, fb, fout, fb, nullptr);
+        s = apply_fields(c, pr, dagger ? 1 : 0, kb, fin, fout, nullptr);
         if (s != LQCD_OK) return s;
         s = download(c, fout, pr, kb, out + (size_t)j0 * 2 * c->N, on_device);
         if (s != LQCD_OK) return s;
@@ -1006,9 +989,9 @@ lqcd_status grow_space(lqcd_ctx* c, int nn, void* work) {
     // projections are FP32 sums as well, and lqcd_eigs recomputes its pencil in FP64)
     char* AV = reinterpret_cast<char*>(work);
     char* AW = AV + (size_t)2 * kk * c->kbytes;
-    lqcd_status s = apply_fields(c, kp, 0, kk, Vn, c->kbytes, AV, c->kbytes, nullptr);
+    lqcd_status s = apply_fields(c, kp, 0, kk, Vn, AV, nullptr);
     if (s != LQCD_OK) return s;
-    s = apply_fields(c, kp, 1, kk, Wn, c->kbytes, AW, c->kbytes, nullptr);
+    s = apply_fields(c, kp, 1, kk, Wn, AW, nullptr);
     if (s != LQCD_OK) return s;
     CK(cudaMemcpyAsync(AV + (size_t)kk * c->kbytes, Vn, (size_t)kk * c->kbytes, cudaMemcpyDeviceToDevice, c->stream));
     CK(cudaMemcpyAsync(AW + (size_t)kk * c->kbytes, Wn, (size_t)kk * c->kbytes, cudaMemcpyDeviceToDevice, c->stream));
@@ -1415,7 +1398,7 @@ lqcd_status project_fp64(lqcd_ctx* c, int n, double2* Hout, double2* Mout, int l
             CK(launch_convert(src, 1, c->x_hi_all, 0, (size_t)kb * c->N, c->stream));
             in = c->x_hi_all;
         }
-        lqcd_status s = apply_fields(c, 0, 0, kb, in, c->kprec ? c->dbytes : c->kbytes, c->rt_all, c->dbytes, nullptr);
+        lqcd_status s = apply_fields(c, 0, 0, kb, in, c->rt_all, nullptr);
         if (s != LQCD_OK) return s;
         CK(launch_multidot(n, c->Ul, c->kprec, kb, c->rt_all, 0, c->N, Hout + j0, ld, 0, c->mdscratch,
                            c->mdscratch_elems, c->stream, c->d_err, c->use_tc));
@@ -1509,7 +1492,7 @@ extern "C" lqcd_status lqcd_eigs(lqcd_ctx* c, int* n_inout, double* evals, doubl
         }
         if (resid) {
             // r_j = A u_j - lam_j u_j ; |r_j| / |u_j|
-            lqcd_status s = apply_fields(c, 0, 0, kb, c->x_hi_all, c->dbytes, c->rt_all, c->dbytes, nullptr);
+            lqcd_status s = apply_fields(c, 0, 0, kb, c->x_hi_all, c->rt_all, nullptr);
             if (s != LQCD_OK) return s;
             double2* D = c->dsmall + (size_t)MAX_SMALL * MAX_SMALL * 6;
             std::vector<double2> hd((size_t)kb * kb, make_double2(0, 0));

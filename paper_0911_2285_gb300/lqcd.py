@@ -361,7 +361,7 @@ class Solver:
         """``A v`` (``A^+ v``) on the solver's space: the full lattice, or A_hat on the
         odd half lattice of an even-odd context."""
         v = _as_batch(v, self.n_space)
-        out = _zeros_like(v)
+        out = _empty_like(v)   # the call writes all of it, or raises
         pv, po, dv = self._fields(v, out)
         _check(lib().lqcd_apply(self._h, int(dagger), _PREC[precision], v.shape[0], pv, po, dv), "lqcd_apply")
         return out
@@ -499,6 +499,16 @@ def _zeros_like(a):
     except ImportError:  # pragma: no cover
         pass
     return np.zeros_like(a)
+
+
+def _empty_like(a):
+    try:
+        import torch
+        if isinstance(a, torch.Tensor):
+            return torch.empty_like(a)
+    except ImportError:  # pragma: no cover
+        pass
+    return np.empty_like(a)
 
 
 def kernel_launches():
