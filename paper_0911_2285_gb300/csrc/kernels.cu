@@ -23,7 +23,8 @@ inline int div_up(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 // Threads per block of the FP64 site and vector kernels: the FP64 pipe of an SM serves
 // 2 lanes per clock, so what matters is how many SMs take part. Below two blocks of
 // the full size per SM, one-warp blocks spread the same warps over the chip: operator
-// pair on 4^4 (16 warps) 42 us on 4 SMs.
+// pair on 4^4 (16 warps) 42 us on 4 SMs, 36 on 16. The smallest operator grids go to
+// fp64_split.cu.
 constexpr int SMALL_GRID = 2 * 152;
 int site_threads(size_t sites, int jobs, int full) { return (sites + full - 1) / full * jobs < SMALL_GRID ? 32 : full; }
 
@@ -1074,6 +1075,10 @@ void set_launches(long long n) { g_launches = n; }
 cudaError_t launch_apply(const Geom& g, const void* links, double kappa, int precision, const void* in, void* out,
                          const double2* aux, int dagger, int nf, cudaStream_t st) {
     int grid = ds_blocks(g.V) * nf;
+    if (precision == 0 && fp64_split_ok(g.V, nf)) {
+        count_launches(1);
+        return launch_apply_split(g, links, kappa, in, out, aux, dagger, nf, st);
+    }
     if (precision == 0) {
         const int t = site_threads(g.V, nf, DS_THREADS);
         if (t == 32) grid = div_up(g.V, 32) * nf;
@@ -1254,7 +1259,10 @@ cudaError_t launch_bicg_matvec(const Geom& g, const void* links, double kappa, i
     if (prec != 0 && variant >= 25 && variant < 30)   // 4-D bricks, every slot per block (dslash_brick.cu)
         return launch_matvec_brick(g, links, kappa, states, ptrs, nslots, s, variant);
     if (prec == 0) {
-        if (site_threads(g.V, 2 * nslots, 128) == 32) matvec_launch<double, 32, 8, false>(g, links, kappa, states, ptrs, nslots, s);
+        if (fp64_split_ok(g.V, 2 * nslots)) {
+            const cudaError_t e = launch_matvec_split(g, links, kappa, states, ptrs, nslots, s);
+            if (e != cudaSuccess) return e;
+        } else if (site_threads(g.V, 2 * nslots, 128) == 32) matvec_launch<double, 32, 8, false>(g, links, kappa, states, ptrs, nslots, s);
         else matvec_launch<double, 128, 1, false>(g, links, kappa, states, ptrs, nslots, s);
     } else {
         switch (variant) {

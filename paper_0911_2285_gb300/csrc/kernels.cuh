@@ -36,6 +36,14 @@ struct EoJob {
 cudaError_t launch_apply(const Geom& g, const void* links, double kappa, int precision, const void* in, void* out,
                          const double2* aux, int dagger, int nf, cudaStream_t st);
 
+// FP64 operator and operator pair with a site's eight terms on eight threads, for
+// grids that leave most of the chip idle (fp64_split.cu).
+bool fp64_split_ok(size_t V, int jobs);
+cudaError_t launch_apply_split(const Geom& g, const void* links64, double kappa, const void* in, void* out,
+                               const double2* aux, int dagger, int nf, cudaStream_t st);
+cudaError_t launch_matvec_split(const Geom& g, const void* links64, double kappa, SlotState* states, const SlotPtrs* ptrs,
+                                int nslots, cudaStream_t st);
+
 // r = b - A x for nf consecutive FP64 fields with the hop in FP32 on FP32 links; x32:
 // FP32 scratch of nf fields (receives x); rprec: storage of r (0 = FP64, 1 = FP32).
 cudaError_t launch_residual32(const Geom& g, const void* links32, double kappa, const double2* x, void* x32,
