@@ -9,6 +9,49 @@ constexpr int RED_MAX_THREADS = 256;   // blocks that reduce have at most this m
 
 __device__ __forceinline__ double2* part(const SlotPtrs& P, int kind) { return P.partials + (size_t)kind * PARTIAL_STRIDE; }
 
+// NR numbers per lane summed over the warp: each of the first steps halves the numbers
+// that a lane holds, the lane's bit says which half it keeps; lane l returns the sum
+// number l / (32 / NR). NR = 4: 6 additions where the sums one by one take 20, each of
+// them 64 clocks of the FP64 pipe.
+template <int NR> __device__ __forceinline__ double lane_sums(const double (&r)[NR]) {
+    static_assert(NR == 2 || NR == 4, "numbers per lane");
+    const int lane = threadIdx.x & 31;
+    const bool u16 = lane & 16, u8 = lane & 8;
+    double t;
+    if constexpr (NR == 4) {
+        const double a = (u16 ? r[2] : r[0]) + __shfl_xor_sync(0xffffffffu, u16 ? r[0] : r[2], 16);
+        const double b = (u16 ? r[3] : r[1]) + __shfl_xor_sync(0xffffffffu, u16 ? r[1] : r[3], 16);
+        t = (u8 ? b : a) + __shfl_xor_sync(0xffffffffu, u8 ? a : b, 8);
+    } else {
+        t = (u16 ? r[1] : r[0]) + __shfl_xor_sync(0xffffffffu, u16 ? r[0] : r[1], 16);
+        t += __shfl_xor_sync(0xffffffffu, t, 8);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+// block_sum of FP64 values by that; v valid in thread 0. smem: 2 NV values per warp.
+template <int NV> __device__ __forceinline__ void block_sum_fp64(double2 (&v)[NV], double* smem) {
+    constexpr int NR = 2 * NV;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double r[NR];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) { r[2 * i] = v[i].x; r[2 * i + 1] = v[i].y; }
+    const double t = lane_sums<NR>(r);
+    __syncthreads();
+    if (lane % (32 / NR) == 0) smem[w * NR + lane / (32 / NR)] = t;
+    __syncthreads();
+    if (w == 0) {
+        double s = lane < nw * NR ? smem[lane] : 0.0;   // number l % NR of warp l / NR: at most 8 warps of 4
+#pragma unroll
+        for (int o = 16; o >= NR; o >>= 1)
+            if (o < nw * NR) s += __shfl_xor_sync(0xffffffffu, s, o);
+#pragma unroll
+        for (int i = 0; i < NV; ++i)
+            v[i] = make_double2(__shfl_sync(0xffffffffu, s, 2 * i), __shfl_sync(0xffffffffu, s, 2 * i + 1));
+    }
+}
+
 // Sum NV complex values per block into part[kind][block*NV + i]; in the last
 // block returns true with tot[] = sum over blocks (thread 0 only). The block
 // sum runs in the precision of v (FP32 for the mixed solver), the cross-block
@@ -18,7 +61,8 @@ __device__ bool reduce_slot(const SlotPtrs& P, int kind, C (&v)[NV], double2 (&t
                             unsigned bid) {
     __shared__ C sm[(RED_MAX_THREADS / 32) * NV];   // blockDim.x <= RED_MAX_THREADS
     __shared__ double2 smd[(RED_MAX_THREADS / 32) * NV];
-    block_sum<NV>(v, sm);
+    if constexpr (sizeof(C) == 16) block_sum_fp64<NV>(v, reinterpret_cast<double*>(sm));
+    else block_sum<NV>(v, sm);
     double2* pp = part(P, kind);
     if (threadIdx.x == 0) {
 #pragma unroll
