@@ -11,8 +11,8 @@ more (the launches an ncu capture skips to). ``eopair``: the even-odd (Schur
 complement) operator pair A_hat p, A_hat^+ phat on the odd half lattice for k
 slots (two stage kernels per pair): one warm-up pair, reps timed, one more.
 ``dots``: the inner-product matrix
-X^H Y of FP32 fields on the tensor cores and on the CUDA cores; the last launch
-is one more tensor-core call. ``restart``: eigBiCG on k sources stopped a few
+X^H Y of FP32 fields by the staged path and by the path 0 kernel; the last launch
+is one more staged call. ``restart``: eigBiCG on k sources stopped a few
 iterations after the first window restart (the m-th iteration launches the
 tensor-core restart product that does work). Inputs are seeded synthetic fields.
 """
@@ -102,7 +102,7 @@ def main(argv=None):
         gb = (args.a + args.b) * args.n * 8 / 1e9
         _, t1 = field_dots(X, Y, path=1, reps=args.reps)
         _, t0 = field_dots(X, Y, path=0, reps=args.reps)
-        print(f"X^H Y {args.a}x{args.b}, n={args.n}: tensor cores {t1:.4f} ms ({gb / t1 * 1e3:.0f} GB/s), "
+        print(f"X^H Y {args.a}x{args.b}, n={args.n}: staged {t1:.4f} ms ({gb / t1 * 1e3:.0f} GB/s), "
               f"CUDA cores {t0:.4f} ms ({gb / t0 * 1e3:.0f} GB/s)")
         field_dots(X, Y, path=1)
 

@@ -24,7 +24,7 @@
 // output each), a rotation costs two barriers, and shifts, deflation scans,
 // norms, pivot searches and substitutions run across the lanes of a warp.
 // Measured: restart coefficients (both eigen-solves and the FP64 finish) 60 x 60
-// 20.2 -> 4.6 ms, 40 x 40 10.9 -> 2.5 ms; FP64 eigen-solve 60 x 60 18.2 -> 10.9 ms.
+// 20.2 -> 5.0 ms, 40 x 40 10.9 -> 2.7 ms; FP64 eigen-solve 60 x 60 18.2 -> 10.9 ms.
 #include <mutex>
 
 #include "../../include/lqcd.h"
