@@ -20,7 +20,8 @@ constexpr int G5_STALL = 200;     // iterations without a reliable update after 
 
 inline int div_up(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 
-// Threads per block of the FP64 site and vector kernels: the FP64 pipe of an SM serves
+// Threads per block of the FP64 site and vector kernels (jobs: of a full batch, so that
+// a source's sums are the same alone and in a batch of its context): the FP64 pipe of an SM serves
 // 2 lanes per clock, so what matters is how many SMs take part. Below two blocks of
 // the full size per SM, one-warp blocks spread the same warps over the chip: operator
 // pair on 4^4 (16 warps) 42 us on 4 SMs, 36 on 16. The smallest operator grids go to
@@ -1254,15 +1255,16 @@ bool matvec_variant_ok(const Geom& g, int v) {
 }
 
 cudaError_t launch_bicg_matvec(const Geom& g, const void* links, double kappa, int prec, SlotState* states,
-                               const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant) {
+                               const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant,
+                                  int kmax) {
     if (prec != 0 && variant == STAGED_VARIANT) return cudaErrorInvalidValue;   // needs the context's tensor maps
     if (prec != 0 && variant >= 25 && variant < 30)   // 4-D bricks, every slot per block (dslash_brick.cu)
         return launch_matvec_brick(g, links, kappa, states, ptrs, nslots, s, variant);
     if (prec == 0) {
-        if (fp64_split_ok(g.V, 2 * nslots)) {
+        if (fp64_split_ok(g.V, 2 * kmax)) {
             const cudaError_t e = launch_matvec_split(g, links, kappa, states, ptrs, nslots, s);
             if (e != cudaSuccess) return e;
-        } else if (site_threads(g.V, 2 * nslots, 128) == 32) matvec_launch<double, 32, 8, false>(g, links, kappa, states, ptrs, nslots, s);
+        } else if (site_threads(g.V, 2 * kmax, 128) == 32) matvec_launch<double, 32, 8, false>(g, links, kappa, states, ptrs, nslots, s);
         else matvec_launch<double, 128, 1, false>(g, links, kappa, states, ptrs, nslots, s);
     } else {
         switch (variant) {
@@ -1309,9 +1311,10 @@ bool matvec_g5_variant_ok(const Geom& g, int v) {
 }
 
 cudaError_t launch_bicg_matvec_g5(const Geom& g, const void* links, double kappa, int prec, SlotState* states,
-                                  const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant) {
+                                  const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant,
+                                  int kmax) {
     if (prec == 0) {
-        if (site_threads(g.V, nslots, 128) == 32) matvec_launch<double, 32, 8, false, 0, 1, true>(g, links, kappa, states, ptrs, nslots, s);
+        if (site_threads(g.V, kmax, 128) == 32) matvec_launch<double, 32, 8, false, 0, 1, true>(g, links, kappa, states, ptrs, nslots, s);
         else matvec_launch<double, 128, 1, false, 0, 1, true>(g, links, kappa, states, ptrs, nslots, s);
     } else {
         switch (variant) {
@@ -1331,9 +1334,10 @@ cudaError_t launch_bicg_matvec_g5(const Geom& g, const void* links, double kappa
     return cudaGetLastError();
 }
 
-cudaError_t launch_bicg_update(int prec, SlotState* states, const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s) {
+cudaError_t launch_bicg_update(int prec, SlotState* states, const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s,
+                               int kmax) {
     dim3 grid(blas_blocks(N / 2), nslots);
-    const int t = site_threads(N / 2, nslots, BL_THREADS);
+    const int t = site_threads(N / 2, kmax, BL_THREADS);
     if (prec == 0) update_kernel<double><<<t == 32 ? dim3(blas_blocks(N / 2 * (BL_THREADS / 32)), nslots) : grid, t, 0, s>>>(states, ptrs, N);
     else update_kernel<float><<<grid, BL_THREADS, 0, s>>>(states, ptrs, N);
     count_launches(1);

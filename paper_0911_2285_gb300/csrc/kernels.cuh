@@ -132,13 +132,15 @@ constexpr int STAGED_VARIANT = 26;
 bool brick_variant_ok(const Geom& g, int v);
 cudaError_t launch_matvec_brick(const Geom& g, const void* links, double kappa, SlotState* states,
                                 const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant);
+// kmax: slots of the context; FP64 shapes go by it, not by nslots, so that a source's
+// sums are the same alone and in a batch.
 cudaError_t launch_bicg_matvec(const Geom& g, const void* links, double kappa, int prec,
-                               SlotState* st_, const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant);
+                               SlotState* st_, const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant, int kmax);
 // gamma5 variant (Sec. 4): A p only, phat = gamma5 p; shapes v with matvec_g5_variant_ok.
 bool matvec_g5_variant_ok(const Geom& g, int v);
 cudaError_t launch_bicg_matvec_g5(const Geom& g, const void* links, double kappa, int prec,
-                                  SlotState* st_, const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant);
-cudaError_t launch_bicg_update(int prec, SlotState* st_, const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s);
+                                  SlotState* st_, const SlotPtrs* ptrs, int nslots, cudaStream_t s, int variant, int kmax);
+cudaError_t launch_bicg_update(int prec, SlotState* st_, const SlotPtrs* ptrs, int nslots, size_t N, cudaStream_t s, int kmax);
 // FP64 residual of the started slots at the end of a solve, in one of
 // true_resid_variants() kernel shapes (timed at init).
 int true_resid_variants();

@@ -1057,7 +1057,7 @@ cudaError_t launch_matvec(lqcd_ctx* c, int nslots, int variant) {
     if (c->p.gamma5) {
         const void* links = c->kprec ? (const void*)c->links32 : (const void*)c->links64;
         return launch_bicg_matvec_g5(c->g, links, c->p.kappa, c->kprec, c->d_state, c->d_ptrs, nslots, c->stream,
-                                     variant);
+                                     variant, c->kmax);
     }
     if (variant == TILED && c->tile_ok[nslots])
         return launch_matvec_tiled(c->g, c->tgeo[nslots], c->links32, c->p.kappa, c->d_state, c->d_ptrs, c->d_err,
@@ -1067,7 +1067,7 @@ cudaError_t launch_matvec(lqcd_ctx* c, int nslots, int variant) {
                                     c->stream);
     const void* links = c->kprec ? (const void*)c->links32 : (const void*)c->links64;
     return launch_bicg_matvec(c->g, links, c->p.kappa, c->kprec, c->d_state, c->d_ptrs, nslots, c->stream,
-                              variant == TILED ? 0 : variant);
+                              variant == TILED ? 0 : variant, c->kmax);
 }
 
 // The reliable update of an iteration (a no-op for slots that need none).
@@ -1094,7 +1094,7 @@ lqcd_status enqueue_chunk(lqcd_ctx* c, int nslots, int kinds) {
                 else
                     CK(launch_window_gemm(c->kprec, 2 * c->nev, c->d_state, c->d_ptrs, nslots, c->N, c->stream));
             }
-            CK(launch_bicg_update(c->kprec, c->d_state, c->d_ptrs, nslots, c->N, c->stream));
+            CK(launch_bicg_update(c->kprec, c->d_state, c->d_ptrs, nslots, c->N, c->stream, c->kmax));
             CK(launch_ru(c, nslots));
             CK(launch_bicg_direction(c->kprec, c->d_state, c->d_ptrs, nslots, c->N, c->stream));
         }
@@ -1693,7 +1693,7 @@ static lqcd_status time_kernel_impl(lqcd_ctx* c, int kernel, int k, int reps, do
         else if (kernel == 0) CK(launch_matvec(c, k, c->dslash_variant));
         else if (kernel == TIME_TILED) CK(launch_matvec(c, k, TILED));
         else if (kernel >= 10) CK(launch_matvec(c, k, kernel - 10));
-        else if (kernel == 1) CK(launch_bicg_update(c->kprec, c->d_state, c->d_ptrs, k, c->N, c->stream));
+        else if (kernel == 1) CK(launch_bicg_update(c->kprec, c->d_state, c->d_ptrs, k, c->N, c->stream, c->kmax));
         else if (kernel == 2) CK(launch_bicg_direction(c->kprec, c->d_state, c->d_ptrs, k, c->N, c->stream));
         else CK(launch_ru(c, k));
         CK(cudaEventRecord(e1, c->stream));

@@ -35,6 +35,8 @@ namespace lqcd {
 namespace {
 
 constexpr int RU_THREADS = 128;
+constexpr int RU_RUNS = 4096;   // partial sums per slot at most (24^3 x 64: 3456 of two units)
+static_assert(2 * RU_RUNS <= PARTIAL_STRIDE, "partials of a slot");
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     unsigned v;
@@ -232,95 +234,99 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
         if (threadIdx.x == 0) atomicExch(err, 1);
         return;
     }
-    // Residual, its norm, the new r and rho. The blocks share the slots' sites in equal
-    // runs of RU_THREADS-site units; a run that ends in another slot is cut there.
+    // Residual, its norm, the new r and rho. A slot's sites are RU_THREADS-site units, its
+    // units runs of `per` with one partial sum each: both follow from the lattice alone, so
+    // the sums of a source do not depend on the grid or on the other slots. The blocks
+    // share the slots' runs equally.
     const int nunits = (Vs + RU_THREADS - 1) / RU_THREADS;
-    const long long T = (long long)nact * nunits;
+    const int per = (nunits + RU_RUNS - 1) / RU_RUNS, nruns = (nunits + per - 1) / per;
+    const long long T = (long long)nact * nruns;
     const long long t0 = blockIdx.x * T / gridDim.x, t1 = (blockIdx.x + 1) * T / gridDim.x;
-    __shared__ double2 smd[RU_THREADS / 32 * 2];
+    __shared__ double smd[RU_THREADS / 32 * 4];
     const double kk = MODE == RU_EO ? kappa * kappa : kappa;
     for (int i = 0; i < nact; ++i) {
         const SlotState& st = states[list[i]];
         const SlotPtrs& P = ptrs[list[i]];
-        const long long u0 = max(t0 - (long long)i * nunits, 0ll), u1 = min(t1 - (long long)i * nunits, (long long)nunits);
+        const int q0 = (int)max(t0 - (long long)i * nruns, 0ll), q1 = (int)min(t1 - (long long)i * nruns, (long long)nruns);
         void* rcur = slot_field<S>(P.V, next_slot(st), N);
         void* hcur = slot_field<S>(P.W, next_slot(st), N);
         const bool g5 = st.g5 != 0, win = st.m > 0, comp = g5 && sizeof(S) == 4;
-        double nrm = 0.0;
-        cplx<S> rho = mk<S>(S(0), S(0));
-        CompC cz;
-        for (long long u = u0; u < u1; ++u) {
-            const int s = (int)u * RU_THREADS + (int)threadIdx.x;
-            if (s >= Vs) continue;
-            double2 r[12];
-            if constexpr (MODE == RU_DF) {
-                Dot2 ax[12], ay[12];
-                hop_site_df(g, links_df, P.x_df, s, ax, ay);
-                const LiveField xin{P.x_hi, Vs}, bin{P.b, Vs};
-                double2 self[12];
-                xin.load(s, self);
-                bin.load(s, r);
+        for (int q = q0; q < q1; ++q) {
+            double nrm = 0.0;
+            cplx<S> rho = mk<S>(S(0), S(0));
+            CompC cz;
+            for (int u = q * per; u < min(q * per + per, nunits); ++u) {
+                const int s = u * RU_THREADS + (int)threadIdx.x;
+                if (s >= Vs) continue;
+                double2 r[12];
+                if constexpr (MODE == RU_DF) {
+                    Dot2 ax[12], ay[12];
+                    hop_site_df(g, links_df, P.x_df, s, ax, ay);
+                    const LiveField xin{P.x_hi, Vs}, bin{P.b, Vs};
+                    double2 self[12];
+                    xin.load(s, self);
+                    bin.load(s, r);
 #pragma unroll
-                for (int c = 0; c < 12; ++c) {   // b - x + kappa D x, the FP64 part of it 4 instructions per real
-                    r[c].x = fma(kk, widen(ax[c].s), fma(kk, widen(ax[c].c), r[c].x - self[c].x));
-                    r[c].y = fma(kk, widen(ay[c].s), fma(kk, widen(ay[c].c), r[c].y - self[c].y));
+                    for (int c = 0; c < 12; ++c) {   // b - x + kappa D x, the FP64 part of it 4 instructions per real
+                        r[c].x = fma(kk, widen(ax[c].s), fma(kk, widen(ax[c].c), r[c].x - self[c].x));
+                        r[c].y = fma(kk, widen(ay[c].s), fma(kk, widen(ay[c].c), r[c].y - self[c].y));
+                    }
+                } else {
+                    const LinksD U{links64, g.V};
+                    double2 acc[12], self[12];
+                    if constexpr (MODE == RU_EO) hop_site<false, double>(g, U, LiveHalf{P.eo64, Vs}, eo_site(g, s, 1), acc);
+                    else hop_site<false, double>(g, U, LiveField{P.x_hi, Vs}, s, acc);
+                    LiveField{P.x_hi, Vs}.load(s, self);
+                    LiveField{P.b, Vs}.load(s, r);
+#pragma unroll
+                    for (int c = 0; c < 12; ++c)
+                        r[c] = r[c] - make_double2(fma(-kk, acc[c].x, self[c].x), fma(-kk, acc[c].y, self[c].y));
                 }
-            } else {
-                const LinksD U{links64, g.V};
-                double2 acc[12], self[12];
-                if constexpr (MODE == RU_EO) hop_site<false, double>(g, U, LiveHalf{P.eo64, Vs}, eo_site(g, s, 1), acc);
-                else hop_site<false, double>(g, U, LiveField{P.x_hi, Vs}, s, acc);
-                LiveField{P.x_hi, Vs}.load(s, self);
-                LiveField{P.b, Vs}.load(s, r);
+                cplx<S> rs[12], hs[12];
 #pragma unroll
-                for (int c = 0; c < 12; ++c)
-                    r[c] = r[c] - make_double2(fma(-kk, acc[c].x, self[c].x), fma(-kk, acc[c].y, self[c].y));
-            }
-            cplx<S> rs[12], hs[12];
-#pragma unroll
-            for (int c = 0; c < 12; ++c) {
-                nrm = fma(r[c].x, r[c].x, fma(r[c].y, r[c].y, nrm));
-                rs[c] = nar<S>(r[c]);
-            }
-            Field<S>::store(rcur, Vs, s, rs);
-            if (g5) {   // the shadow residual follows: rhat = gamma5 r
-#pragma unroll
-                for (int c = 0; c < 12; ++c) hs[c] = c < 6 ? rs[c] : -rs[c];
-                if (win) Field<S>::store(hcur, Vs, s, hs);
-            } else {
-                Field<S>::load(hcur, Vs, s, hs);
-            }
-            if (comp) {
-                if constexpr (sizeof(S) == 4) {
-#pragma unroll
-                    for (int c = 0; c < 12; ++c) cz.add(cdot(hs[c], rs[c]));
+                for (int c = 0; c < 12; ++c) {
+                    nrm = fma(r[c].x, r[c].x, fma(r[c].y, r[c].y, nrm));
+                    rs[c] = nar<S>(r[c]);
                 }
-            } else {
+                Field<S>::store(rcur, Vs, s, rs);
+                if (g5) {   // the shadow residual follows: rhat = gamma5 r
 #pragma unroll
-                for (int c = 0; c < 12; ++c) rho = cdot_acc(rho, hs[c], rs[c]);
+                    for (int c = 0; c < 12; ++c) hs[c] = c < 6 ? rs[c] : -rs[c];
+                    if (win) Field<S>::store(hcur, Vs, s, hs);
+                } else {
+                    Field<S>::load(hcur, Vs, s, hs);
+                }
+                if (comp) {
+                    if constexpr (sizeof(S) == 4) {
+#pragma unroll
+                        for (int c = 0; c < 12; ++c) cz.add(cdot(hs[c], rs[c]));
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 12; ++c) rho = cdot_acc(rho, hs[c], rs[c]);
+                }
+            }
+            double2 v[2] = {comp ? cz.value() : to_d(rho), make_double2(nrm, 0.0)};
+            block_sum_fp64<2>(v, smd);
+            if (threadIdx.x == 0) {
+                double2* pp = part(P, CNT_RU) + 2 * (size_t)q;
+                pp[0] = v[0];
+                pp[1] = v[1];
             }
         }
-        double2 v[2] = {comp ? cz.value() : to_d(rho), make_double2(nrm, 0.0)};
-        block_sum<2>(v, smd);
-        if (threadIdx.x == 0) {
-            double2* pp = part(P, CNT_RU) + 2 * (size_t)blockIdx.x;
-            pp[0] = v[0];
-            pp[1] = v[1];
-        }
-        __syncthreads();
     }
-    // the last block adds the partials in block order and ends the iteration
+    // the last block adds the partials in a fixed order and ends the iteration
     if (!last_block(ptrs[0].counters + CNT_RU, gridDim.x)) return;
     for (int i = 0; i < nact; ++i) {
         SlotState& st = states[list[i]];
         const SlotPtrs& P = ptrs[list[i]];
         const double2* pp = part(P, CNT_RU);
         double2 v[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
-        for (unsigned b = threadIdx.x; b < gridDim.x; b += RU_THREADS) {
+        for (int b = threadIdx.x; b < nruns; b += RU_THREADS) {
             v[0] = v[0] + __ldcg(pp + 2 * (size_t)b);
             v[1] = v[1] + __ldcg(pp + 2 * (size_t)b + 1);
         }
-        block_sum<2>(v, smd);
+        block_sum_fp64<2>(v, smd);
         if (threadIdx.x == 0) {
             st.true_rnorm = sqrt_fp64(v[1].x);
             st.matvecs += 1;
