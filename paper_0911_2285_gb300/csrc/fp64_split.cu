@@ -96,10 +96,16 @@ __global__ void __launch_bounds__(SPLIT_THREADS) apply_split_kernel(Geom g, cons
 __global__ void __launch_bounds__(SPLIT_THREADS) matvec_split_kernel(Geom g, const double2* links, double kappa,
                                                                      SlotState* states, const SlotPtrs* ptrs, int njobs) {
     __shared__ double2 sm[8][12][SPLIT_SITES];
+    __shared__ int go;
     const int job = blockIdx.x % njobs, sblock = blockIdx.x / njobs, which = job & 1;
     SlotState& st = states[job >> 1];
     const SlotPtrs& P = ptrs[job >> 1];
-    if (st.status != ST_RUNNING || st.stab) return;
+    // One thread reads the status for the block: the last even block may store a breakdown
+    // while an odd block, which it does not wait for, still starts; threads that read it
+    // themselves could part before the barrier in split_terms.
+    if (threadIdx.x == 0) go = st.status == ST_RUNNING && !st.stab;
+    __syncthreads();
+    if (!go) return;
     const int par = st.iter & 1, s0 = sblock * SPLIT_SITES;
     const double2* src = reinterpret_cast<const double2*>(which ? P.phat : P.p);
     const double2* ph = reinterpret_cast<const double2*>(P.phat);
