@@ -13,7 +13,8 @@ namespace lqcd {
 // Bound of every device-side wait, in SM clock cycles (default about 2 s at
 // 2 GHz). Each translation unit that includes this header holds its own copy
 // on each device; set_wait_cycles_here() sets the copy of the including unit on
-// the current device (the C ABI's lqcd_set_wait_limit sets all of them).
+// the current device (the C ABI's lqcd_set_wait_limit sets all of them). A kernel that
+// gives up still waits for its copies in flight with the default limit (mbar_drain).
 constexpr long long DEFAULT_WAIT_CYCLES = 4000000000ll;
 static __device__ long long g_wait_cycles = DEFAULT_WAIT_CYCLES;
 __device__ __forceinline__ long long wait_cycles() { return *(volatile long long*)&g_wait_cycles; }
@@ -51,6 +52,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
     while (!mbar_test(bar, parity))
         if (clock64() - t0 > lim) return false;
     return true;
+}
+// Wait for the copies or MMAs in flight before the block exits: one that lands later would
+// land in the shared or tensor memory of another block. Never less than the default limit,
+// whatever shorter limit made the kernel give up.
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, unsigned parity) {
+    const long long t0 = clock64(), lim = wait_cycles();
+    while (!mbar_test(bar, parity))
+        if (clock64() - t0 > (lim > DEFAULT_WAIT_CYCLES ? lim : DEFAULT_WAIT_CYCLES)) return;
 }
 // Wait for a device word to become nonzero, at most wait_cycles().
 __device__ __forceinline__ bool flag_wait(const volatile int* flag) {

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(32 * DT_WARPS, 1)
         if (tid == 0) {
             atomicExch(err, 1);
             for (int s = 0; s < S; ++s)   // copies in flight land before the block exits
-                if (issued[s]) mbar_wait(&full[s], (issued[s] - 1) & 1u);
+                if (issued[s]) mbar_drain(&full[s], (issued[s] - 1) & 1u);
         }
         return;
     }

@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         if (tid == 0) {
             atomicExch(err, 1);
             for (int i = 0; i < 3; ++i)
-                if (issued[i] > 0) mbar_wait(&bars[i], (unsigned)((issued[i] - 1) & 1));
+                if (issued[i] > 0) mbar_drain(&bars[i], (unsigned)((issued[i] - 1) & 1));
         }
         __syncthreads();
         return;

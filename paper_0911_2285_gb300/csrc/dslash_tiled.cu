@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(TILE_MAX_THREADS, 1)
         if (threadIdx.x == 0) {
             atomicExch(err, 1);
             for (int i = 0; i < 5; ++i)
-                if (issued[i] > 0) mbar_wait(&bars[i], (unsigned)((issued[i] - 1) & 1));
+                if (issued[i] > 0) mbar_drain(&bars[i], (unsigned)((issued[i] - 1) & 1));
         }
         __syncthreads();
         return;

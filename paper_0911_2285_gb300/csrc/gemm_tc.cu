@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             }
             // every issued copy must land before the CTA may exit
             for (int q = j - TC_STAGES > 0 ? j - TC_STAGES : 0; q < j; ++q)
-                mbar_wait(&B->full[q % TC_STAGES], (unsigned)(q / TC_STAGES) & 1u);
+                mbar_drain(&B->full[q % TC_STAGES], (unsigned)(q / TC_STAGES) & 1u);
         }
     } else if (warp == 1) {
         if (lane == 0) {   // ---------------- MMA issuer
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 if (i % TC_FLUSH == TC_FLUSH - 1 || i == n - 1) mma_commit(&B->accfull[b]);
             }
             if (i > 0)   // the last MMAs must finish before tensor memory is released
-                mbar_wait(&B->empty[(i - 1) % TC_STAGES], (unsigned)((i - 1) / TC_STAGES) & 1u);
+                mbar_drain(&B->empty[(i - 1) % TC_STAGES], (unsigned)((i - 1) / TC_STAGES) & 1u);
         }
     } else {   // ---------------------------- split warps (+ accumulator readers)
         const int xt = tid - 64;
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
                                   RT_E * 8, &S->raw_full[s]);
             }
             for (int h = g - RT_STAGES > 0 ? g - RT_STAGES : 0; h < g; ++h)
-                mbar_wait(&S->raw_full[h % RT_STAGES], (unsigned)(h / RT_STAGES) & 1u);
+                mbar_drain(&S->raw_full[h % RT_STAGES], (unsigned)(h / RT_STAGES) & 1u);
         }
     } else if (warp == 1) {
         if (lane == 0) {   // ------------------------------ MMAs
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
                 mma_commit(&S->a_empty[b]);
                 if (q == Q - 1) mma_commit(&S->acc_full[acc]);
             }
-            if (g > 0) mbar_wait(&S->a_empty[(g - 1) & 1], (unsigned)((g - 1) / 2) & 1u);
+            if (g > 0) mbar_drain(&S->a_empty[(g - 1) & 1], (unsigned)((g - 1) / 2) & 1u);
         }
     } else if (warp < 2 + RT_XW) {   // ------------------- transpose + 3xTF32 split
         const int xt = tid - 64;
