@@ -714,6 +714,24 @@ lqcd_status apply_fields(lqcd_ctx* c, int prec, int dagger, int nf, const void* 
     return LQCD_OK;
 }
 
+// A bounded device wait gave up: the work since the last check is discarded by the caller,
+// the reduction counters may be stale.
+lqcd_status wait_gave_up(lqcd_ctx* c) {
+    CK(cudaMemsetAsync(c->counters, 0, (size_t)c->kmax * CNT_COUNT * sizeof(unsigned), c->stream));
+    CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    g_last_error = "a bounded device wait gave up (its limit: lqcd_set_wait_limit)";
+    return LQCD_ERR_TIMEOUT;
+}
+
+// Waits for the stream; LQCD_ERR_TIMEOUT if a kernel since the last check gave up.
+lqcd_status check_waits(lqcd_ctx* c) {
+    int herr = 0;
+    CK(cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    return herr ? wait_gave_up(c) : LQCD_OK;
+}
+
 bool residual_in_fp32(const lqcd_ctx* c, bool precise) { return c->kprec && !precise && !c->eo; }
 
 // r = b - A x_hi for slots s0 .. s0+nf-1: FP32 hop arithmetic in mixed precision (the
@@ -1010,6 +1028,9 @@ lqcd_status grow_space(lqcd_ctx* c, int nn, void* work) {
         count_launches(2);
         CK(cudaGetLastError());
     }
+    // inner products that a kernel gave up on must not enter the space: n_def stays, and
+    // everything written so far lies beyond it
+    if (kp && (s = check_waits(c)) != LQCD_OK) return s;
     c->n_def = n + kk;
     return refactor(c);
 }
@@ -1029,6 +1050,8 @@ extern "C" lqcd_status lqcd_deflate(lqcd_ctx* c, int k, const double* b, double*
                                      on_device);
         if (s != LQCD_OK) return s;
         s = deflate_slots(c, kb);
+        if (s != LQCD_OK) return s;
+        s = check_waits(c);   // U_l^H r of a kernel that gave up must not reach the caller
         if (s != LQCD_OK) return s;
         s = store_solutions(c, 0, kb, x0 + (size_t)j0 * 2 * c->Nfull, on_device);
         if (s != LQCD_OK) return s;
@@ -1161,14 +1184,7 @@ lqcd_status solve_slots(lqcd_ctx* c, int k, int windowed, double tol, bool rec_s
         CK(cudaMemcpyAsync(c->h_state, c->d_state, sizeof(SlotState) * k, cudaMemcpyDeviceToHost, c->stream));
         CK(cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
-        if (herr) {
-            // a bounded device wait gave up: the reduction counters may be stale
-            CK(cudaMemsetAsync(c->counters, 0, (size_t)c->kmax * CNT_COUNT * sizeof(unsigned), c->stream));
-            CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
-            CK(cudaStreamSynchronize(c->stream));
-            g_last_error = "operator kernel: bounded wait on a TMA copy timed out";
-            return LQCD_ERR_TIMEOUT;
-        }
+        if (herr) return wait_gave_up(c);
         bool any = false;
         for (int j = 0; j < k; ++j) any = any || c->h_state[j].status == ST_RUNNING;
         if (!any) break;
@@ -1984,13 +2000,16 @@ lqcd_status retire(lqcd_ctx* c, int s) {
         return begin_slot(c, s, job.md, c->p.tol, false, false, c->kprec != 0, c->p.maxiter, c->p.bicgstab != 0);
     }
     if (job.windowed) {
-        lqcd_status r = grow_slot(c, s);
-        if (r != LQCD_OK) return r;
+        const lqcd_status grown = grow_slot(c, s);
+        if (grown != LQCD_OK && grown != LQCD_ERR_TIMEOUT) return grown;
         c->last_window_valid = 1;
         c->eig_inflight -= 1;
         job.windowed = false;
-        r = detach_window(c, s);   // its memory is free for the next eigBiCG request
+        lqcd_status r = detach_window(c, s);   // its memory is free for the next eigBiCG request
         if (r != LQCD_OK) return r;
+        // the growth works in the window's memory, so its Ritz vectors are lost; the
+        // request goes on with the next call
+        if (grown != LQCD_OK) return grown;
     }
     if (job.correction_pending) {
         // mixed eigBiCG: the window leg stopped at the recursive tolerance; the
@@ -2072,13 +2091,7 @@ extern "C" lqcd_status lqcd_progress(lqcd_ctx* c, int wait, int* pending) {
     CK(cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     c->chunk_inflight = false;
-    if (herr) {
-        CK(cudaMemsetAsync(c->counters, 0, (size_t)c->kmax * CNT_COUNT * sizeof(unsigned), c->stream));
-        CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
-        CK(cudaStreamSynchronize(c->stream));
-        g_last_error = "operator kernel: bounded wait on a TMA copy timed out";
-        return LQCD_ERR_TIMEOUT;
-    }
+    if (herr) return wait_gave_up(c);
     // 2. retire slots that stopped iterating
     for (int s = 0; s < c->kmax; ++s)
         if (c->jobs[s].busy && c->h_state[s].status != ST_RUNNING) {
