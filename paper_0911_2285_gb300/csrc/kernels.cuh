@@ -148,8 +148,7 @@ cudaError_t launch_true_resid(int variant, const Geom& g, const void* links64, d
                               const SlotPtrs* ptrs, int nslots, cudaStream_t s);
 // Reliable update of the slots that asked for it (reliable.cu): x_hi += x_lo, the
 // true residual b - A x_hi, and unless it meets the tolerance the recursive residual
-// is replaced by it; ends the iteration of these slots (scalars). One cooperative
-// launch. links_df != null: A x_hi in double-float arithmetic (needs the slots'
+// is replaced by it; ends the iteration of these slots (scalars). links_df != null: A x_hi in double-float arithmetic (needs the slots'
 // x_df), else FP64; eo: the even-odd Schur residual (FP64). err: device word set to
 // 1 if a bounded wait gave up. max_blocks: ru_max_blocks().
 cudaError_t launch_bicg_ru(const Geom& g, const void* links64, double kappa, int prec, SlotState* st_,

@@ -6,13 +6,19 @@
 //   gamma5 variant's shadow follows) and rho is recomputed;
 //   the scalars that end the iteration.
 //
-// One cooperative launch per iteration, a block set that the GPU holds at once,
-// with a grid barrier between the fold and the residual (whose neighbours it
-// reads). The former three kernels plus the scalar kernel cost four launches in
-// every iteration though a solve updates about six times; with grids of one
-// thread per site their empty launches alone took 50 us of a 2.7 ms iteration at
-// 24^3 x 64 (now one launch of at most 456 blocks), and 8 of 39 us on small
-// lattices. All blocks share the work of however many slots need it.
+// One kernel, whose blocks share the work of however many slots need it and return at once
+// when none does, which is all but about six times in a solve (one thread per site in four
+// kernels took 50 us of a 2.7 ms iteration at 24^3 x 64 in empty launches and 8 of 39 us on
+// small lattices). It has two (even-odd: three) phases, each reading neighbours that the
+// one before wrote:
+//  * up to RU_COOP units of work: one cooperative launch with a grid barrier between the
+//    phases, 1.5 us per iteration less than a launch per phase (FP64 solve on 4^4 2.44 ms,
+//    2.57 the other way; 10x6x14x9 mixed 5.53 and 5.72);
+//  * above: a launch per phase. A cooperative launch starts only when all its blocks fit on
+//    the GPU at once, so that a large one waited in every iteration for room beside the
+//    kernels of another context: 16^3 x 32 solves beside 24^3 x 64 ones 346 ms, now 253
+//    (four kernels: 284), alone 15.7 and 15.8. With 128 blocks (8^4, 4 slots) both ways
+//    take 104 and 101 ms beside, with 256 blocks 137 and 129 (four kernels: 143).
 //
 // Double-float residual: about 10^4 FP32 instructions per site. Written out for
 // eight hops that is 175 KB of code, more than the instruction caches hold: ncu
@@ -35,6 +41,7 @@ namespace lqcd {
 namespace {
 
 constexpr int RU_THREADS = 128;
+constexpr int RU_COOP = 2 * 152;   // 128-site units (slots x units) of a cooperative launch: two blocks per SM
 constexpr int RU_RUNS = 4096;   // partial sums per slot at most (24^3 x 64: 3456 of two units)
 static_assert(2 * RU_RUNS <= PARTIAL_STRIDE, "partials of a slot");
 
@@ -171,11 +178,12 @@ __device__ __forceinline__ void hop_site_df(const Geom& g, const float4* __restr
 }
 
 enum RuMode { RU_F64 = 0, RU_DF = 1, RU_EO = 2 };
+enum RuPhase { RU_ALL = -1, RU_FOLD = 0, RU_STAGE = 1, RU_RESID = 2 };   // RU_ALL: cooperative launch
 
 template <typename S, int MODE>
 __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
     ru_kernel(Geom g, const double2* links64, const float4* links_df, double kappa, SlotState* states,
-              const SlotPtrs* ptrs, int nslots, size_t N, int* err) {
+              const SlotPtrs* ptrs, int nslots, size_t N, int phase, int* err) {
     __shared__ int list[MAX_SLOTS];
     __shared__ int s_n;
     if (threadIdx.x == 0) {
@@ -192,7 +200,7 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
     unsigned* gen = ptrs[0].counters + CNT_GEN;
     // x_hi += x_lo, x_lo = 0
     const size_t units = N / 2;
-    for (int i = 0; i < nact; ++i) {
+    for (int i = 0; i < nact && phase <= RU_FOLD; ++i) {
         const SlotState& st = states[list[i]];
         const SlotPtrs& P = ptrs[list[i]];
         const cplx<S> al = cvt<S>(st.alpha);
@@ -215,9 +223,10 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
             }
         }
     }
-    bool ok = grid_barrier(bar, gen, gridDim.x);
+    if (phase == RU_FOLD) return;
+    bool ok = phase != RU_ALL || grid_barrier(bar, gen, gridDim.x);
     const int Vs = MODE == RU_EO ? g.V / 2 : g.V;   // sites of the solver's space
-    if (MODE == RU_EO && ok) {   // stage 1: D_eo x_hi on the even sites
+    if (MODE == RU_EO && ok && phase != RU_RESID) {   // stage 1: D_eo x_hi on the even sites
         const LinksD U{links64, g.V};
         for (int i = 0; i < nact; ++i) {
             const SlotPtrs& P = ptrs[list[i]];
@@ -228,6 +237,7 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
                 Field<double>::store(P.eo64, Vs, h, acc);
             }
         }
+        if (phase == RU_STAGE) return;
         ok = grid_barrier(bar, gen, gridDim.x);
     }
     if (!ok) {   // uniform over the block: report and leave, the host discards the solve
@@ -358,7 +368,7 @@ __global__ void links_df_kernel(const double2* l64, float4* ldf, size_t n) {
     }
 }
 
-using RuKernel = void (*)(Geom, const double2*, const float4*, double, SlotState*, const SlotPtrs*, int, size_t, int*);
+using RuKernel = void (*)(Geom, const double2*, const float4*, double, SlotState*, const SlotPtrs*, int, size_t, int, int*);
 RuKernel ru_select(int prec, int df, int eo) {
     if (prec == 0) return eo ? ru_kernel<double, RU_EO> : ru_kernel<double, RU_F64>;
     if (eo) return ru_kernel<float, RU_EO>;
@@ -391,6 +401,17 @@ cudaError_t launch_bicg_ru(const Geom& g, const void* links64, double kappa, int
                            int max_blocks, int* err) {
     const int Vs = eo ? g.V / 2 : g.V;
     const long long units = (long long)((Vs + RU_THREADS - 1) / RU_THREADS) * nslots;
+    const RuKernel kernel = ru_select(prec, links_df && !eo, eo);
+    const double2* l64 = reinterpret_cast<const double2*>(links64);
+    if (units > RU_COOP) {
+        const unsigned grid = (unsigned)(units < max_blocks ? units : max_blocks);
+        for (int phase : {RU_FOLD, RU_STAGE, RU_RESID}) {
+            if (phase == RU_STAGE && !eo) continue;
+            kernel<<<grid, RU_THREADS, 0, s>>>(g, l64, links_df, kappa, states, ptrs, nslots, N, phase, err);
+            count_launches(1);
+        }
+        return cudaGetLastError();
+    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(units < max_blocks ? units : max_blocks));
     cfg.blockDim = dim3(RU_THREADS);
@@ -400,9 +421,7 @@ cudaError_t launch_bicg_ru(const Geom& g, const void* links64, double kappa, int
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, ru_select(prec, links_df && !eo, eo), g,
-                                       reinterpret_cast<const double2*>(links64), links_df, kappa, states, ptrs, nslots, N,
-                                       err);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, g, l64, links_df, kappa, states, ptrs, nslots, N, (int)RU_ALL, err);
     count_launches(1);
     return e;
 }
