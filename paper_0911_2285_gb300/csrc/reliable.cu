@@ -190,7 +190,10 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
         int n = 0;
         for (int j = 0; j < nslots; ++j)
             if (states[j].status == ST_RUNNING && states[j].live && states[j].need_ru) list[n++] = j;
-        s_n = n;
+        // After a wait that gave up, the counters may be stale until the host has seen err:
+        // no further update. (Set by a block of this launch while others start, it only
+        // makes them give up too.)
+        s_n = *(volatile int*)err ? 0 : n;
     }
     __syncthreads();
     const int nact = s_n;

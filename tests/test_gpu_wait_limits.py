@@ -99,3 +99,23 @@ def test_growth_reports_the_timeout_and_keeps_the_space(short_waits):
         assert s.eigspace_size() == 40
         s.solve(b, mode="eigbicg")
         assert s.eigspace_size() > 40
+
+
+@pytest.mark.parametrize("variant", [{}, {"evenodd": True}, {"precision": "fp64"}])
+def test_reliable_update_barrier(short_waits, variant):
+    """The grid barriers of a small lattice's reliable update: the solve reports the
+    timeout, and the next one gives the bits of the one before."""
+    from paper_0911_2285_gb300 import Solver, lqcd
+    from seeded_inputs import z2_source
+    from tests.gpu_util import small_problem
+    dims = (8, 8, 8, 8)
+    links, _ = small_problem(dims)
+    b = np.stack([z2_source(dims, 60 + j) for j in range(3)])
+    with Solver(links, dims, 0.12, nev=4, m=12, tol=1e-10, k_max=3, autotune=False, **variant) as s:
+        good = s.solve(b, mode="plain")[0]
+        for mode in ("plain", "eigbicg" if variant == {"precision": "fp64"} else "plain"):
+            short_waits(True)
+            st = s.solve(b, mode=mode, raise_on_fail=False)[2]
+            assert st == lqcd.ERR_TIMEOUT
+            short_waits(False)
+            assert np.array_equal(s.solve(b, mode="plain")[0], good)
