@@ -16,7 +16,7 @@ namespace {
 
 constexpr int DS_THREADS = 128;   // operator kernels
 constexpr int BL_THREADS = 256;   // vector kernels
-constexpr int G5_STALL = 200;     // iterations without a reliable update after which the gamma5 variant starts over
+constexpr int G5_STALL = 500;     // least number of iterations that make a stall of the gamma5 variant
 
 inline int div_up(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 
@@ -393,6 +393,9 @@ __global__ void __launch_bounds__(BL_THREADS) start_kernel(SlotState* states, co
         st.rhat_norm = st.rnorm;
         st.rmax = st.rnorm;
         st.r_ru = st.rnorm;
+        st.r_min = st.r_best = st.rnorm;
+        st.ru_iter = 0; st.min_iter = 0; st.fresh_dir = FRESH_NONE;
+        st.x_best = 1; st.best_used = 0; st.stall_lim = G5_STALL;
         st.true_rnorm = st.rnorm;
         st.iter = 0; st.vs = 0; st.need_ru = 0; st.ru_count = 0; st.restarts = 0; st.restart_r = 0;
         st.matvecs = 1; st.live = 1;
@@ -682,10 +685,25 @@ __global__ void __launch_bounds__(BL_THREADS) update_kernel(SlotState* states, c
             if (st.delta > 0.0 && (st.rnorm_new < st.delta * st.r_ru || st.rnorm_new < 1e-3 * st.rmax)) st.need_ru = 1;
             // gamma5 variant with FP32 vectors: its shadow recursion can lose its
             // biorthogonality for good, which rounding decides (about one deflated solve
-            // in twelve on a near-free 4^4 field, whatever the kernels); a residual that
-            // has not earned a reliable update in G5_STALL iterations starts over from
-            // the true residual with a fresh direction.
-            if (st.g5 && st.delta > 0.0 && st.iter - st.ru_iter >= G5_STALL) st.need_ru = st.fresh_dir = 1;
+            // in twelve on a near-free 4^4 field, whatever the kernels). A residual whose
+            // minimum has not halved in stall_lim iterations is taken for lost: the solve
+            // starts over with a fresh direction, from the current x if its residual is
+            // below that of every update so far, else from the best x of them (a second
+            // time from the same x would repeat the first: then from the current x if its
+            // residual is not far above). stall_lim is at least four times the iterations of
+            // any update so far, so that slow convergence is not a stall, and doubles with
+            // each restart. Solves that fail: near-free 4^4, 35 of 336 without restarts, 7
+            // with them; 6^4 at kappa 0.130 and 0.134, 8 of 16 and none; 4^3 x 6 past critical
+            // (0.16) end at 3e-5 to 0.2 ||b||, without restarts at 0.01 to 2e5. (Restarts
+            // after 200 iterations without an update, from whatever x there was, ended there
+            // at up to 1e15 and did not wait for slow solves.)
+            if (st.g5 && st.delta > 0.0) {
+                if (st.rnorm_new < 0.5 * st.r_min) { st.r_min = st.rnorm_new; st.min_iter = st.iter; }
+                if (!st.need_ru && st.iter - st.min_iter >= st.stall_lim) {
+                    st.need_ru = 1;
+                    st.fresh_dir = st.rnorm_new < (st.best_used ? 1e3 : 1.0) * st.r_best ? FRESH_HERE : FRESH_BEST;
+                }
+            }
             if (!st.need_ru) bicg_scalars(st, P);   // else the reliable update ends the iteration
         }
     }
@@ -904,13 +922,15 @@ __global__ void fold_kernel(SlotState* states, const SlotPtrs* ptrs, size_t N) {
     const SlotPtrs& P = ptrs[blockIdx.y];
     if (st.status == ST_IDLE) return;
     const bool zero_src = st.bnorm == 0.0;
-    const bool owed = st.x_owed != 0;   // the last residual update's alpha p (no direction update ran)
+    // a gamma5 solve that failed returns its best x (see ru_kernel)
+    const bool back = sizeof(S) == 4 && st.g5 && st.delta > 0.0 && st.status != ST_CONVERGED && !(st.rnorm_new <= st.r_best);
+    const bool owed = st.x_owed != 0 && !back;   // the last residual update's alpha p (no direction update ran)
     const cplx<S> al = cvt<S>(st.alpha);
     const size_t units = N / 2;
     Unit<S> zero{mk<S>(0, 0), mk<S>(0, 0)};
     for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < units; u += (size_t)gridDim.x * blockDim.x) {
-        Unit<double> xh = Unit<double>::load(P.x_hi, u);
-        Unit<S> xl = Unit<S>::load(P.x_lo, u);
+        Unit<double> xh = Unit<double>::load(back && !st.x_best ? P.r_true : P.x_hi, u);
+        Unit<S> xl = back ? zero : Unit<S>::load(P.x_lo, u);
         if (owed) {
             const Unit<S> p = Unit<S>::load(P.p, u);
             xl.a = cfma(xl.a, al, p.a); xl.b = cfma(xl.b, al, p.b);

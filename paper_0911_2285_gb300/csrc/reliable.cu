@@ -207,11 +207,16 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
         const SlotState& st = states[list[i]];
         const SlotPtrs& P = ptrs[list[i]];
         const cplx<S> al = cvt<S>(st.alpha);
-        const bool owed = st.x_owed != 0;
+        // gamma5 variant, FP32 vectors: the best x so far is kept in r_true (free between the
+        // start and the end of a solve), for a solve that has to go back to it
+        const bool guard = sizeof(S) == 4 && st.g5 != 0, back = guard && st.fresh_dir == FRESH_BEST;
+        const bool keep = guard && st.x_best != 0 && !back, fetch = back && !st.x_best;
+        const bool owed = st.x_owed != 0 && !back;
         const Unit<S> zero{mk<S>(0, 0), mk<S>(0, 0)};
         for (size_t u = gt; u < units; u += gn) {
-            Unit<double> xh = Unit<double>::load(P.x_hi, u);
-            Unit<S> xl = Unit<S>::load(P.x_lo, u);
+            Unit<double> xh = Unit<double>::load(fetch ? P.r_true : P.x_hi, u);
+            Unit<S> xl = back ? zero : Unit<S>::load(P.x_lo, u);
+            if (keep) xh.store(P.r_true, u);
             if (owed) {   // alpha p of this iteration's residual update
                 const Unit<S> p = Unit<S>::load(P.p, u);
                 xl.a = cfma(xl.a, al, p.a); xl.b = cfma(xl.b, al, p.b);
@@ -353,6 +358,17 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
             }
             st.need_ru = 0;
             st.ru_count += 1;
+            if (sizeof(S) == 4 && st.g5) {
+                if (st.fresh_dir == FRESH_NONE) st.stall_lim = max(st.stall_lim, 4 * (st.iter + 1 - st.ru_iter));
+                else st.stall_lim = min(2 * st.stall_lim, 1 << 28);
+                st.x_best = st.fresh_dir == FRESH_BEST || st.true_rnorm < st.r_best;
+                if (st.x_best) {
+                    st.r_best = st.true_rnorm;
+                    st.best_used = st.fresh_dir == FRESH_BEST;
+                }
+                st.r_min = st.true_rnorm;
+                st.min_iter = st.iter + 1;
+            }
             st.ru_iter = st.iter + 1;
             st.x_owed = 0;   // the fold added alpha p
             if (st.stab) stab_scalars(st);

@@ -9,6 +9,7 @@
 
 namespace lqcd {
 
+enum FreshDir : int { FRESH_NONE = 0, FRESH_HERE = 1, FRESH_BEST = 2 };   // ... from the current x, from the best x
 enum SlotStatus : int { ST_RUNNING = 0, ST_CONVERGED = 1, ST_BREAKDOWN = 2, ST_NOCONV = 3, ST_IDLE = 4 };
 
 struct SlotState {
@@ -34,7 +35,13 @@ struct SlotState {
     int need_ru;          // 1: recompute the FP64 residual in this iteration
     int ru_count;
     int ru_iter;          // iteration of the last reliable update (or the start)
-    int fresh_dir;        // 1: the next direction starts over (beta = 0)
+    int fresh_dir;        // FreshDir: the next direction starts over (beta = 0; gamma5 variant, FP32 vectors)
+    int stall_lim;        // iterations without a halved minimum of ||r|| that make a stall (the same)
+    int min_iter;         // iteration of that minimum
+    int x_best;           // 1: x_hi is the best x so far, 0: the best one is in r_true
+    int best_used;        // 1: the solve has started over from the best x
+    double r_min;         // last minimum of ||r|| that counted, since the last update
+    double r_best;        // true residual of the best x
     int restarts;
     int restart_r;        // vectors kept by the restart in this iteration (0 = none)
     int matvecs;
