@@ -33,18 +33,25 @@ __device__ __forceinline__ double widen(float a) {
     const bool zero = m == 0u;
     return __hiloint2double((int)((b & 0x80000000u) | (zero ? 0u : (m >> 3) + up)), zero ? 0 : (int)(b << 29));
 }
-// FP64 to FP32, to nearest (ties away from zero; subnormal results rounded twice);
-// from FP32's largest number up infinity, NaN kept.
+// The bits below FP32's normal range, |a| < 2^-126 (m: high word of |a|): a whole number of
+// 2^-149. A call: inlined, its 64-bit shifts are issued for every conversion (deflation of
+// 8 guesses on 16^3 x 32 0.98 -> 1.03 ms).
+static __device__ __noinline__ unsigned narrow_small(unsigned m, unsigned lo) {
+    const unsigned sh = 926u - (m >> 20);   // places of the 53-bit mantissa below 2^-149: 30 and more
+    const unsigned long long v = ((unsigned long long)((m & 0xfffffu) | 0x100000u) << 32) | lo;
+    return sh > 54u ? 0u : (unsigned)((v + ((1ull << (sh - 1u)) - 1ull) + ((v >> sh) & 1ull)) >> sh);
+}
+// FP64 to FP32, to nearest (ties to even) over FP32's whole range, as the conversion
+// instruction rounds; from FP32's largest number up infinity, NaN kept.
 __device__ __forceinline__ float narrow(double a) {
-    const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a), sign = hi & 0x80000000u;
-    const bool sub = (hi & 0x7fffffffu) < (897u << 20);         // below 2^-126: by way of 2^64 a
-    const unsigned l2 = lo + 0x10000000u;                       // half a unit of FP32's last place
-    const unsigned h2 = (hi & 0x7fffffffu) + (l2 < lo ? 1u : 0u) + (sub ? (64u << 20) : 0u);
+    const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a), m = hi & 0x7fffffffu;
+    const unsigned l2 = lo + 0x0fffffffu + ((lo >> 29) & 1u);   // half a unit of FP32's last place, to even
+    const unsigned h2 = m + (l2 < lo ? 1u : 0u);
     unsigned r = ((h2 - (896u << 20)) << 3) | (l2 >> 29);
-    if (h2 < (897u << 20)) r = 0u;
     if (h2 >= (1151u << 20)) r = 0x7f800000u;
-    if ((hi & 0x7fffffffu) + (lo != 0u ? 1u : 0u) > 0x7ff00000u) r = 0x7fffffffu;   // NaN
-    return __uint_as_float(sign | r) * (sub ? 5.42101086242752217e-20f : 1.f);
+    if (m < (897u << 20)) r = (m | lo) == 0u ? 0u : narrow_small(m, lo);
+    if (m + (lo != 0u ? 1u : 0u) > 0x7ff00000u) r = 0x7fffffffu;   // NaN
+    return __uint_as_float((hi & 0x80000000u) | r);
 }
 __device__ __forceinline__ float2 narrow(double2 a) { return make_float2(narrow(a.x), narrow(a.y)); }
 __device__ __forceinline__ double2 widen(float2 a) { return make_double2(widen(a.x), widen(a.y)); }
