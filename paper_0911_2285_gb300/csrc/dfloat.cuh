@@ -37,10 +37,12 @@ __device__ __forceinline__ dfc operator+(dfc a, dfc b) { return {a.x + b.x, a.y 
 __device__ __forceinline__ dfc operator-(dfc a, dfc b) { return {a.x - b.x, a.y - b.y}; }
 __device__ __forceinline__ dfc operator-(dfc a) { return {-a.x, -a.y}; }
 
-// One FP64 instruction each (the conversions run on the integer pipe).
+// One FP64 instruction each (the conversions run on the integer pipe). In a split the side
+// that a tie goes to costs nothing: l holds the rest of h exactly, and is off by half a unit
+// of its own either way.
 __device__ __forceinline__ dfl df_split(double v) {
-    const float h = narrow(v);
-    return {h, narrow(v - widen(h))};
+    const float h = narrow_to<false>(v);
+    return {h, narrow_to<false>(v - widen(h))};
 }
 __device__ __forceinline__ double df_value(dfl a) { return widen(a.h) + widen(a.l); }
 

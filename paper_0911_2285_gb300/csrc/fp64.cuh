@@ -41,11 +41,11 @@ static __device__ __noinline__ unsigned narrow_small(unsigned m, unsigned lo) {
     const unsigned long long v = ((unsigned long long)((m & 0xfffffu) | 0x100000u) << 32) | lo;
     return sh > 54u ? 0u : (unsigned)((v + ((1ull << (sh - 1u)) - 1ull) + ((v >> sh) & 1ull)) >> sh);
 }
-// FP64 to FP32, to nearest (ties to even) over FP32's whole range, as the conversion
-// instruction rounds; from FP32's largest number up infinity, NaN kept.
-__device__ __forceinline__ float narrow(double a) {
+// FP64 to FP32, to nearest over FP32's whole range; EVEN: ties to even, as the conversion
+// instruction rounds, else away from zero. From FP32's largest number up infinity, NaN kept.
+template <bool EVEN> __device__ __forceinline__ float narrow_to(double a) {
     const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a), m = hi & 0x7fffffffu;
-    const unsigned l2 = lo + 0x0fffffffu + ((lo >> 29) & 1u);   // half a unit of FP32's last place, to even
+    const unsigned l2 = lo + (EVEN ? 0x0fffffffu + ((lo >> 29) & 1u) : 0x10000000u);   // half a unit of FP32's last place
     const unsigned h2 = m + (l2 < lo ? 1u : 0u);
     unsigned r = ((h2 - (896u << 20)) << 3) | (l2 >> 29);
     if (h2 >= (1151u << 20)) r = 0x7f800000u;
@@ -53,6 +53,7 @@ __device__ __forceinline__ float narrow(double a) {
     if (m + (lo != 0u ? 1u : 0u) > 0x7ff00000u) r = 0x7fffffffu;   // NaN
     return __uint_as_float((hi & 0x80000000u) | r);
 }
+__device__ __forceinline__ float narrow(double a) { return narrow_to<true>(a); }
 __device__ __forceinline__ float2 narrow(double2 a) { return make_float2(narrow(a.x), narrow(a.y)); }
 __device__ __forceinline__ double2 widen(float2 a) { return make_double2(widen(a.x), widen(a.y)); }
 // FP64 to storage precision S and back.
