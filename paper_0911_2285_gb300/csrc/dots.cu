@@ -207,9 +207,10 @@ __global__ void __launch_bounds__(32 * DT_WARPS, 1)
     if (i < a && j < b) part[(((size_t)blockIdx.x * pl.EG + eg) * a + i) * b + j] = *sum;
 }
 
-// C[i][j] (or its conjugate into C[j][i]) = sum over the np partials, one warp each.
+// C[i][j] (or its conjugate into C[j][i]) = sum over the np partials, one warp each; zero
+// after a wait that gave up (some partials are then from an earlier call).
 __global__ void __launch_bounds__(128) dots_reduce_kernel(int a, int b, int np, const double2* part, double2* Cm, int ldc,
-                                                          int conj_store) {
+                                                          int conj_store, const int* err) {
     const int q = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (q >= a * b) return;
     double2 s0 = make_double2(0.0, 0.0), s1 = s0;
@@ -220,6 +221,7 @@ __global__ void __launch_bounds__(128) dots_reduce_kernel(int a, int b, int np, 
     }
     if (p < np) s0 = s0 + part[(size_t)p * a * b + q];
     s0 = warp_sum(s0 + s1);
+    if (*(const volatile int*)err) s0 = make_double2(0.0, 0.0);
     if (lane == 0) {
         const int i = q / b, j = q % b;
         if (conj_store) Cm[(size_t)j * ldc + i] = conj_(s0);
@@ -277,7 +279,7 @@ cudaError_t launch_dots(int a, const void* X, int b, const void* Y, size_t N, do
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         double2* Cj = conj_store ? Cm + (size_t)j0 * ldc : Cm + j0;
-        dots_reduce_kernel<<<(a * bb + 3) / 4, 128, 0, st>>>(a, bb, p.nx * p.EG, scratch, Cj, ldc, conj_store);
+        dots_reduce_kernel<<<(a * bb + 3) / 4, 128, 0, st>>>(a, bb, p.nx * p.EG, scratch, Cj, ldc, conj_store, err);
         count_launches(2);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
 // C[i][j] (or conj into C[j][i]) = sum over the split-K partials, FP64.
 __global__ void dots_tc_reduce_kernel(int a, int b, int nb, int nblk, const double* part, double2* Cm, int ldc,
-                                      int conj_store) {
+                                      int conj_store, const int* err) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= a * b) return;
     const int i = q / b, j = q % b, ty = i / TC_M, r = i % TC_M;
@@ -288,6 +288,7 @@ __global__ void dots_tc_reduce_kernel(int a, int b, int nb, int nblk, const doub
         re += p[j];
         im += p[nb + j];
     }
+    if (err && *(const volatile int*)err) re = im = 0.0;   // a wait gave up: stale partials
     if (conj_store) Cm[(size_t)j * ldc + i] = make_double2(re, -im);
     else Cm[(size_t)i * ldc + j] = make_double2(re, im);
 }
@@ -699,7 +700,7 @@ cudaError_t launch_dots_tc(int a, const void* X, size_t x_stride, int b, const v
         if (e != cudaSuccess) return e;
         double2* Cj = conj_store ? Cm + (size_t)j0 * ldc : Cm + j0;
         dots_tc_reduce_kernel<<<(int)(((size_t)a * bb + 127) / 128), 128, 0, st>>>(a, bb, nb, nblk, scratch, Cj,
-                                                                            ldc, conj_store);
+                                                                            ldc, conj_store, err);
         count_launches(1);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -1051,13 +1051,11 @@ extern "C" lqcd_status lqcd_deflate(lqcd_ctx* c, int k, const double* b, double*
         if (s != LQCD_OK) return s;
         s = deflate_slots(c, kb);
         if (s != LQCD_OK) return s;
-        s = check_waits(c);   // U_l^H r of a kernel that gave up must not reach the caller
-        if (s != LQCD_OK) return s;
         s = store_solutions(c, 0, kb, x0 + (size_t)j0 * 2 * c->Nfull, on_device);
         if (s != LQCD_OK) return s;
     }
-    CK(cudaStreamSynchronize(c->stream));
-    return LQCD_OK;
+    // inner products that a kernel gave up on come as zeros, which leave the guesses as they were
+    return check_waits(c);
 }
 
 // ============================================================ the solve
