@@ -116,10 +116,15 @@ __device__ __forceinline__ double2 cdiv_fp64(double2 a, double2 b) {
     return make_double2(fma(-a.y, t.y, a.x * t.x), fma(a.y, t.x, a.x * t.y));
 }
 
-// |z| >= tol s1 s2 (s1, s2 >= 0), without the square root of |z|; false for NaN.
+// |z| >= tol s1 s2 (s1, s2 >= 0); false for NaN. On squares where both sides' stay in
+// FP64's range (exponents within +-480), else by hypot.
+static __device__ __noinline__ bool abs_at_least_far(double2 z, double t) { return cabs_(z) >= t; }
 __device__ __forceinline__ bool abs_at_least(double2 z, double tol, double s1, double s2) {
     const double t = tol * s1 * s2;
-    return fma(z.y, z.y, z.x * z.x) >= t * t && !(z.x == 0.0 && z.y == 0.0 && t > 0.0);
+    const unsigned fx = (unsigned)__double2hiint(z.x) & 0x7fffffffu, fy = (unsigned)__double2hiint(z.y) & 0x7fffffffu;
+    const unsigned fz = max(fx, fy) >> 20, ft = (unsigned)__double2hiint(t) >> 20;
+    if (fz - 543u < 961u && ft - 543u < 961u) return fma(z.y, z.y, z.x * z.x) >= t * t;
+    return abs_at_least_far(z, t);
 }
 
 }  // namespace lqcd

@@ -1,6 +1,7 @@
 """The FP64 helpers that carry the scalars of every solver (fp64.cuh), called one value per
 thread, against numpy: conversions bit for bit over both types' whole ranges, reciprocal,
-roots and complex quotient to their error bounds.
+roots and complex quotient to their error bounds, the breakdown comparison also where
+squares leave FP64's range.
 
 Bounds: a third-order step from an FP32 seed (relative error 2^-22 or less) leaves 2^-65, so
 the results carry the rounding of the last multiply-add (half a unit) and, for 1/sqrt, of
@@ -151,3 +152,22 @@ def test_complex_quotient(probe):
     mag = np.maximum(np.abs(ref[0]), np.abs(ref[1]))
     err = np.maximum(np.abs(q[:, 0] - ref[0]), np.abs(q[:, 1] - ref[1])) / mag
     assert float(err.max()) <= 8 * 2.0 ** -53
+
+
+def test_breakdown_comparison_over_the_whole_range(probe):
+    """|z| >= 1e-14 s1 s2 with |z| a little above and below the line, and zero."""
+    rng = np.random.default_rng(5)
+    n = 1 << 16
+    p = rng.uniform(-290, 290, n)                        # 1e-14 s1 s2 = 10^p (every factor in range)
+    s1 = 10.0 ** (p / 2)
+    s2 = 10.0 ** (p / 2 + 14)
+    t = 1e-14 * s1 * s2
+    c = rng.uniform(0.1, 0.99, n)
+    s = np.sqrt(1 - c * c)
+    for f, want in ((1 + 1e-9, 1.0), (1 - 1e-9, 0.0), (1e-40, 0.0), (1e10, 1.0)):
+        x, y = f * t * c, f * t * s
+        ok = (np.abs(x) > 1e-300) & (np.abs(y) > 1e-300) & np.isfinite(x) & np.isfinite(y)
+        assert np.all(probe(6, x[ok], y[ok], s1[ok], s2[ok])[:, 0] == want)
+    zero = np.zeros(4)
+    assert np.all(probe(6, zero, zero, np.array([1.0, 1e-80, 1e-100, 1e100]), np.ones(4))[:, 0] == 0.0)
+    assert np.all(probe(6, np.full(2, np.nan), np.zeros(2), np.ones(2), np.ones(2))[:, 0] == 0.0)
