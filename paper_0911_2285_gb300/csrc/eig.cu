@@ -97,6 +97,7 @@ __device__ __forceinline__ bool df_seed_ok(float h) { return h > 1e-28f && h < 1
 struct NumD {
     using C = double2;
     using R = double;
+    static constexpr bool WIDE = true;   // squares may leave FP64's range
     static __device__ __forceinline__ C zero() { return czero(); }
     static __device__ __forceinline__ C one() { return cone(); }
     static __device__ __forceinline__ C from(double2 a) { return a; }
@@ -139,6 +140,7 @@ struct NumD {
 struct NumF {
     using C = dfc;
     using R = dfl;
+    static constexpr bool WIDE = false;
     static __device__ __forceinline__ C zero() { return {{0.f, 0.f}, {0.f, 0.f}}; }
     static __device__ __forceinline__ C one() { return {{1.f, 0.f}, {0.f, 0.f}}; }
     static __device__ __forceinline__ C from(double2 a) { return dc_from(a); }
@@ -296,12 +298,30 @@ __device__ int schur(double2* A64, double2* Q64, int n, int lda, double2* v64, d
             last = __reduce_max_sync(FULL, last);
             const bool work = last > k + 1;
             if (work) {   // v = x + e^{i theta} ||x|| e1, tau = 2/||v||^2
-                // the norm in FP64: squares of small entries leave FP32's range
+                // The norm in FP64: squares of small entries leave FP32's range. Where they
+                // would leave FP64's as well, v is formed from the column times a power of
+                // two (its length does not matter).
+                bool far = false;
+                double up = 1.0;
+                if constexpr (M::WIDE) {
+                    unsigned f = 0;   // largest exponent field of the column
+                    for (int i = k + 1 + lane; i <= last; i += 32) {
+                        const double2 x = M::to(A[i * lda + k]);
+                        f = max(f, max((unsigned)__double2hiint(x.x) & 0x7ff00000u, (unsigned)__double2hiint(x.y) & 0x7ff00000u) >> 20);
+                    }
+                    f = __reduce_max_sync(FULL, f);
+                    far = f - 543u > 960u;
+                    if (far) up = pow2_field(max(2046 - (int)f, 1));
+                }
+                auto entry = [&](int i) {
+                    const double2 x = M::to(A[i * lda + k]);
+                    return far ? up * x : x;
+                };
                 double nrm2 = 0.0;
-                for (int i = k + 1 + lane; i <= last; i += 32) nrm2 += NumD::abs2(M::to(A[i * lda + k]));
+                for (int i = k + 1 + lane; i <= last; i += 32) nrm2 += NumD::abs2(entry(i));
                 nrm2 = warp_sum(nrm2);
                 const double alpha = sqrt_fp64(nrm2);
-                const double2 x0 = M::to(A[(k + 1) * lda + k]);
+                const double2 x0 = entry(k + 1);
                 const double a0 = NumD::abs2(x0);
                 double2 ph = cone();
                 double ax0 = 0.0;
@@ -312,6 +332,7 @@ __device__ int schur(double2* A64, double2* Q64, int n, int lda, double2* v64, d
                 }
                 for (int i = k + 1 + lane; i <= last; i += 32) {
                     C x = A[i * lda + k];
+                    if (far) x = M::from(entry(i));
                     if (i == k + 1) x = M::from(x0 + alpha * ph);
                     v[i - k - 1] = x;
                 }
