@@ -11,16 +11,16 @@ __device__ __forceinline__ double2* part(const SlotPtrs& P, int kind) { return P
 
 // NR numbers per lane summed over the warp: each of the first steps halves the numbers
 // that a lane holds, the lane's bit says which half it keeps; lane l returns the sum
-// number l / (32 / NR). NR = 4: 6 additions where the sums one by one take 20, each of
-// them 64 clocks of the FP64 pipe.
-template <int NR> __device__ __forceinline__ double lane_sums(const double (&r)[NR]) {
+// number l / (32 / NR). NR = 4: 6 additions where the sums one by one take 20, in FP64 each
+// of them 64 clocks of its pipe.
+template <int NR, typename T> __device__ __forceinline__ T lane_sums(const T (&r)[NR]) {
     static_assert(NR == 2 || NR == 4, "numbers per lane");
     const int lane = threadIdx.x & 31;
     const bool u16 = lane & 16, u8 = lane & 8;
-    double t;
+    T t;
     if constexpr (NR == 4) {
-        const double a = (u16 ? r[2] : r[0]) + __shfl_xor_sync(0xffffffffu, u16 ? r[0] : r[2], 16);
-        const double b = (u16 ? r[3] : r[1]) + __shfl_xor_sync(0xffffffffu, u16 ? r[1] : r[3], 16);
+        const T a = (u16 ? r[2] : r[0]) + __shfl_xor_sync(0xffffffffu, u16 ? r[0] : r[2], 16);
+        const T b = (u16 ? r[3] : r[1]) + __shfl_xor_sync(0xffffffffu, u16 ? r[1] : r[3], 16);
         t = (u8 ? b : a) + __shfl_xor_sync(0xffffffffu, u8 ? a : b, 8);
     } else {
         t = (u16 ? r[1] : r[0]) + __shfl_xor_sync(0xffffffffu, u16 ? r[0] : r[1], 16);
@@ -30,14 +30,22 @@ template <int NR> __device__ __forceinline__ double lane_sums(const double (&r)[
     for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     return t;
 }
-// block_sum of FP64 values by that; v valid in thread 0. smem: 2 NV values per warp.
-template <int NV> __device__ __forceinline__ void block_sum_fp64(double2 (&v)[NV], double* smem) {
+__device__ __forceinline__ double wid(float a) { return widen(a); }
+__device__ __forceinline__ double wid(double a) { return a; }
+// Sums of NV complex values over the block, valid in thread 0: over a warp in the precision
+// of v, across the warps in FP64. FP32 across the warps as well would leave the rounding of
+// one number per block, and red_blocks has few blocks: rms error of a squared norm on the
+// half lattice of 16^3 x 32 (random fields, the order of the sums restated in numpy) 2.5e-9,
+// 1.1e-9 with the 1216 blocks of blas_blocks, this way 0.7e-9. smem: 2 NV doubles per warp.
+template <int NV, typename C>
+__device__ __forceinline__ void block_sum_wide(const C (&v)[NV], double2 (&out)[NV], double* smem) {
+    using T = decltype(v[0].x + v[0].x);
     constexpr int NR = 2 * NV;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double r[NR];
+    T r[NR];
 #pragma unroll
     for (int i = 0; i < NV; ++i) { r[2 * i] = v[i].x; r[2 * i + 1] = v[i].y; }
-    const double t = lane_sums<NR>(r);
+    const double t = wid(lane_sums<NR, T>(r));
     __syncthreads();
     if (lane % (32 / NR) == 0) smem[w * NR + lane / (32 / NR)] = t;
     __syncthreads();
@@ -48,25 +56,24 @@ template <int NV> __device__ __forceinline__ void block_sum_fp64(double2 (&v)[NV
             if (o < nw * NR) s += __shfl_xor_sync(0xffffffffu, s, o);
 #pragma unroll
         for (int i = 0; i < NV; ++i)
-            v[i] = make_double2(__shfl_sync(0xffffffffu, s, 2 * i), __shfl_sync(0xffffffffu, s, 2 * i + 1));
+            out[i] = make_double2(__shfl_sync(0xffffffffu, s, 2 * i), __shfl_sync(0xffffffffu, s, 2 * i + 1));
     }
 }
 
 // Sum NV complex values per block into part[kind][block*NV + i]; in the last
-// block returns true with tot[] = sum over blocks (thread 0 only). The block
-// sum runs in the precision of v (FP32 for the mixed solver), the cross-block
-// sum in FP64.
+// block returns true with tot[] = sum over blocks (thread 0 only). The sum over a
+// warp runs in the precision of v (FP32 for the mixed solver), the sums across
+// warps and blocks in FP64.
 template <int NV, typename C>
 __device__ bool reduce_slot(const SlotPtrs& P, int kind, C (&v)[NV], double2 (&tot)[NV], unsigned nblocks,
                             unsigned bid) {
-    __shared__ C sm[(RED_MAX_THREADS / 32) * NV];   // blockDim.x <= RED_MAX_THREADS
-    __shared__ double2 smd[(RED_MAX_THREADS / 32) * NV];
-    if constexpr (sizeof(C) == 16) block_sum_fp64<NV>(v, reinterpret_cast<double*>(sm));
-    else block_sum<NV>(v, sm);
+    __shared__ double2 smd[(RED_MAX_THREADS / 32) * NV];   // blockDim.x <= RED_MAX_THREADS
+    double2 bs[NV];
+    block_sum_wide<NV>(v, bs, reinterpret_cast<double*>(smd));
     double2* pp = part(P, kind);
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int i = 0; i < NV; ++i) pp[(size_t)bid * NV + i] = to_d(v[i]);
+        for (int i = 0; i < NV; ++i) pp[(size_t)bid * NV + i] = bs[i];
     }
     bool last = last_block(P.counters + kind, nblocks);
     if (last) {
@@ -106,10 +113,9 @@ __device__ bool reduce_slot(const SlotPtrs& P, int kind, C (&v)[NV], double2 (&t
     return last;
 }
 
-// Per-thread and per-block partial sums accumulate in the storage precision
-// (FP32 for the mixed solver: FP64 arithmetic runs at a small fraction of the
-// FP32 rate on this GPU and would bound these bandwidth kernels); only the
-// cross-block sum is FP64.
+// Per-thread sums accumulate in the storage precision (FP32 for the mixed solver:
+// FP64 arithmetic runs at a small fraction of the FP32 rate on this GPU and would
+// bound these bandwidth kernels).
 template <typename S> struct Acc {
     cplx<S> z;      // complex sum
     S a, b;         // two real sums

@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
                 }
             }
             double2 v[2] = {comp ? cz.value() : to_d(rho), make_double2(nrm, 0.0)};
-            block_sum_fp64<2>(v, smd);
+            block_sum_wide<2>(v, v, smd);
             if (threadIdx.x == 0) {
                 double2* pp = part(P, CNT_RU) + 2 * (size_t)q;
                 pp[0] = v[0];
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
             v[0] = v[0] + __ldcg(pp + 2 * (size_t)b);
             v[1] = v[1] + __ldcg(pp + 2 * (size_t)b + 1);
         }
-        block_sum_fp64<2>(v, smd);
+        block_sum_wide<2>(v, v, smd);
         if (threadIdx.x == 0) {
             st.true_rnorm = sqrt_fp64(v[1].x);
             st.matvecs += 1;

@@ -45,8 +45,8 @@ struct CompC {
     __device__ __forceinline__ double2 value() const { return make_double2((double)sx + cx, (double)sy + cy); }
 };
 
-// Block and cross-block sum of (z, (a, b)) per slot: in the storage precision,
-// or (gamma5 variant with FP32 storage, compensated z) in FP64 throughout.
+// Block and cross-block sum of (z, (a, b)) per slot: over the warp in the storage
+// precision, or (gamma5 variant with FP32 storage, compensated z) in FP64 throughout.
 template <typename S>
 __device__ __forceinline__ bool reduce2(const SlotPtrs& P, int kind, bool comp, const CompC& cz, const Acc<S>& acc,
                                         double2 (&tot)[2], unsigned nblocks, unsigned bid) {
