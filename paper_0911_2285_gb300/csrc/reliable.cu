@@ -44,6 +44,7 @@ constexpr int RU_THREADS = 128;
 constexpr int RU_COOP = 2 * 152;   // 128-site units (slots x units) of a cooperative launch: two blocks per SM
 constexpr int RU_RUNS = 4096;   // partial sums per slot at most (24^3 x 64: 3456 of two units)
 static_assert(2 * RU_RUNS <= PARTIAL_STRIDE, "partials of a slot");
+static_assert(MAX_SLOTS <= 32, "a slot per lane");
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     unsigned v;
@@ -186,14 +187,16 @@ __global__ void __launch_bounds__(RU_THREADS, MODE == RU_DF ? 3 : 2)
               const SlotPtrs* ptrs, int nslots, size_t N, int phase, int* err) {
     __shared__ int list[MAX_SLOTS];
     __shared__ int s_n;
-    if (threadIdx.x == 0) {
-        int n = 0;
-        for (int j = 0; j < nslots; ++j)
-            if (states[j].status == ST_RUNNING && states[j].live && states[j].need_ru) list[n++] = j;
+    if (threadIdx.x < 32) {   // a slot per lane, its words read at once: most launches end here
+        const int j = threadIdx.x;
+        const SlotState& st = states[j < nslots ? j : 0];
         // After a wait that gave up, the counters may be stale until the host has seen err:
         // no further update. (Set by a block of this launch while others start, it only
         // makes them give up too.)
-        s_n = *(volatile int*)err ? 0 : n;
+        const bool on = (j < nslots) & (st.status == ST_RUNNING) & (st.live != 0) & (st.need_ru != 0) & (*(volatile int*)err == 0);
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        if (on) list[__popc(m & ((1u << j) - 1u))] = j;
+        if (j == 0) s_n = __popc(m);
     }
     __syncthreads();
     const int nact = s_n;
