@@ -400,4 +400,6 @@ cudaError_t launch_matvec_staged(const Geom& g, const void* maps, double kappa, 
     return cudaGetLastError();
 }
 
+cudaError_t set_wait_cycles_staged(long long cycles) { return set_wait_cycles_here(cycles); }
+
 }  // namespace lqcd

@@ -232,10 +232,12 @@ cudaError_t launch_eo_pair(const Geom& g, const void* links, double kappa, int p
 cudaError_t launch_eo_true_resid(const Geom& g, const void* links64, double kappa, SlotState* states,
                                  const SlotPtrs* ptrs, int nslots, cudaStream_t st);
 
-// Bound of the device-side waits (SM clock cycles) of the kernels of gemm_tc.cu
-// and dslash_tiled.cu on the current device; cycles <= 0 restores the default.
+// Bound of the device-side waits (SM clock cycles) of the kernels of gemm_tc.cu,
+// dslash_tiled.cu and dslash_staged.cu on the current device (those of dots.cu and
+// reliable.cu above); cycles <= 0 restores the default.
 cudaError_t set_wait_cycles_tc(long long cycles);
 cudaError_t set_wait_cycles_tiled(long long cycles);
+cudaError_t set_wait_cycles_staged(long long cycles);
 // One-thread kernel: bounded wait for *flag != 0; *status = 1 if it gave up.
 cudaError_t launch_flag_wait(const int* flag, int* status, cudaStream_t st);
 

@@ -2175,6 +2175,7 @@ __device__ int g_flag_status;   // status word of lqcd_wait_flag
 extern "C" lqcd_status lqcd_set_wait_limit(long long cycles) {
     CK(set_wait_cycles_tc(cycles));
     CK(set_wait_cycles_tiled(cycles));
+    CK(set_wait_cycles_staged(cycles));
     CK(set_wait_cycles_ru(cycles));
     CK(set_wait_cycles_dots(cycles));
     return LQCD_OK;
