@@ -363,7 +363,8 @@ lqcd_status lqcd_small_eig_noalloc(int n, const double *C, double *evals, double
 /* Failure-detection hook (no counterpart in the paper): bound of every
  * device-side wait in this library's kernels (TMA/mbarrier pipelines, the flag
  * wait below), in SM clock cycles, on the current device.  A kernel whose wait
- * runs out records an error word and returns; the call that launched it then
+ * runs out records an error word and returns (its copies in flight it waits
+ * for with the default limit all the same); the call that launched it then
  * returns LQCD_ERR_TIMEOUT.  cycles <= 0 restores the default (4e9 cycles,
  * about 2 s at 2 GHz).  Affects kernels launched after the call. */
 lqcd_status lqcd_set_wait_limit(long long cycles);

@@ -1,8 +1,8 @@
 // Tall-skinny complex inner-product matrices on the tensor cores (tcgen05):
 //   C[i][j] = sum_e conj(X_i(e)) Y_j(e),   i < a, j < b,
-// over FP32 fields of N complex numbers. These are the Galerkin projections
-// of the deflation and of the eigenspace growth (Alg. Incremental eigBiCG:
-// U_l^H r, U_l^H A U_r and the oblique orthogonalisation of new Ritz vectors).
+// over FP32 fields of N complex numbers, for blocks that fill its tiles (see
+// launch_multidot). The Galerkin projections of the solver are smaller (a <= 80)
+// and run on dots.cu; lqcd_field_dots comes here for a >= 85.
 //
 // Real form: with x' = (re x, im x) interleaved along K (K = 2N reals),
 //   Re C_ij = x'_i . y'_j,   Im C_ij = x'_i . z_j,  z = (im y, -re y),
@@ -10,8 +10,7 @@
 // gives both parts (M = 128 rows of X per CTA tile, N = 48 = 24 Y columns and
 // their Z twins, FP32 accumulators in tensor memory). Its time is that of a full
 // tile, 4.3 ms at N = 10.6 M for any a <= 128 and b <= 24 (moving the split tiles
-// through shared memory), so it serves the large blocks; the others go to the FP32
-// form of launch_dots.
+// through shared memory).
 //
 // Precision: 3xTF32. Each operand v is split into big = tf32(v) and
 // small = v - big, and the tile product is big.big + big.small + small.big,
@@ -21,13 +20,13 @@
 // runs and the CTAs (split-K) are summed in FP64.
 //
 // Data movement: TMA tensor copies with 128-byte swizzle bring 32-real K-tiles
-// of X (128 rows) and Y (8 rows) into a 4-stage shared-memory ring; the split
+// of X (128 rows) and Y (24 rows) into a 5-stage shared-memory ring; the split
 // is elementwise in place (the swizzle moves 16-byte granules only, so every
-// complex pair keeps its position), the Z twins go to the second 8-row atom.
+// complex pair keeps its position), the Z twins go behind the Y rows.
 // Warp-specialised: one thread issues the TMA copies, one the MMAs (committed
 // to the stage's mbarrier, which frees the stage for the next copy), eight
-// warps split the tiles; two tensor-memory accumulators alternate between
-// runs so that reading one run overlaps the MMAs of the next.
+// warps split the tiles; four tensor-memory accumulators take turns, so that
+// reading one run overlaps the MMAs of the next.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
@@ -90,7 +89,7 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, unsigned parity, vo
 // copies; warp 1 (lane 0) issues the MMAs; warps 2.. split the tiles into
 // TF32 big/small parts, and warps 2-5 (one per tensor-memory lane quarter)
 // also move each finished accumulation run into their FP64 sums.
-// Grid (split-K CTAs, row tiles of 128). part: [gridDim.y][gridDim.x][128][16] FP64.
+// Grid (split-K CTAs, row tiles of 128). part: [gridDim.y][gridDim.x][128][48] FP64.
 __global__ void __launch_bounds__(TC_THREADS, 1)
     dots_tc_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap my, int box_rows,
                    long long tiles, double* part, int* err) {

@@ -1170,7 +1170,8 @@ cudaError_t launch_multidot(int a, const void* X, int xp, int b, const void* Y, 
     if (a <= 0 || b <= 0) return cudaSuccess;
     // The tensor-core form takes a tile of 128 X against 24 Y fields whatever part of it is
     // filled (4.3 ms at N = 10.6 M), the FP32 form 1.35 ms per 80 X and 8 Y fields: 128 x 24
-    // cost as much as 252 x 8.
+    // cost as much as 252 x 8. With a <= MAX_SMALL = 80 fields the line is never crossed; the
+    // blocks beyond it come from lqcd_field_dots.
     if (staged && xp == 1 && yp == 1 && div_up(b, 8) * a > 252 * div_up(a, 128) * div_up(b, 24) &&
         dots_tc_supported(a, X, Y, N) && dots_tc_scratch_doubles(a) <= 2 * scratch_elems)
         return launch_dots_tc(a, X, N * 8, b, Y, N * 8, N, Cm, ldc, conj_store, reinterpret_cast<double*>(scratch),

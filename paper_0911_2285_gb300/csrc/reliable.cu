@@ -12,13 +12,13 @@
 // small lattices). It has two (even-odd: three) phases, each reading neighbours that the
 // one before wrote:
 //  * up to RU_COOP units of work: one cooperative launch with a grid barrier between the
-//    phases, 1.5 us per iteration less than a launch per phase (FP64 solve on 4^4 2.44 ms,
-//    2.57 the other way; 10x6x14x9 mixed 5.53 and 5.72);
+//    phases, about 1.5 us per iteration less than a launch per phase (FP64 solve on 4^4
+//    2.33 ms, 2.42 the other way; 10x6x14x9 mixed 5.25 and 5.31);
 //  * above: a launch per phase. A cooperative launch starts only when all its blocks fit on
 //    the GPU at once, so that a large one waited in every iteration for room beside the
-//    kernels of another context: 16^3 x 32 solves beside 24^3 x 64 ones 346 ms, now 253
-//    (four kernels: 284), alone 15.7 and 15.8. With 128 blocks (8^4, 4 slots) both ways
-//    take 104 and 101 ms beside, with 256 blocks 137 and 129 (four kernels: 143).
+//    kernels of another context: 16^3 x 32 solves beside 24^3 x 64 ones 343 ms, now 264
+//    (four kernels: 284); alone 15.7 and 15.9, even-odd batches 51.3 and 51.8. At the line
+//    (8^4, 8 slots, 256 units) 125 ms beside, 143 with four kernels.
 //
 // Double-float residual: about 10^4 FP32 instructions per site. Written out for
 // eight hops that is 175 KB of code, more than the instruction caches hold: ncu

@@ -519,7 +519,7 @@ def kernel_launches():
 def field_dots(X, Y, path=1, reps=0):
     """``C = X^H Y`` (a x b, complex128) of FP32 fields: ``X`` (a, n) and ``Y`` (b, n)
     contiguous complex64 CUDA tensors. ``path`` 0 = plain kernel, 1 = TMA-staged
-    (3xTF32). Returns ``(C, avg_ms)``; ``avg_ms`` is the mean time of ``reps`` more
+    (FP32 products; 3xTF32 tensor-core MMAs for large ``a`` and ``b``). Returns ``(C, avg_ms)``; ``avg_ms`` is the mean time of ``reps`` more
     calls (None when ``reps == 0``)."""
     import torch
     for t in (X, Y):
