@@ -27,7 +27,7 @@
 // sources and swaps as selects and its signs as FMA factors; and the FP64 pipe,
 // which fold, residual and rounding to FP32 filled with conversions (44 % busy),
 // keeps only the additions (fp64.cuh). Fold, residual and replacement of one
-// field at 24^3 x 64: 1.7 -> 0.71 ms; what bounds it now is issue (a third of
+// field at 24^3 x 64: 1.7 -> 0.75 ms; what bounds it now is issue (a third of
 // the time) and the latency of the neighbour loads at 12 warps per SM.
 #include "async.cuh"
 #include "dfloat.cuh"
