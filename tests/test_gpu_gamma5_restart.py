@@ -17,7 +17,8 @@ def _solve(dims, eps, seed, kappa, n, mode="plain", **kw):
     links = gauge_links(dims, eps, seed)
     op = WilsonOperator(links, kappa, dims)
     b = np.stack([gaussian_source(dims, 100 + i) for i in range(n)])
-    args = dict(nev=4, m=12, n1=1, tol=1e-10, maxiter=4000, precision="mixed", k_max=4, gamma5=True)
+    # one operator shape: which sources are lost depends on the order of the sums
+    args = dict(nev=4, m=12, n1=1, tol=1e-10, maxiter=4000, precision="mixed", k_max=4, gamma5=True, autotune=False)
     with Solver(links, dims, kappa, **{**args, **kw}) as s:
         x, info, _ = s.solve(b, mode=mode, raise_on_fail=False)
     return [(info[j], true_resid(op, b[j], x[j])) for j in range(n)]
